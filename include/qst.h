@@ -75,7 +75,9 @@ typedef enum {
  * rho = T^dag T / Tr(T^dag T).  The mixed modes support QST_MAP_CHOL_H only
  * (QST_E_UNSUPPORTED otherwise). */
 enum { QST_MAP_CHOL_H = 0, QST_MAP_ABS_P = 1, QST_MAP_CHOL_DELTA = 2 };
-/* Precisions.  QST_MIXED runs the two complex d x d products on tensor cores
+/* Precisions.  QST_FP32 runs the complex d x d products of QST_MAP_CHOL_H and QST_MAP_CHOL_DELTA with N >= 7
+ * on tensor cores too, each operand as the exact sum of three BF16 terms (all 24 bits), summed in FP32;
+ * where the device or device_memory_limit has no room for those operands, on the CUDA cores.  QST_MIXED runs the two complex d x d products on tensor cores
  * (tcgen05) with each FP32 operand split into FP16 hi + lo after a power-of-two
  * scaling (about 2^-21 relative error); QST_MIXED_BF16 uses a BF16 hi + lo split
  * without scaling (about 2^-16).  Everything else stays FP32 in both.  Mixed
@@ -343,7 +345,8 @@ qst_status qst_graph_enable(qst_ctx* ctx, int enable);
  * earlier keeps the values it was captured with until its inputs change.  QST_E_INVAL for values out of
  * range (nothing changed). */
 /* Testing hook for the device-side wait limits; it involves no GPU fault.  With what =
- * QST_INJECT_TC_LOADS the next `count` launches of the tensor-core products (QST_MIXED, QST_MIXED_BF16),
+ * QST_INJECT_TC_LOADS the next `count` launches of the tensor-core products (QST_MIXED, QST_MIXED_BF16, and
+ * QST_FP32 with N >= 7),
  * with QST_INJECT_WPASS_LOADS the next `count` launches of the FP32 bulk weight passes, issue none of
  * their operand copies: the waits for those copies run out after their limit (about 2 s), the kernels
  * leave their results unwritten and return, and the call that reads the loss (qst_step, qst_loss_grad,

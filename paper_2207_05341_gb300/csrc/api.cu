@@ -237,6 +237,17 @@ template <class T> cudaError_t dalloc(qst_ctx* c, T** p, size_t count) {
   return cudaSuccess;
 }
 
+// An allocation the context can do without: skipped where it fails, or where it would leave less of the
+// budget than `later` bytes (the scratch that calls may still allocate on first use).
+template <class T> void dalloc_optional(qst_ctx* c, T** p, size_t count, size_t later) {
+  const size_t lim = c->opt.device_memory_limit;
+  if (lim && c->dev_bytes + count * sizeof(T) + later > lim) return;
+  if (dalloc(c, p, count) != cudaSuccess) {
+    cudaGetLastError();
+    *p = nullptr;
+  }
+}
+
 template <class R> Work<R>* W(qst_ctx* c) { return reinterpret_cast<Work<R>*>(c->work); }
 template <class R> const PovmB<R>& povmB(qst_ctx* c);
 template <> const PovmB<float>& povmB<float>(qst_ctx* c) { return c->Bf; }
@@ -249,6 +260,8 @@ size_t theta_size(int N) {
 
 size_t rsize(const qst_ctx* c) { return c->prec == QST_FP64 ? sizeof(double) : sizeof(float); }
 bool is_mixed(const qst_ctx* c) { return c->prec == QST_MIXED || c->prec == QST_MIXED_BF16; }
+// FP32 products on tensor cores (gemm_tc_fp32.cu): decided once, by whether the operand planes were allocated
+bool is_tc32(const qst_ctx* c) { return c->prec == QST_FP32 && reinterpret_cast<const Work<float>*>(c->work)->P6; }
 int tc_fmt(const qst_ctx* c) { return c->prec == QST_MIXED_BF16 ? TC_BF16 : TC_FP16_SCALED; }
 
 template <class R> qst_status alloc_work(qst_ctx* c) {
@@ -340,6 +353,17 @@ template <class R> qst_status alloc_work(qst_ctx* c) {
     QST_CU(dalloc(c, &gb, 4 * nn));
     w->Gb = gb;
   }
+  // FP32 products on tensor cores where their operand planes fit (else on the CUDA cores)
+  if (c->prec == QST_FP32 && c->opt.mapping != QST_MAP_ABS_P && tc32_ok(D.d)) {
+    const size_t later = 8 * (2 * (size_t)D.n + (size_t)D.n / 512) + 24 * nn + 512 * (size_t)D.d + 65536;
+    unsigned short *p9 = nullptr, *p6 = nullptr;
+    dalloc_optional(c, &p9, 9 * nn, 12 * nn + later);
+    if (p9) dalloc_optional(c, &p6, 6 * nn, later);
+    if (p6) {
+      w->P9 = p9;
+      w->P6 = p6;
+    }
+  }
   return QST_OK;
 }
 
@@ -373,9 +397,9 @@ template <class R> qst_status validate_f(qst_ctx* c, const void* fdev) {
   return QST_OK;
 }
 
-// The producer-side max slot of the scaled FP16 split (NULL on the other paths).
+// The producer-side max slot of the scaled splits (NULL on the other paths).
 unsigned int* amax_slot(qst_ctx* c, int slot) {
-  if (!is_mixed(c) || tc_fmt(c) != TC_FP16_SCALED) return nullptr;
+  if (!is_tc32(c) && (!is_mixed(c) || tc_fmt(c) != TC_FP16_SCALED)) return nullptr;
   return (c->prec == QST_FP64 ? W<double>(c)->counters : W<float>(c)->counters) + slot;
 }
 
@@ -391,17 +415,27 @@ template <class R> struct Engine {
     // t = W2 h + b2 in the dt buffer (free until the backward writes dL/dt), then T (or its 16-bit planes)
     // Chol_Delta: T lower triangular and T^dag (in Y, free until the backward) for X = T^dag T
     const bool delta = c->opt.mapping == QST_MAP_CHOL_DELTA;
+    const bool tc32 = is_tc32(c), planes = mixed || (tc32 && !delta);  // T only as its planes, made from t
     if (c->cnn) {
       QST_CU(cnn_output<R>(D, theta, w->hid, w->dt, amax_slot(c, CNT_AMAXT), c->stream));
-      if (!mixed) QST_CU(net_hermitian_T<R>(D, w->dt, w->T, delta ? w->Y : nullptr, c->stream));
+      if (!planes) QST_CU(net_hermitian_T<R>(D, w->dt, w->T, delta ? w->Y : nullptr, c->stream));
     } else {
       const bool absp = c->opt.mapping == QST_MAP_ABS_P;  // the cold start's Jacobi sweeps read T itself
-      QST_CU(net_build_T<R>(D, theta, w->hid, w->dt, mixed && !absp ? nullptr : w->T, amax_slot(c, CNT_AMAXT),
+      QST_CU(net_build_T<R>(D, theta, w->hid, w->dt, planes && !absp ? nullptr : w->T, amax_slot(c, CNT_AMAXT),
                             c->stream, delta ? w->Y : nullptr));
     }
     if (mixed) {
       QST_CU(tc_planes_T(D.d, reinterpret_cast<const float*>(w->dt), w->Tb, tc_fmt(c), w->scal,
                          amax_slot(c, CNT_AMAXT), c->stream));
+    } else if (tc32) {
+      unsigned int* am = amax_slot(c, CNT_AMAXT);
+      if (delta) {
+        QST_CU(tc32_split(D.d, reinterpret_cast<const float2*>(w->Y), w->P9, 9, false, am, w->scal + kScaleT,
+                          c->stream));
+        c->launches += 1;
+      } else {
+        QST_CU(tc32_planes_T(D.d, reinterpret_cast<const float*>(w->dt), w->P9, am, w->scal + kScaleT, c->stream));
+      }
     }
     c->launches += 2;
     tmark(c, QST_PH_BUILD_T);
@@ -488,6 +522,9 @@ template <class R> struct Engine {
     } else if (mixed) {
       QST_CU(tc_herm_square(D.d, w->Tb, tc_fmt(c), w->scal, reinterpret_cast<float2*>(w->X), w->flags + 1,
                             amax_slot(c, CNT_AMAXT), c->stream));
+    } else if (tc32) {  // A and B^dag: T itself (Hermitian), or T^dag (upper triangular) for X = T^dag T
+      QST_CU(tc32_product(D.d, w->P9, w->P9, w->scal + kScaleT, w->scal + kScaleT, reinterpret_cast<float2*>(w->X),
+                          true, delta ? 1 : 0, w->flags + 1, amax_slot(c, CNT_AMAXT), c->stream));
     } else {
       QST_CU(cgemm_simt<R>(D.d, delta ? w->Y : w->T, w->T, w->X, true, c->stream));
     }
@@ -579,15 +616,36 @@ template <class R> struct Engine {
       c->launches += 2;
     } else if (c->opt.mapping == QST_MAP_CHOL_DELTA) {
       // dL = 2 Re Tr[G T^dag dT] for lower-triangular dT: only the lower tiles of Z = T G are needed
-      QST_CU(cgemm_simt<R>(D.d, w->T, w->G, w->Y, true, c->stream));
+      if (is_tc32(c)) {
+        QST_CU(tc32_split(D.d, reinterpret_cast<const float2*>(w->T), w->P6, 6, true, nullptr, w->scal + kScaleT,
+                          c->stream));
+        QST_CU(tc32_split(D.d, reinterpret_cast<const float2*>(w->G), w->P9, 9, false, amax_slot(c, CNT_AMAXG),
+                          w->scal + kScaleG, c->stream));
+        QST_CU(tc32_product(D.d, w->P6, w->P9, w->scal + kScaleT, w->scal + kScaleG,
+                            reinterpret_cast<float2*>(w->Y), true, 2, w->flags + 1, amax_slot(c, CNT_AMAXG),
+                            c->stream));
+        c->launches += 2;
+      } else {
+        QST_CU(cgemm_simt<R>(D.d, w->T, w->G, w->Y, true, c->stream));
+      }
       tmark(c, QST_PH_GT);
       QST_CU(net_tri_grad<R>(D, w->Y, w->dt, c->stream));
       tmark(c, QST_PH_SYM);
       c->launches += 2;
     } else {
-      QST_CU(cgemm_simt<R>(D.d, w->G, w->T, w->Y, false, c->stream));
+      if (is_tc32(c)) {
+        QST_CU(tc32_split(D.d, reinterpret_cast<const float2*>(w->G), w->P6, 6, false, amax_slot(c, CNT_AMAXG),
+                          w->scal + kScaleG, c->stream, reinterpret_cast<const float2*>(w->X), w->scal, w->partials,
+                          w->counters + CNT_GX, w->flags));
+        QST_CU(tc32_product(D.d, w->P6, w->P9, w->scal + kScaleG, w->scal + kScaleT,
+                            reinterpret_cast<float2*>(w->Y), false, 0, w->flags + 1, amax_slot(c, CNT_AMAXG),
+                            c->stream));
+        c->launches += 1;
+      } else {
+        QST_CU(cgemm_simt<R>(D.d, w->G, w->T, w->Y, false, c->stream));
+      }
       tmark(c, QST_PH_GT);
-      QST_CU(net_symmetrize<R>(D, w->Y, w->dt, c->stream));
+      QST_CU(net_symmetrize<R>(D, w->Y, w->dt, c->stream, is_tc32(c) ? w->scal + kGauge : nullptr));
       tmark(c, QST_PH_SYM);
       c->launches += 2;
     }
@@ -635,12 +693,14 @@ template <class R> struct Engine {
     if (c->h_flags[1] != 0u) {
       // a kernel that gave up returned before its last-block reduction: restart every counter
       QST_CU(cudaMemsetAsync(w->flags, 0, 2 * sizeof(unsigned int), c->stream));
+      QST_CU(cudaMemsetAsync(w->flags + 4, 0, sizeof(unsigned int), c->stream));
       QST_CU(cudaMemsetAsync(w->counters, 0, CNT_COUNT * sizeof(unsigned int), c->stream));
       QST_CU(cudaStreamSynchronize(c->stream));
       return QST_E_TIMEOUT;
     }
     if (c->h_flags[0] != 0u) {
       QST_CU(cudaMemsetAsync(w->flags, 0, sizeof(unsigned int), c->stream));
+      QST_CU(cudaMemsetAsync(w->flags + 4, 0, sizeof(unsigned int), c->stream));
       return QST_W_CLAMP;
     }
     return QST_OK;

@@ -371,11 +371,11 @@ __global__ void __launch_bounds__(256, 2) k_w1_pass(R* __restrict__ theta, R* __
 // Gamma = Y + Y^dag;  dR_ij = 2 Re Gamma_ij, dR_ji = 2 Im Gamma_ij (i > j), dR_ii = Re Gamma_ii.
 template <class R>
 __global__ void __launch_bounds__(256) k_symmetrize(const cx_t<R>* __restrict__ Y, R* __restrict__ dt, int d,
-                                                     const void* const* tab) {
+                                                     const double* gauge, const void* const* tab) {
   __shared__ R Ar[32][33], Ai[32][33], Br[32][33], Bi[32][33];
-  rebind(tab, Y, dt);
+  rebind(tab, Y, dt, gauge);
   grid_dep_wait();
-  after_wait(Y, dt);
+  after_wait(Y, dt, gauge);
   const int TS = d < 32 ? d : 32;
   int I, J;
   tri_decode(blockIdx.x, I, J);
@@ -401,13 +401,21 @@ __global__ void __launch_bounds__(256) k_symmetrize(const cx_t<R>* __restrict__ 
       __syncthreads();
       const int r = t >> 3, c = (t & 7) * 4;
       float v[4];
+      // Y + g T: 4 g R_ij off the diagonal, 2 g R_ii on it (each thread replaces the entries of t it reads)
+      const float g4 = gauge ? 4.f * (float)*gauge : 0.f;
+      float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), tb = ta;
+      if (gauge) {
+        ta = *reinterpret_cast<const float4*>(dt + (long long)(I * 32 + r) * d + J * 32 + c);
+        if (I != J) tb = *reinterpret_cast<const float4*>(dt + (long long)(J * 32 + r) * d + I * 32 + c);
+      }
+      const float tav[4] = {ta.x, ta.y, ta.z, ta.w}, tbv[4] = {tb.x, tb.y, tb.z, tb.w};
       if (I != J) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = R(2) * (Ar[r][c + u] + Br[c + u][r]);
+        for (int u = 0; u < 4; ++u) v[u] = fmaf(g4, tav[u], R(2) * (Ar[r][c + u] + Br[c + u][r]));
         *reinterpret_cast<float4*>(dt + (long long)(I * 32 + r) * d + J * 32 + c) = make_float4(v[0], v[1], v[2], v[3]);
         // upper tile (J, I): element (J 32 + r, I 32 + c + u) = 2 Im Gamma_{(I 32 + c + u), (J 32 + r)}
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = R(2) * (Ai[c + u][r] - Bi[r][c + u]);
+        for (int u = 0; u < 4; ++u) v[u] = fmaf(g4, tbv[u], R(2) * (Ai[c + u][r] - Bi[r][c + u]));
         *reinterpret_cast<float4*>(dt + (long long)(J * 32 + r) * d + I * 32 + c) = make_float4(v[0], v[1], v[2], v[3]);
       } else {
 #pragma unroll
@@ -416,6 +424,7 @@ __global__ void __launch_bounds__(256) k_symmetrize(const cx_t<R>* __restrict__ 
           if (r > cc) v[u] = R(2) * (Ar[r][cc] + Ar[cc][r]);
           else if (r < cc) v[u] = R(2) * (Ai[cc][r] - Ai[r][cc]);
           else v[u] = R(2) * Ar[r][r];
+          v[u] = fmaf(r == cc ? 0.5f * g4 : g4, tav[u], v[u]);
         }
         *reinterpret_cast<float4*>(dt + (long long)(I * 32 + r) * d + J * 32 + c) = make_float4(v[0], v[1], v[2], v[3]);
       }
@@ -595,13 +604,15 @@ cudaError_t net_w1_pass(const Dims& D, R* theta, R* step, const R* f, const R* d
   return cudaGetLastError();
 }
 
-template <class R> cudaError_t net_symmetrize(const Dims& D, const cx_t<R>* Y, R* dt, cudaStream_t s) {
+template <class R>
+cudaError_t net_symmetrize(const Dims& D, const cx_t<R>* Y, R* dt, cudaStream_t s, const double* gauge) {
   const int TS = D.d < 32 ? D.d : 32;
   const int nt = D.d / TS;
+  if (gauge && (TS != 32 || sizeof(R) != 4)) return cudaErrorInvalidValue;
   BatchArgs ba;
-  if (batch_take(ba, {Y, dt})) return cudaSuccess;
+  if (batch_take(ba, {Y, dt, gauge})) return cudaSuccess;
   return launch_dep(k_symmetrize<R>, dim3((unsigned)(nt * (nt + 1) / 2), 1, ba.nz), dim3(256), 0, s, Y, dt, D.d,
-                    ba.tab);
+                    gauge, ba.tab);
 }
 
 template <class R> cudaError_t net_tri_grad(const Dims& D, const cx_t<R>* Z, R* dt, cudaStream_t s) {
@@ -622,7 +633,7 @@ template <class R> cudaError_t net_tri_grad(const Dims& D, const cx_t<R>* Z, R* 
                                       unsigned int*, const NetCfg&, bool, cudaStream_t);                         \
   template cudaError_t net_w1_pass<R>(const Dims&, R*, R*, const R*, const R*, R*, R*, R*, double*,     \
                                       double*, unsigned int*, const NetCfg&, bool, cudaStream_t);                \
-  template cudaError_t net_symmetrize<R>(const Dims&, const cx_t<R>*, R*, cudaStream_t);
+  template cudaError_t net_symmetrize<R>(const Dims&, const cx_t<R>*, R*, cudaStream_t, const double*);
 QST_INST(float)
 QST_INST(double)
 #undef QST_INST

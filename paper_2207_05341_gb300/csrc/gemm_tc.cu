@@ -37,6 +37,7 @@
 #include <stdint.h>
 
 #include "impl.h"
+#include "tc.cuh"
 
 namespace qst {
 
@@ -52,53 +53,11 @@ constexpr int kTileBytes = 128 * kBK * 2;        // one 128-row x 32-col 16-bit 
 constexpr int kStageBytes = 6 * kTileBytes;      // 96 KB
 constexpr int kTmemCols = 512;   // two 128 x 256 FP32 accumulators: hi*hi, and hi*lo + lo*hi
 constexpr int kSmemBytes = kStages * kStageBytes + 1024 + 256;
-constexpr unsigned long long kWaitCycles = 4000000000ULL;  // ~2 s at 2 GHz
 
 struct TcMaps {
   CUtensorMap a[4];  // A planes: re_hi, im_hi, re_lo, im_lo
   CUtensorMap b[6];  // T planes: re_hi, im_hi, nim_hi, re_lo, im_lo, nim_lo
 };
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-      "selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(bar), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait on an mbarrier phase; false after ~kWaitCycles.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  if (mbar_try(bar, parity)) return true;
-  const unsigned long long t0 = clock64();
-  while (!mbar_try(bar, parity)) {
-    if (clock64() - t0 > kWaitCycles) return false;
-  }
-  return true;
-}
-
-__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(bar)
-      : "memory");
-}
 
 // Shared-memory matrix descriptor: K-major, swizzled rows of kRowBytes, 8-row atoms of 8 kRowBytes bytes.
 __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
@@ -115,28 +74,6 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t addr) {
 // K-major, M = 128, N = 256.
 __host__ __device__ constexpr uint32_t make_idesc(uint32_t fmt) {
   return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(2 * kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accum) {
-  asm volatile(
-      "{\n.reg .pred p;\n"
-      "setp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accum)
-      : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint32_t bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
 }
 
 // tab: a batched launch (grid z = tomography); row z holds the tensor maps' device copy, C, sA, sB, err, clear
@@ -303,14 +240,6 @@ template <> __device__ __forceinline__ __half to16<__half>(float v) { return __f
 template <> __device__ __forceinline__ __nv_bfloat16 to16<__nv_bfloat16>(float v) { return __float2bfloat16_rn(v); }
 __device__ __forceinline__ float from16(__half v) { return __half2float(v); }
 __device__ __forceinline__ float from16(__nv_bfloat16 v) { return __bfloat162float(v); }
-
-// Scale of the FP16 split: 2^-e for the largest |re|, |im| in [2^e, 2^(e+1)) (*amax, float bits, folded
-// in by the kernel that wrote the matrix), i.e. the power of two that brings it into [1, 2); 1 without amax.
-__device__ __forceinline__ double split_scale(const unsigned int* amax) {
-  if (!amax) return 1.0;
-  const double m = (double)__uint_as_float(*reinterpret_cast<const volatile unsigned int*>(amax));
-  return (m > 0.0 && isfinite(m)) ? ldexp(1.0, -ilogb(m)) : 1.0;
-}
 
 // hi = 16-bit rounding of v, lo = 16-bit rounding of the remainder
 template <class H> __device__ __forceinline__ void hi_lo(float v, H& hi, H& lo) {

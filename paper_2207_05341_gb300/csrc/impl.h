@@ -111,13 +111,18 @@ template <class R> struct Work {
   R* fstage;           // staging copy of a host f, n reals
   R* fperm;            // f in the order of the structured likelihood pass (FP32 fast path), n reals
   double* scal;        // [0] Tr X, [1] sum f, [2] loss, [3] scale of T, [4] scale of G, [5] F_c,
-                       // [8..10] state fidelity (sum g, bracket bound, F_q)
+                       // [8..10] state fidelity (sum g, bracket bound, F_q), [12] kGauge
   double* partials;    // per-block partial sums
   unsigned int* counters;  // last-block counters, one per reduction site
-  unsigned int* flags;     // [0] clamp count, [1] device-side wait timeouts
+  unsigned int* flags;     // [0] clamp count, [1] device-side wait timeouts, [2] sampler's bad input, [4] the
+                           // clamp count when kGauge was last made
   // mixed precision operands (BF16 hi / lo planes), NULL when unused
   void* Tb;            // 6 planes of d x d bf16: re_hi, im_hi, nim_hi, re_lo, im_lo, nim_lo
   void* Gb;            // 4 planes of d x d bf16: re_hi, im_hi, re_lo, im_lo
+  // FP32 products on tensor cores (gemm_tc_fp32.cu): three-term BF16 planes, NULL when those products run on
+  // the CUDA cores.  Chol_H: T (9 planes) and G (6); Chol_Delta: T^dag, then G (9) and T (6).
+  void* P9;
+  void* P6;
 };
 
 // Host helpers of the C ABI entry points (api.cu).
@@ -135,10 +140,12 @@ enum Counter {
                   // writer, cleared by the product that reads the planes
   CNT_AMAXG = 9,  // the same for G
   CNT_FID = 10,   // classical fidelity reductions
+  CNT_GX = 11,    // Tr(G X)
   CNT_COUNT = 16
 };
 constexpr int kScaleT = 3;  // scal slot of the power-of-two scale of T (mixed path)
 constexpr int kScaleG = 4;  // scal slot of the scale of G
+constexpr int kGauge = 12;  // scal slot of the multiple of T that makes Tr(G X) = 0 (FP32 tensor-core products)
 constexpr int kPartialBlocks = 1024;   // max blocks of a reducing kernel
 constexpr int kPartialStride = 32;     // doubles per block in `partials` (>= H + 1)
 
@@ -291,7 +298,9 @@ cudaError_t w1_pass_bulk(const Dims& D, float* theta, float* step, const float* 
                          float* pre, float* hid, double* scal, double* partials, unsigned int* counter,
                          unsigned int* flags, const NetCfg& c, cudaStream_t s);
 // dL/dt from Y = G T:  dR_ij = 2(Re Y_ij + Re Y_ji), dR_ji = 2(Im Y_ij - Im Y_ji) (i > j), dR_ii = 2 Re Y_ii
-template <class R> cudaError_t net_symmetrize(const Dims& D, const cx_t<R>* Y, R* dt, cudaStream_t s);
+// gauge (FP32, may be NULL): Y + *gauge T in the place of Y, T's entries read from dt, which then still holds t
+template <class R> cudaError_t net_symmetrize(const Dims& D, const cx_t<R>* Y, R* dt, cudaStream_t s,
+                                              const double* gauge = nullptr);
 
 // ---- P-order absolute projection (eigh.cu) ----
 template <class R> struct AbsPWork {
@@ -406,6 +415,22 @@ cudaError_t tc_planes_op(int d, const float2* M, int op, int nplanes, void* P, i
                          double* s_slot, cudaStream_t s);
 // *amax = the largest |re|, |im| of n complex entries (float bits; the slot is cleared first)
 cudaError_t absmax_to(long long n, const float2* M, unsigned int* amax, cudaStream_t s);
+
+// ---- FP32 products on tensor cores, operands as exact three-term BF16 sums (gemm_tc_fp32.cu) ----
+bool tc32_ok(int d);  // d a multiple of 128, on a device that has tcgen05
+// The 9 planes (re, im, -im; each h, m, l) of the Hermitian T of t, scaled by the power of two that brings
+// *amax into [1, 2) (written to *s_slot).
+cudaError_t tc32_planes_T(int d, const float* t, void* P, const unsigned int* amax, double* s_slot, cudaStream_t s);
+// The planes of a complex matrix: 6 (re, im: a left operand) or 9 (a right operand, given as its B^dag).
+// keep_scale: the scale already in *s_slot instead of *amax's.
+// X (Chol_H's G only; lower 128 x 128 tiles): also scal[kGauge] = -Tr(G X) / Tr X, for net_symmetrize.
+cudaError_t tc32_split(int d, const float2* A, void* P, int planes, bool keep_scale, const unsigned int* amax,
+                       double* s_slot, cudaStream_t s, const float2* X = nullptr, double* scal = nullptr,
+                       double* partials = nullptr, unsigned int* counter = nullptr, unsigned int* flags = nullptr);
+// C = A B from the (first) 6 planes of A and the 9 planes of B^dag; lower: 128 x 128 tiles I >= J only.
+// krange: 0 all of k; 1 A and B^dag upper triangular (with lower); 2 A lower triangular.  err, clear as above.
+cudaError_t tc32_product(int d, const void* Ap, const void* Bp, const double* sA, const double* sB, float2* C,
+                         bool lower, int krange, unsigned int* err, unsigned int* clear, cudaStream_t s);
 
 // ---- synthetic data on the GPU (sampler.cu) ----
 // rho = w |psi><psi| + (1 - w) I / d for the test state `kind` (QST_STATE_*), d x d complex.
