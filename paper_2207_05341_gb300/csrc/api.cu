@@ -177,6 +177,8 @@ struct qst_ctx {
   // a captured step with a page-locked host f copies f on a side stream, beside its first kernels
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_f = nullptr;
+  cudaEvent_t ev_check = nullptr;  // the result of the latest check of f
+  bool f_checked = false;  // the next step's new f has been checked by the batch that runs it
   bool f_wait = false;  // the stream must join ev_f before its first read of f
 };
 
@@ -216,6 +218,11 @@ void tmark_begin(qst_ctx* c) {
   c->tslot = c->tcount++;
   c->tmask[c->tslot] = 0u;
   record_mark(c, c->tev[(size_t)c->tslot * (QST_NPHASE + 1)]);
+}
+void tmark_drop(qst_ctx* c) {  // the step was refused: its slot is free again
+  if (c->tslot < 0) return;
+  c->tslot = -1;
+  c->tcount -= 1;
 }
 void tmark(qst_ctx* c, int phase) {
   if (c->tslot < 0) return;
@@ -381,20 +388,19 @@ const void* stage_input(qst_ctx* c, const void* f, size_t bytes, void* stage, qs
   return stage;
 }
 
-// Validate f (finite, >= 0, sum 1 within 1e-4) on the host: copies n reals back.
-template <class R> qst_status validate_f(qst_ctx* c, const void* fdev) {
-  const size_t n = (size_t)c->D.n;
-  std::vector<R> h(n);
-  QST_CU(cudaMemcpyAsync(h.data(), fdev, n * sizeof(R), cudaMemcpyDeviceToHost, c->stream));
-  QST_CU(cudaStreamSynchronize(c->stream));
-  double s = 0.0;
-  for (size_t i = 0; i < n; ++i) {
-    const double v = (double)h[i];
-    if (!(v >= 0.0) || !isfinite(v)) return QST_E_INPUT;
-    s += v;
-  }
-  if (fabs(s - 1.0) > 1e-4) return QST_E_INPUT;
+// Check f (finite, >= 0, sum 1 within 1e-4) on the GPU: check_f_begin enqueues the pass and the copy of its
+// result, check_f_end waits for that result alone, so that work enqueued in between runs while the host waits.
+template <class R> qst_status check_f_begin(qst_ctx* c, const void* fdev) {
+  Work<R>* w = W<R>(c);
+  if (!c->ev_check) QST_CU(cudaEventCreateWithFlags(&c->ev_check, cudaEventDisableTiming));
+  QST_CU(net_check_f<R>(c->D.n, (const R*)fdev, w->partials, w->counters + CNT_CHECK, w->scal + kCheckF, c->stream));
+  QST_CU(cudaMemcpyAsync(c->h_scal + kCheckF, w->scal + kCheckF, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  QST_CU(cudaEventRecord(c->ev_check, c->stream));
   return QST_OK;
+}
+qst_status check_f_end(qst_ctx* c) {
+  QST_CU(cudaEventSynchronize(c->ev_check));
+  return fabs(c->h_scal[kCheckF] - 1.0) <= 1e-4 ? QST_OK : QST_E_INPUT;  // NaN: refused
 }
 
 // The producer-side max slot of the scaled splits (NULL on the other paths).
@@ -684,6 +690,22 @@ template <class R> struct Engine {
     return QST_OK;
   }
 
+  // f's check and the hidden layer of a new f.  Where no other input's hidden layer is kept, the layer runs
+  // while the host waits for the check (an f aligned for its vector loads); otherwise it runs once f is
+  // accepted (a refused call changes nothing).
+  static qst_status check_and_hidden(qst_ctx* c, const R* theta, const R* f, bool run_hidden) {
+    if (c->f_checked) {
+      c->f_checked = false;
+      return run_hidden ? hidden(c, theta, f) : QST_OK;
+    }
+    qst_status st = check_f_begin<R>(c, f);
+    if (st != QST_OK) return st;
+    const bool beside = run_hidden && !c->hidden_valid && ((uintptr_t)f & 15u) == 0;
+    if (beside && (st = hidden(c, theta, f)) != QST_OK) return st;
+    if ((st = check_f_end(c)) != QST_OK) return st;
+    return run_hidden && !beside ? hidden(c, theta, f) : QST_OK;
+  }
+
   static qst_status read_loss(qst_ctx* c, double* loss) {
     Work<R>* w = W<R>(c);
     QST_CU(cudaMemcpyAsync(c->h_scal, w->scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
@@ -858,11 +880,8 @@ template <class R> struct Engine {
       const R* f = kind == 2 ? (const R*)f_user
                              : (const R*)stage_input(c, f_user, (size_t)D.n * sizeof(R), w->fstage, &st);
       if (kind != 2 && st != QST_OK) return st;
-      if (new_f && (st = validate_f<R>(c, f)) != QST_OK) return st;
       tmark_begin(c);
-      if (new_f && !c->cnn) {
-        if ((st = hidden(c, w->theta, f)) != QST_OK) return st;
-      }
+      if (new_f && (st = check_and_hidden(c, w->theta, f, !c->cnn)) != QST_OK) { tmark_drop(c); return st; }
       if ((st = step_body(c, f)) != QST_OK) return st;
       c->tslot = -1;
     }
@@ -881,10 +900,9 @@ template <class R> struct Engine {
     qst_status st;
     const R* f = (const R*)stage_input(c, f_user, (size_t)D.n * sizeof(R), w->fstage, &st);
     if (st != QST_OK) return st;
-    if ((st = validate_f<R>(c, f)) != QST_OK) return st;
+    if ((st = check_and_hidden(c, theta, f, true)) != QST_OK) return st;
     c->hidden_valid = false;  // the hidden buffers now hold the external parameters' activation
     c->fperm_stale = true;    // f is taken as new on every call
-    if ((st = hidden(c, theta, f)) != QST_OK) return st;
     if ((st = forward_state(c, theta, false)) != QST_OK) return st;
     if ((st = povm_likelihood(c, f, true)) != QST_OK) return st;
     if ((st = backward_state(c)) != QST_OK) return st;
@@ -930,8 +948,7 @@ template <class R> struct Engine {
     const R* f = (const R*)stage_input(c, f_user, (size_t)D.n * sizeof(R), w->fstage, &st);
     if (st != QST_OK) return st;
     if (c->cnn || !c->hidden_valid || f_user != c->f_last) {
-      if ((st = validate_f<R>(c, f)) != QST_OK) return st;
-      if ((st = hidden(c, w->theta, f)) != QST_OK) return st;
+      if ((st = check_and_hidden(c, w->theta, f, true)) != QST_OK) return st;
       c->hidden_valid = true;
       c->f_last = f_user;
     }
@@ -979,8 +996,7 @@ template <class R> struct Engine {
     const R* f = (const R*)stage_input(c, f_user, (size_t)D.n * sizeof(R), w->fstage, &st);
     if (st != QST_OK) return st;
     if (c->cnn || !c->hidden_valid || f_user != c->f_last) {
-      if ((st = validate_f<R>(c, f)) != QST_OK) return st;
-      if ((st = hidden(c, w->theta, f)) != QST_OK) return st;
+      if ((st = check_and_hidden(c, w->theta, f, true)) != QST_OK) return st;
       c->hidden_valid = true;
       c->f_last = f_user;
     }
@@ -1038,8 +1054,7 @@ template <class R> struct Engine {
     const R* f = (const R*)stage_input(c, f_user, (size_t)D.n * sizeof(R), w->fstage, &st);
     if (st != QST_OK) return st;
     if (c->cnn || !c->hidden_valid || f_user != c->f_last) {
-      if ((st = validate_f<R>(c, f)) != QST_OK) return st;
-      if ((st = hidden(c, w->theta, f)) != QST_OK) return st;
+      if ((st = check_and_hidden(c, w->theta, f, true)) != QST_OK) return st;
       c->hidden_valid = true;
       c->f_last = f_user;
     }
@@ -1065,10 +1080,9 @@ template <class R> struct Engine {
 #define QST_DISPATCH(c, call) ((c)->prec == QST_FP64 ? Engine<double>::call : Engine<float>::call)
 
 template <class R> qst_status reset_rprop(qst_ctx* c) {
-  Work<R>* w = W<R>(c);
-  const size_t P = c->P;
-  std::vector<R> h(P, rprop_encode((R)c->opt.lr, 0));  // step lr, previous sign 0
-  QST_CU(cudaMemcpyAsync(w->step, h.data(), P * sizeof(R), cudaMemcpyHostToDevice, c->stream));
+  // step lr, previous sign 0 (a fill on the GPU: the host copy of the state words it replaces took most of
+  // qst_set_params)
+  QST_CU(net_fill<R>(W<R>(c)->step, (long long)c->P, rprop_encode((R)c->opt.lr, 0), c->stream));
   QST_CU(cudaStreamSynchronize(c->stream));
   return QST_OK;
 }
@@ -1761,6 +1775,7 @@ void qst_destroy(qst_ctx* c) {
   if (c->h_flags) cudaFreeHost(c->h_flags);
   if (c->ev_fork) cudaEventDestroy(c->ev_fork);
   if (c->ev_f) cudaEventDestroy(c->ev_f);
+  if (c->ev_check) cudaEventDestroy(c->ev_check);
   if (c->copy_stream) cudaStreamDestroy(c->copy_stream);
   delete c;
 }
@@ -1832,10 +1847,18 @@ qst_status qst_batch_step(qst_batch* bt, const void* const* f, double* losses) {
   if (!steady) {
     // first iteration for these inputs: validate all of them before any tomography steps (a refused call
     // changes nothing), then build each hidden layer (not captured)
+    QST_CU(cudaEventRecord(bt->fork, bt->root));  // an earlier iteration may still use the contexts' scratch
     for (int b = 0; b < bt->B; ++b) {
       qst_ctx* c = bt->ctx[b];
       if (c->hidden_valid && c->f_last == f[b]) continue;
-      const qst_status st = c->prec == QST_FP64 ? validate_f<double>(c, f[b]) : validate_f<float>(c, f[b]);
+      QST_CU(cudaStreamWaitEvent(c->stream, bt->fork, 0));
+      const qst_status st = c->prec == QST_FP64 ? check_f_begin<double>(c, f[b]) : check_f_begin<float>(c, f[b]);
+      if (st != QST_OK) return st;
+    }
+    for (int b = 0; b < bt->B; ++b) {  // every check is in flight
+      qst_ctx* c = bt->ctx[b];
+      if (c->hidden_valid && c->f_last == f[b]) continue;
+      const qst_status st = check_f_end(c);
       if (st != QST_OK) return st;
     }
     QST_CU(cudaEventRecord(bt->fork, bt->root));
@@ -1843,7 +1866,9 @@ qst_status qst_batch_step(qst_batch* bt, const void* const* f, double* losses) {
       qst_ctx* c = bt->ctx[b];
       QST_CU(cudaStreamWaitEvent(c->stream, bt->fork, 0));
       const long long l0 = c->launches;
+      c->f_checked = !(c->hidden_valid && c->f_last == f[b]);
       const qst_status st = qst_step(c, f[b], nullptr);
+      c->f_checked = false;
       if (st < 0) return st;
       bt->launches += c->launches - l0;
       QST_CU(cudaEventRecord(bt->done[b], c->stream));

@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(256, 2) k_w1_pass(R* __restrict__ theta, R* __
 
 // ------------------------------------------------------------------ dL/dt from Y = G T
 // Gamma = Y + Y^dag;  dR_ij = 2 Re Gamma_ij, dR_ji = 2 Im Gamma_ij (i > j), dR_ii = Re Gamma_ii.
-template <class R>
+// GAUGE: Y + *gauge T in the place of Y (an instantiation of its own: the plain one keeps its registers).
+template <class R, bool GAUGE>
 __global__ void __launch_bounds__(256) k_symmetrize(const cx_t<R>* __restrict__ Y, R* __restrict__ dt, int d,
                                                      const double* gauge, const void* const* tab) {
   __shared__ R Ar[32][33], Ai[32][33], Br[32][33], Bi[32][33];
@@ -402,20 +403,26 @@ __global__ void __launch_bounds__(256) k_symmetrize(const cx_t<R>* __restrict__ 
       const int r = t >> 3, c = (t & 7) * 4;
       float v[4];
       // Y + g T: 4 g R_ij off the diagonal, 2 g R_ii on it (each thread replaces the entries of t it reads)
-      const float g4 = gauge ? 4.f * (float)*gauge : 0.f;
+      const float g4 = GAUGE ? 4.f * (float)*gauge : 0.f;
       float4 ta = make_float4(0.f, 0.f, 0.f, 0.f), tb = ta;
-      if (gauge) {
+      if (GAUGE) {
         ta = *reinterpret_cast<const float4*>(dt + (long long)(I * 32 + r) * d + J * 32 + c);
         if (I != J) tb = *reinterpret_cast<const float4*>(dt + (long long)(J * 32 + r) * d + I * 32 + c);
       }
       const float tav[4] = {ta.x, ta.y, ta.z, ta.w}, tbv[4] = {tb.x, tb.y, tb.z, tb.w};
       if (I != J) {
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = fmaf(g4, tav[u], R(2) * (Ar[r][c + u] + Br[c + u][r]));
+        for (int u = 0; u < 4; ++u) {
+          v[u] = R(2) * (Ar[r][c + u] + Br[c + u][r]);
+          if (GAUGE) v[u] = fmaf(g4, tav[u], v[u]);
+        }
         *reinterpret_cast<float4*>(dt + (long long)(I * 32 + r) * d + J * 32 + c) = make_float4(v[0], v[1], v[2], v[3]);
         // upper tile (J, I): element (J 32 + r, I 32 + c + u) = 2 Im Gamma_{(I 32 + c + u), (J 32 + r)}
 #pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = fmaf(g4, tbv[u], R(2) * (Ai[c + u][r] - Bi[r][c + u]));
+        for (int u = 0; u < 4; ++u) {
+          v[u] = R(2) * (Ai[c + u][r] - Bi[r][c + u]);
+          if (GAUGE) v[u] = fmaf(g4, tbv[u], v[u]);
+        }
         *reinterpret_cast<float4*>(dt + (long long)(J * 32 + r) * d + I * 32 + c) = make_float4(v[0], v[1], v[2], v[3]);
       } else {
 #pragma unroll
@@ -424,7 +431,7 @@ __global__ void __launch_bounds__(256) k_symmetrize(const cx_t<R>* __restrict__ 
           if (r > cc) v[u] = R(2) * (Ar[r][cc] + Ar[cc][r]);
           else if (r < cc) v[u] = R(2) * (Ai[cc][r] - Ai[r][cc]);
           else v[u] = R(2) * Ar[r][r];
-          v[u] = fmaf(r == cc ? 0.5f * g4 : g4, tav[u], v[u]);
+          if (GAUGE) v[u] = fmaf(r == cc ? 0.5f * g4 : g4, tav[u], v[u]);
         }
         *reinterpret_cast<float4*>(dt + (long long)(I * 32 + r) * d + J * 32 + c) = make_float4(v[0], v[1], v[2], v[3]);
       }
@@ -498,6 +505,62 @@ __global__ void __launch_bounds__(256) k_tri_grad(const cx_t<R>* __restrict__ Z,
   }
 }
 
+// ------------------------------------------------------------------ input check, Rprop reset
+// *out = sum f in FP64, or NaN when an entry is negative or not finite (a fixed order: per-thread sums, then the
+// blocks in turn).  One read of f, where the check on the host cost a copy of f to pageable memory and a serial
+// loop (3 ms of a 3.8 ms loss and gradient at N = 11; this pass takes about 10 us there, bound by FP64 adds).
+template <class R>
+__global__ void __launch_bounds__(256) k_check_f(const R* __restrict__ f, long long n, double* partials,
+                                                  unsigned int* counter, double* out) {
+  using VV = Vec<R>;
+  constexpr int VW = VV::W;
+  const bool vec = (reinterpret_cast<uintptr_t>(f) & 15u) == 0 && n % VW == 0;
+  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
+  double s = 0.0;
+  bool bad = false;
+  if (vec) {
+    for (long long i = tid; i < n / VW; i += nt) {
+      R v[VW];
+      VV::ld(f + i * VW, v);
+#pragma unroll
+      for (int u = 0; u < VW; ++u) {
+        bad |= !(v[u] >= R(0)) || !isfinite(v[u]);
+        s += (double)v[u];
+      }
+    }
+  } else {
+    for (long long i = tid; i < n; i += nt) {
+      const R v = f[i];
+      bad |= !(v >= R(0)) || !isfinite(v);
+      s += (double)v;
+    }
+  }
+  if (bad) s = nan("");
+  __shared__ double red[8];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double b = 0.0;
+    for (int w = 0; w < 8; ++w) b += red[w];
+    partials[blockIdx.x] = b;
+  }
+  if (last_block_arrived(counter) && threadIdx.x < 32) {
+    double b = 0.0;
+    for (int k = threadIdx.x; k < (int)gridDim.x; k += 32) b += partials[k];
+    b = warp_sum(b);
+    if (threadIdx.x == 0) {
+      *out = b;
+      *counter = 0u;
+    }
+  }
+}
+
+template <class R> __global__ void __launch_bounds__(256) k_fill(R* __restrict__ p, long long n, R v) {
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
+    p[i] = v;
+}
+
 // ------------------------------------------------------------------ launchers
 #define QST_SWITCH_H(H, ...)                      \
   switch (H) {                                    \
@@ -520,6 +583,18 @@ template <class R> static RpropCfg<R> rcfg(const NetCfg& c) {
   RpropCfg<R> r;
   r.eta_minus = (R)c.eta_minus; r.eta_plus = (R)c.eta_plus; r.step_min = (R)c.step_min; r.step_max = (R)c.step_max;
   return r;
+}
+
+template <class R>
+cudaError_t net_check_f(long long n, const R* f, double* partials, unsigned int* counter, double* out, cudaStream_t s) {
+  const int grid = stream_grid(k_check_f<R>, n / Vec<R>::W);
+  k_check_f<R><<<grid, 256, 0, s>>>(f, n, partials, counter, out);
+  return cudaGetLastError();
+}
+
+template <class R> cudaError_t net_fill(R* p, long long n, R v, cudaStream_t s) {
+  k_fill<R><<<stream_grid(k_fill<R>, n), 256, 0, s>>>(p, n, v);
+  return cudaGetLastError();
 }
 
 template <class R>
@@ -611,8 +686,9 @@ cudaError_t net_symmetrize(const Dims& D, const cx_t<R>* Y, R* dt, cudaStream_t 
   if (gauge && (TS != 32 || sizeof(R) != 4)) return cudaErrorInvalidValue;
   BatchArgs ba;
   if (batch_take(ba, {Y, dt, gauge})) return cudaSuccess;
-  return launch_dep(k_symmetrize<R>, dim3((unsigned)(nt * (nt + 1) / 2), 1, ba.nz), dim3(256), 0, s, Y, dt, D.d,
-                    gauge, ba.tab);
+  const dim3 grid((unsigned)(nt * (nt + 1) / 2), 1, ba.nz);
+  if (gauge) return launch_dep(k_symmetrize<R, true>, grid, dim3(256), 0, s, Y, dt, D.d, gauge, ba.tab);
+  return launch_dep(k_symmetrize<R, false>, grid, dim3(256), 0, s, Y, dt, D.d, gauge, ba.tab);
 }
 
 template <class R> cudaError_t net_tri_grad(const Dims& D, const cx_t<R>* Z, R* dt, cudaStream_t s) {
@@ -623,6 +699,8 @@ template <class R> cudaError_t net_tri_grad(const Dims& D, const cx_t<R>* Z, R* 
 }
 
 #define QST_INST(R)                                                                                              \
+  template cudaError_t net_check_f<R>(long long, const R*, double*, unsigned int*, double*, cudaStream_t);       \
+  template cudaError_t net_fill<R>(R*, long long, R, cudaStream_t);                                              \
   template cudaError_t net_l1_forward<R>(const Dims&, const R*, const R*, R*, R*, double*, double*, unsigned int*, \
                                          const NetCfg&, cudaStream_t);                                           \
   template cudaError_t net_build_T<R>(const Dims&, const R*, const R*, R*, cx_t<R>*, unsigned int*, cudaStream_t,  \

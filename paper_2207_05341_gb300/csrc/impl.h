@@ -111,7 +111,7 @@ template <class R> struct Work {
   R* fstage;           // staging copy of a host f, n reals
   R* fperm;            // f in the order of the structured likelihood pass (FP32 fast path), n reals
   double* scal;        // [0] Tr X, [1] sum f, [2] loss, [3] scale of T, [4] scale of G, [5] F_c,
-                       // [8..10] state fidelity (sum g, bracket bound, F_q), [12] kGauge
+                       // [8..10] state fidelity (sum g, bracket bound, F_q), [12] kGauge, [13] kCheckF
   double* partials;    // per-block partial sums
   unsigned int* counters;  // last-block counters, one per reduction site
   unsigned int* flags;     // [0] clamp count, [1] device-side wait timeouts, [2] sampler's bad input, [4] the
@@ -141,11 +141,13 @@ enum Counter {
   CNT_AMAXG = 9,  // the same for G
   CNT_FID = 10,   // classical fidelity reductions
   CNT_GX = 11,    // Tr(G X)
+  CNT_CHECK = 12,  // the check of f
   CNT_COUNT = 16
 };
 constexpr int kScaleT = 3;  // scal slot of the power-of-two scale of T (mixed path)
 constexpr int kScaleG = 4;  // scal slot of the scale of G
 constexpr int kGauge = 12;  // scal slot of the multiple of T that makes Tr(G X) = 0 (FP32 tensor-core products)
+constexpr int kCheckF = 13;  // scal slot of the sum of a new f, NaN for a bad entry
 constexpr int kPartialBlocks = 1024;   // max blocks of a reducing kernel
 constexpr int kPartialStride = 32;     // doubles per block in `partials` (>= H + 1)
 
@@ -233,6 +235,10 @@ cudaError_t tomo_fused_list(const TomoDesc* list, int count, const PovmB<float>&
                             unsigned int* next, cudaStream_t s);
 
 // ---- network (fnn.cu) ----
+// *out = sum f (FP64), or NaN when an entry is negative or not finite
+template <class R>
+cudaError_t net_check_f(long long n, const R* f, double* partials, unsigned int* counter, double* out, cudaStream_t s);
+template <class R> cudaError_t net_fill(R* p, long long n, R v, cudaStream_t s);
 template <class R> cudaError_t net_l1_forward(const Dims& D, const R* theta, const R* f, R* pre, R* hid,
                                               double* scal, double* partials, unsigned int* counter,
                                               const NetCfg& c, cudaStream_t s);
