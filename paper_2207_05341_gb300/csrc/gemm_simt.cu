@@ -1,4 +1,4 @@
-// Complex d x d products on the CUDA cores (the plain FP32 and FP64 paths):
+// Complex d x d products on the CUDA cores (FP64, and FP32 where gemm_tc_fp32.cu does not run them):
 //   X = T T   (Sec. 3.2 eq. unified_DP, Hermitian: only tiles I >= J are computed)
 //   Y = G T   (backward of X = T T)
 // Row-major complex operands.  Classic register-blocked tiling: a CTA computes a
@@ -8,6 +8,11 @@
 // (8 k by 4 m) fall in distinct bank groups; a thread's TN columns of B are
 // 16-byte chunks (CW complex each) spaced by the chunks of the other threads of
 // its row, so that the 16 threads of a row read consecutive chunks.
+//
+// FP64 has its own kernel (k_cgemm_f64): this part does 2 FP64 FMAs per clock and SM, a fortieth of its FP32
+// rate, so what counts is that every SM gets the same share of them, not the operand traffic.
+#include <cooperative_groups.h>
+
 #include "impl.h"
 
 namespace qst {
@@ -114,6 +119,84 @@ __global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_cgemm(int d, const cx
   }
 }
 
+// FP64, d >= 32: 16 x 16 output tiles, each the work of a cluster of gridDim.x / tiles CTAs that split K between
+// them (CTA r of a cluster takes d / ks consecutive k), so that the small sizes reach all SMs: at d = 128 the
+// 64 x 64 tiles it replaces were 3 and 4 CTAs on 152 SMs (521 us each; the FMAs alone are 7 and 13 us spread
+// over the chip, and 14 and 21 us is what this kernel takes).  A thread holds one row and two columns (8 FMAs per k from 3 entries).  The partial tiles
+// meet in distributed shared memory: CTA r sums rows r 16 / ks .. of all ranks, in the order of the ranks.
+constexpr int kT64 = 16;
+
+__global__ void __launch_bounds__(128) k_cgemm_f64(int d, const double2* __restrict__ A,
+                                                    const double2* __restrict__ B, double2* __restrict__ C, int lower,
+                                                    int ks) {
+  namespace cg = cooperative_groups;
+  __shared__ double2 As[2][kT64][kT64 + 1];
+  __shared__ double2 Bs[2][kT64][kT64];
+  __shared__ double2 part[kT64][kT64];
+  const int tile = (int)blockIdx.x / ks, rank = (int)blockIdx.x % ks, nt = d / kT64;
+  int I, J;
+  if (lower) tri_decode((uint32_t)tile, I, J);
+  else { I = tile / nt; J = tile % nt; }
+  const int tid = threadIdx.x, row = tid >> 3, col = tid & 7;
+  const int k0 = rank * (d / ks), steps = d / ks / kT64;
+  double2 ra[2], rb[2];
+  auto gload = [&](int k) {
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const int e = tid + 128 * l, r = e >> 4, c = e & 15;
+      ra[l] = A[(long long)(I * kT64 + r) * d + k + c];
+      rb[l] = B[(long long)(k + r) * d + J * kT64 + c];
+    }
+  };
+  double re[2] = {0.0, 0.0}, im[2] = {0.0, 0.0};
+  gload(k0);
+  for (int s = 0; s < steps; ++s) {
+    const int buf = s & 1;
+#pragma unroll
+    for (int l = 0; l < 2; ++l) {
+      const int e = tid + 128 * l;
+      As[buf][e >> 4][e & 15] = ra[l];
+      Bs[buf][e >> 4][e & 15] = rb[l];
+    }
+    __syncthreads();
+    if (s + 1 < steps) gload(k0 + (s + 1) * kT64);
+#pragma unroll
+    for (int k = 0; k < kT64; ++k) {
+      const double2 a = As[buf][row][k];
+#pragma unroll
+      for (int j = 0; j < 2; ++j) {
+        const double2 b = Bs[buf][k][col + 8 * j];
+        re[j] = fma(a.x, b.x, re[j]);
+        im[j] = fma(a.x, b.y, im[j]);
+        re[j] = fma(-a.y, b.y, re[j]);
+        im[j] = fma(a.y, b.x, im[j]);
+      }
+    }
+  }
+  double2* out = C + (long long)(I * kT64) * d + J * kT64;
+  if (ks == 1) {
+#pragma unroll
+    for (int j = 0; j < 2; ++j) out[(long long)row * d + col + 8 * j] = make_double2(re[j], im[j]);
+    return;
+  }
+#pragma unroll
+  for (int j = 0; j < 2; ++j) part[row][col + 8 * j] = make_double2(re[j], im[j]);
+  cg::cluster_group cl = cg::this_cluster();
+  cl.sync();
+  const int rows = kT64 / ks;
+  for (int e = tid; e < rows * kT64; e += 128) {
+    const int r = rank * rows + (e >> 4), c = e & 15;
+    double2 s = make_double2(0.0, 0.0);
+    for (int q = 0; q < ks; ++q) {
+      const double2 v = *cl.map_shared_rank(&part[r][c], q);
+      s.x += v.x;
+      s.y += v.y;
+    }
+    out[(long long)r * d + c] = s;
+  }
+  cl.sync();  // no CTA leaves while its part may still be read
+}
+
 // Small matrices (d <= 16): one thread per output element.
 template <class R>
 __global__ void k_cgemm_small(int d, const cx_t<R>* A, const cx_t<R>* B, cx_t<R>* C, int lower) {
@@ -153,12 +236,29 @@ cudaError_t cgemm_simt<float>(int d, const float2* A, const float2* B, float2* C
   return cudaGetLastError();
 }
 
+// At least four CTAs per SM where K can be split that far (16 elements of K per CTA, clusters of up to 8).
 template <>
 cudaError_t cgemm_simt<double>(int d, const double2* A, const double2* B, double2* C, bool lower, cudaStream_t s) {
-  if (d >= 64) return run_tiled<double, 64, 64, 8, 4, 4>(d, A, B, C, lower, s);
-  if (d == 32) return run_tiled<double, 32, 32, 8, 2, 2>(d, A, B, C, lower, s);
-  k_cgemm_small<double><<<1, 256, 0, s>>>(d, A, B, C, lower ? 1 : 0);
-  return cudaGetLastError();
+  if (d <= kT64) {
+    k_cgemm_small<double><<<1, 256, 0, s>>>(d, A, B, C, lower ? 1 : 0);
+    return cudaGetLastError();
+  }
+  if (d % kT64) return cudaErrorInvalidValue;
+  const int nt = d / kT64, tiles = lower ? nt * (nt + 1) / 2 : nt * nt;
+  int ks = 1;
+  while (ks < 8 && tiles * ks < 4 * 152 && d / (2 * ks) >= kT64) ks *= 2;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(tiles * ks));
+  cfg.blockDim = dim3(128);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)ks;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_cgemm_f64, d, A, B, C, lower ? 1 : 0, ks);
 }
 
 }  // namespace qst

@@ -168,7 +168,7 @@ template <class R>
 cudaError_t povm_lo_adj(const Dims& D, const R* Wadj, cx_t<R>* G, const PovmB<R>& B, unsigned int* amax,
                         cudaStream_t s);
 // Pauli-basis implementations of the high pass (povm_pauli.cu), used when povm_hi_pauli_ok(D)
-bool povm_hi_pauli_ok(const Dims& D);
+template <class R> bool povm_hi_pauli_ok(const Dims& D);
 template <class R> cudaError_t povm_hi_fwd_pauli(const Dims& D, const R* W, R* p, const PovmB<R>& B, cudaStream_t s);
 template <class R> cudaError_t povm_hi_nll_pauli(const Dims& D, const R* W, const R* f, double* scal, R* Wadj,
                                                  double* partials, unsigned int* counter, unsigned int* flags,

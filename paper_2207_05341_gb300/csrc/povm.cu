@@ -45,6 +45,9 @@ Dims make_dims(int N, bool fp64) {
   D.H = 2 * N;
   int g = N < 6 ? N : 6;
   if (!fp64 && N >= 12) g = 7;
+  // FP64 runs at 2 FMAs per clock and SM: small tiles, so that both passes reach every SM (a 64 x 64 tile is
+  // 65 us of one SM's FP64 pipe, and N = 7 has three), with at most 5 high qubits (the high pass's limit)
+  if (fp64 && N >= 5) g = N == 5 ? 3 : (N - 5 > 4 ? N - 5 : 4);
   D.g = g;
   D.h = N - g;
   D.S = 1 << g;
@@ -103,7 +106,8 @@ template <class R, bool ADJ>
 __device__ void apply_modes_tile(cx_t<R>* Z, int g, int pitch, const PovmB<R>& B) {
   using V = cx_t<R>;
   int b = 0;
-  for (; b + 1 < g; b += 2) {
+  // FP64: one qubit per sweep, so that a 16 x 16 tile keeps two warps on two FP64 pipes instead of half a warp
+  for (; sizeof(R) == 4 && b + 1 < g; b += 2) {
     const int gh = g - 2;
     const int groups = 1 << (2 * gh);
     const int low = (1 << b) - 1;
@@ -139,7 +143,7 @@ __device__ void apply_modes_tile(cx_t<R>* Z, int g, int pitch, const PovmB<R>& B
     }
     __syncthreads();
   }
-  if (b < g) {  // odd g: the last qubit alone
+  for (; b < g; ++b) {  // odd g: the last qubit alone
     const int half = g - 1;
     const int groups = 1 << (2 * half);
     const int bit = 1 << b, low = bit - 1;
@@ -463,7 +467,7 @@ cudaError_t povm_lo_adj(const Dims& D, const R* Wadj, cx_t<R>* G, const PovmB<R>
 
 template <class R>
 cudaError_t povm_hi_fwd(const Dims& D, const R* W, R* p, const PovmB<R>& B, cudaStream_t s) {
-  if (povm_hi_pauli_ok(D)) return povm_hi_fwd_pauli<R>(D, W, p, B, s);
+  if (povm_hi_pauli_ok<R>(D)) return povm_hi_fwd_pauli<R>(D, W, p, B, s);
   const size_t sm = (size_t)D.nb * D.nb * D.C * sizeof(cx_t<R>);
   cudaError_t e = set_smem<R>((const void*)k_povm_hi_fwd<R>, sm);
   if (e != cudaSuccess) return e;
@@ -476,7 +480,7 @@ template <class R>
 cudaError_t povm_hi_nll(const Dims& D, const R* W, const R* f, double* scal, R* Wadj, double* partials,
                         unsigned int* counter, unsigned int* flags, const PovmB<R>& B, bool adjoint,
                         cudaStream_t s) {
-  if (povm_hi_pauli_ok(D)) return povm_hi_nll_pauli<R>(D, W, f, scal, Wadj, partials, counter, flags, B, adjoint, s);
+  if (povm_hi_pauli_ok<R>(D)) return povm_hi_nll_pauli<R>(D, W, f, scal, Wadj, partials, counter, flags, B, adjoint, s);
   const size_t sm = (size_t)D.nb * D.nb * D.C * sizeof(cx_t<R>);
   cudaError_t e = set_smem<R>((const void*)k_povm_hi_nll<R>, sm);
   if (e != cudaSuccess) return e;

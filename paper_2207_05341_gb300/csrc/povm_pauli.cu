@@ -32,9 +32,9 @@ template <class T> __device__ __forceinline__ T min_norm();
 template <> __device__ __forceinline__ float min_norm<float>() { return FLT_MIN; }
 template <> __device__ __forceinline__ double min_norm<double>() { return DBL_MIN; }
 
-template <int NB> struct PGeo {
+template <int NB, int NW> struct PGeo {
   static constexpr int G = 32 / NB;          // matrices (low outcomes) per warp
-  static constexpr int CB = 8 * G;           // low outcomes per block (8 warps)
+  static constexpr int CB = NW * G;          // low outcomes per block (NW warps)
   static constexpr int LD = NB + 1;          // padded row of one staged matrix
   // pitch of one staged matrix: NB * LD rounded up to 32 / CB (mod 32), so that the
   // staging loop's 32 consecutive threads (CB low outcomes x 32 / CB entries) hit 32 banks
@@ -44,6 +44,12 @@ template <int NB> struct PGeo {
   static constexpr int FS = NB * NB * CB;    // staged f (reals)
   static_assert(MAT >= FS, "the matrix staging area also holds one value per outcome");
 };
+
+// Warps per block: 8; FP64, whose arithmetic is the bound, takes small blocks so that every SM gets some (N = 7:
+// 64 blocks of one warp, where 8 warps left 8 blocks).
+template <class R, int NB> __host__ __device__ constexpr int pauli_warps() {
+  return sizeof(R) == 4 ? 8 : (NB <= 8 ? 1 : NB / 8);
+}
 
 // In-register Walsh-Hadamard transform of v[0..NB): v_z <- sum_r (-1)^(z.r) v_r.
 template <class R, int NB> __device__ __forceinline__ void wht(R (&v)[NB]) {
@@ -129,11 +135,12 @@ __device__ __forceinline__ bool neg_phase(int x, int z) { return (__popc(x & z) 
 
 // MODE 0: forward only, write q to p.  MODE 1: likelihood (+ adjoint when adjoint != 0).
 template <class R, int NB, int MODE>
-__global__ void __launch_bounds__(256) k_povm_hi_pauli(const R* __restrict__ W, R* __restrict__ p,
+__global__ void __launch_bounds__(32 * pauli_warps<R, NB>()) k_povm_hi_pauli(const R* __restrict__ W, R* __restrict__ p,
                                                         const R* __restrict__ f, double* scal, R* __restrict__ Wadj,
                                                         double* partials, unsigned int* counter, unsigned int* flags,
                                                         int g, PovmB<R> B, int adjoint) {
-  using Gm = PGeo<NB>;
+  constexpr int NW = pauli_warps<R, NB>();
+  using Gm = PGeo<NB, NW>;
   constexpr int CB = Gm::CB, LD = Gm::LD, CP = Gm::CP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   R* mat = reinterpret_cast<R*>(smem_raw);
@@ -231,7 +238,7 @@ __global__ void __launch_bounds__(256) k_povm_hi_pauli(const R* __restrict__ W, 
   }
   __syncthreads();
   if (tid < 32) {
-    double v = tid < 8 ? red[tid] : 0.0;
+    double v = tid < NW ? red[tid] : 0.0;
     v = warp_sum(v);
     if (tid == 0) partials[blockIdx.x] = v;
   }
@@ -258,14 +265,15 @@ template <class R, int NB, int MODE>
 cudaError_t launch_pauli(const Dims& D, const R* W, R* p, const R* f, double* scal, R* Wadj, double* partials,
                          unsigned int* counter, unsigned int* flags, const PovmB<R>& B, bool adjoint,
                          cudaStream_t s) {
-  using Gm = PGeo<NB>;
+  constexpr int NW = pauli_warps<R, NB>();
+  using Gm = PGeo<NB, NW>;
   const size_t sm = (size_t)(Gm::MAT + (MODE == 1 ? Gm::FS : 0)) * sizeof(R);
   cudaError_t e = ensure_dynamic_smem((const void*)k_povm_hi_pauli<R, NB, MODE>, sm);
   if (e != cudaSuccess) return e;
   const long long SS = 1LL << (2 * D.g);
   const unsigned blocks = (unsigned)(SS / Gm::CB);
   if (MODE == 1 && blocks > (unsigned)kPartialBlocks * kPartialStride) return cudaErrorInvalidConfiguration;
-  k_povm_hi_pauli<R, NB, MODE><<<blocks, 256, sm, s>>>(W, p, f, scal, Wadj, partials, counter, flags, D.g, B,
+  k_povm_hi_pauli<R, NB, MODE><<<blocks, 32 * NW, sm, s>>>(W, p, f, scal, Wadj, partials, counter, flags, D.g, B,
                                                        adjoint ? 1 : 0);
   return cudaGetLastError();
 }
@@ -286,7 +294,11 @@ cudaError_t dispatch_pauli(const Dims& D, const R* W, R* p, const R* f, double* 
 
 }  // namespace
 
-bool povm_hi_pauli_ok(const Dims& D) { return D.nb >= 2 && D.nb <= 32 && D.g >= 6; }
+template <class R> bool povm_hi_pauli_ok(const Dims& D) {
+  return D.nb >= 2 && D.nb <= 32 && D.g >= (sizeof(R) == 4 ? 6 : 3);  // whole blocks of low outcomes
+}
+template bool povm_hi_pauli_ok<float>(const Dims&);
+template bool povm_hi_pauli_ok<double>(const Dims&);
 
 template <class R>
 cudaError_t povm_hi_fwd_pauli(const Dims& D, const R* W, R* p, const PovmB<R>& B, cudaStream_t s) {
