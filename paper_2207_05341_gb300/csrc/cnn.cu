@@ -414,9 +414,9 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
   }
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
 #pragma unroll
-  for (int j = 0; j < H; ++j) {
-    const double x = warp_sum((double)acc[j]);
-    if (lane == 0) red[wp][j] = x;
+  for (int j0 = 0; j0 < H; j0 += 4) {  // H = 4 N: four rows at a time
+    const R a4[4] = {acc[j0], acc[j0 + 1], acc[j0 + 2], acc[j0 + 3]};
+    warp_sums<4>(a4, [&](int j, double x) { red[wp][j0 + j] = x; });
   }
   __syncthreads();
   for (int j = threadIdx.x; j < H; j += blockDim.x) {

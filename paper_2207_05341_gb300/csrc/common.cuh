@@ -135,6 +135,45 @@ __device__ __forceinline__ double warp_sum(double v) {
   return v;
 }
 
+// Sums of M values each over a warp: out(j, sum) is called once per j, by one lane.  Step by step a lane hands half
+// of the values it still carries to its partner, which hands over the other half, so M = 11 takes 16 FP64 adds
+// where M butterflies take 55 (an FP64 add is 64 issue cycles of a scheduler here: two per clock and SM).  The
+// pairs added are warp_sum's, so every sum has its bits.
+template <int M, class R, class F> __device__ __forceinline__ void warp_sums(const R (&v)[M], F out) {
+  static_assert(M >= 1 && M <= 32, "at most one value per lane");
+  constexpr int L = M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : M <= 16 ? 4 : 5, P = 1 << L;
+  const int lane = threadIdx.x & 31;
+  double a[P > 1 ? P / 2 : 1];
+  if constexpr (P == 1) {
+    a[0] = warp_sum((double)v[0]);
+  } else {
+    const bool up = (lane & 16) != 0;
+#pragma unroll
+    for (int k = 0; k < P / 2; ++k) {
+      const R lo = k < M ? v[k < M ? k : 0] : R(0), hi = k + P / 2 < M ? v[k + P / 2 < M ? k + P / 2 : 0] : R(0);
+      const R keep = up ? hi : lo, send = up ? lo : hi;
+      a[k] = (double)keep + (double)__shfl_xor_sync(0xffffffffu, send, 16);
+    }
+#pragma unroll
+    for (int o = 8, c = P / 2; o > 0; o >>= 1) {
+      if (c > 1) {
+        c >>= 1;
+        const bool u = (lane & o) != 0;
+#pragma unroll
+        for (int k = 0; k < P / 4; ++k) {
+          if (k >= c) break;
+          const double keep = u ? a[k + c] : a[k], send = u ? a[k] : a[k + c];
+          a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+      } else {
+        a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+      }
+    }
+  }
+  const int j = lane >> (5 - L);
+  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) out(j, a[0]);
+}
+
 // "Last block done": every block has written its partial; the last one to arrive
 // returns true (for all its threads).  The counter is reset by the caller's last block.
 __device__ __forceinline__ bool last_block_arrived(unsigned int* counter) {

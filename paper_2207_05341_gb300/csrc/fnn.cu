@@ -31,12 +31,8 @@ constexpr int kRowBatch = 4;
 template <int M, class R>
 __device__ __forceinline__ void block_reduce_to(const R (&v)[M], double* out) {
   __shared__ double red[8][M];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    double x = warp_sum((double)v[j]);
-    if (lane == 0) red[w][j] = x;
-  }
+  const int w = threadIdx.x >> 5;
+  warp_sums<M>(v, [&](int j, double x) { red[w][j] = x; });
   __syncthreads();
   const int nw = blockDim.x >> 5;
   for (int j = threadIdx.x; j < M; j += blockDim.x) {

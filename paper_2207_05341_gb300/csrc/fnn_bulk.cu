@@ -125,14 +125,8 @@ template <class R> __device__ __forceinline__ R leaky_b(R x, R slope) { return x
 template <int M>
 __device__ __forceinline__ void block_sum_to(const float (&v)[M], double* out) {
   __shared__ double red[kConsumerWarps][M];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  if (w < kConsumerWarps) {
-#pragma unroll
-    for (int j = 0; j < M; ++j) {
-      double x = warp_sum((double)v[j]);
-      if (lane == 0) red[w][j] = x;
-    }
-  }
+  const int w = threadIdx.x >> 5;
+  if (w < kConsumerWarps) warp_sums<M>(v, [&](int j, double x) { red[w][j] = x; });
   __syncthreads();
   for (int j = threadIdx.x; j < M; j += blockDim.x) {
     double s = 0.0;
@@ -314,11 +308,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
   {
     __shared__ double red[kGroups * kConsumerWarps][RPT + 1];
     if (warp < kConsumers / 32) {
-#pragma unroll
-      for (int l = 0; l < RPT; ++l) {
-        const double x = warp_sum((double)acc[l]);
-        if (lane == 0) red[warp][l] = x;
-      }
+      warp_sums<RPT>(acc, [&](int l, double x) { red[warp][l] = x; });
       if (!W2 && rg == 0) {
         const double x = warp_sum((double)accf);
         if (lane == 0) red[warp][RPT] = x;

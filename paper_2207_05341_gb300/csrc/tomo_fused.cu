@@ -49,12 +49,8 @@ struct Smem {
 constexpr int kTot = 31 * 16;
 template <int M> __device__ void block_sum(const float (&v)[M], double* red) {
   static_assert(M <= 16, "at most 16 values per reduction");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-#pragma unroll
-  for (int j = 0; j < M; ++j) {
-    const double s = warp_sum((double)v[j]);
-    if (lane == 0) red[warp * 16 + j] = s;
-  }
+  const int warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  warp_sums<M>(v, [&](int j, double s) { red[warp * 16 + j] = s; });
   __syncthreads();
   if (threadIdx.x < M) {
     double s = 0.0;
