@@ -1058,9 +1058,22 @@ template <class R> struct Engine {
       c->hidden_valid = true;
       c->f_last = f_user;
     }
-    if ((st = forward_state(c, w->theta)) != QST_OK) return st;
     const bool dev = is_device_ptr(rho_out);
     V* dst = dev ? (V*)rho_out : w->G;
+    if constexpr (std::is_same<R, float>::value) {
+      if (fused(c)) {  // rho and its loss in one launch
+        TomoDesc td = tomo_desc(c, f);
+        td.rho = dst;
+        QST_CU(tomo_fused_one(td, c->Bf, c->net, c->stream));
+        c->launches += 1;
+        if (rho_out && !dev) {
+          QST_CU(cudaMemcpyAsync(rho_out, dst, (size_t)D.d * D.d * sizeof(V), cudaMemcpyDeviceToHost, c->stream));
+          QST_CU(cudaStreamSynchronize(c->stream));
+        }
+        return loss ? read_loss(c, loss) : QST_OK;
+      }
+    }
+    if ((st = forward_state(c, w->theta)) != QST_OK) return st;
     if (rho_out) {
       QST_CU(hermitian_complete<R>(D, w->X, dst, w->scal, c->stream));
       c->launches += 1;

@@ -224,6 +224,7 @@ struct TomoDesc {
   float2 *T, *X, *G, *Y;  // d x d complex scratch
   double* scal;         // [0] Tr X, [1] sum f (read, then rewritten), [2] loss
   unsigned int* flags;  // [0] clamp count
+  float2* rho;          // not NULL: rho = X / Tr X into it (d x d) and the loss, no update
   int N;
 };
 // max_qubits: the context's option (0: the tuned default, < 0: never)
