@@ -1062,8 +1062,9 @@ template <class R> struct Engine {
     V* dst = dev ? (V*)rho_out : w->G;
     if constexpr (std::is_same<R, float>::value) {
       if (fused(c)) {  // rho and its loss in one launch
+        if (!dev) dst = w->Y;  // G is written after rho where the matrices are in the context's buffers
         TomoDesc td = tomo_desc(c, f);
-        td.rho = dst;
+        td.rho = reinterpret_cast<float2*>(dst);
         QST_CU(tomo_fused_one(td, c->Bf, c->net, c->stream));
         c->launches += 1;
         if (rho_out && !dev) {
