@@ -387,72 +387,83 @@ __device__ __forceinline__ double2 ld_after_wait(const double2* p) {
   return v;
 }
 
-// One warp per coset: the G x G principal block B of A on the coset and U = R_1 ... R_{G-1} in shared memory,
-// round s (s = 1 .. G - 1, the subspace element of local index s) rotating the local pairs {x, x ^ s}, each
-// rotation computed from B after the rounds before it (B <- R^dag B R, U <- U R).  Writes U to Ug[coset].
-// Lets the pass's block kernel start (its loads of A do not depend on U).
-template <class R, int G>
-__global__ void __launch_bounds__(32) k_coset_unitaries(const cx_t<R>* __restrict__ A, int d, JacobiPass p,
-                                                        cx_t<R>* __restrict__ Ug) {
-  using V = cx_t<R>;
-  asm volatile("griddepcontrol.launch_dependents;");
-  __shared__ V B[G][G + 1], U[G][G + 1];
-  __shared__ Rot2<R> rot[G / 2];
-  __shared__ int e[G];
-  const int c = blockIdx.x, lane = threadIdx.x;
-  if (lane < G) e[lane] = coset_element(coset_rep(c, p), lane, p);
-  __syncwarp();
-  for (int x = lane; x < G * G; x += 32) {
-    const int i = x / G, j = x % G;
-    B[i][j] = A[(long long)e[i] * d + e[j]];
-    U[i][j] = cmake<V>(i == j ? R(1) : R(0), R(0));
-  }
-  __syncwarp();
-  for (int s = 1; s < G; ++s) {
-    const int hb = 31 - __clz(s);
-    if (lane < G / 2) {
-      const int pp = insert_zero(lane, hb), q = pp ^ s;
-      rot[lane] = rotation_for<R>(B[pp][pp].x, B[q][q].x, B[pp][q]);
-    }
-    __syncwarp();
-    for (int x = lane; x < G * (G / 2); x += 32) {  // columns p, q of row i of B and of U: X <- X R
-      const int i = x / (G / 2), l = x % (G / 2);
-      const int pp = insert_zero(l, hb), q = pp ^ s;
-      const Rot2<R> r = rot[l];
-      const V rqp = cmake<V>(-r.emph.x * r.sn, -r.emph.y * r.sn), rqq = cmake<V>(r.emph.x * r.cs, r.emph.y * r.cs);
-      const V bp = B[i][pp], bq = B[i][q];
-      B[i][pp] = cadd(cmake<V>(bp.x * r.cs, bp.y * r.cs), cmul(bq, rqp));
-      B[i][q] = cadd(cmake<V>(bp.x * r.sn, bp.y * r.sn), cmul(bq, rqq));
-      const V up = U[i][pp], uq = U[i][q];
-      U[i][pp] = cadd(cmake<V>(up.x * r.cs, up.y * r.cs), cmul(uq, rqp));
-      U[i][q] = cadd(cmake<V>(up.x * r.sn, up.y * r.sn), cmul(uq, rqq));
-    }
-    __syncwarp();
-    for (int x = lane; x < (G / 2) * G; x += 32) {  // rows p, q of B: B <- R^dag B
-      const int l = x / G, j = x % G;
-      const int pp = insert_zero(l, hb), q = pp ^ s;
-      const Rot2<R> r = rot[l];
-      const V rqp = cmake<V>(-r.emph.x * r.sn, -r.emph.y * r.sn), rqq = cmake<V>(r.emph.x * r.cs, r.emph.y * r.cs);
-      const V bp = B[pp][j], bq = B[q][j];
-      B[pp][j] = cadd(cmake<V>(r.cs * bp.x, r.cs * bp.y), cmulc(rqp, bq));
-      B[q][j] = cadd(cmake<V>(r.sn * bp.x, r.sn * bp.y), cmulc(rqq, bq));
-    }
-    __syncwarp();
-  }
-  V* out = Ug + (size_t)c * G * G;
-  for (int x = lane; x < G * G; x += 32) out[x] = U[x / G][x % G];
+// Entries of X R and R^dag X for a rotation: s p + q z and s p + conj(z) q, rounded in one fixed way, so that the
+// bits of a decomposition do not depend on how a kernel around them is compiled (at FP32 two roundings of the
+// same sweeps give states that differ by 2.6e-5 at N = 9, more than any one of them changes in use).
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+template <class R, class V> __device__ __forceinline__ V rot_col(R s, V p, V q, V z) {
+  return cmake<V>(fma(s, p.x, fma(q.x, z.x, -mul_rn(q.y, z.y))), fma(s, p.y, fma(q.x, z.y, mul_rn(q.y, z.x))));
+}
+template <class R, class V> __device__ __forceinline__ V rot_row(R s, V p, V z, V q) {
+  return cmake<V>(fma(s, p.x, fma(z.x, q.x, mul_rn(z.y, q.y))), fma(s, p.y, fma(z.x, q.y, -mul_rn(z.y, q.x))));
 }
 
-// Asynchronous copy of one complex entry from global to shared memory (no register on the way), and the wait
-// for all of this thread's copies.
-template <class V> __device__ __forceinline__ void cp_async_entry(V* dst, const V* src) {
-  const uint32_t s = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
-  if constexpr (sizeof(V) == 8)
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(s), "l"(src) : "memory");
-  else
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(s), "l"(src) : "memory");
+// The unitary of one coset per CTA of G^2 / 2 threads: the G x G principal block B of A on the coset and
+// U = R_1 ... R_{G-1} in shared memory, round s (s = 1 .. G - 1, the subspace element of local index s) rotating
+// the local pairs {x, x ^ s}, each rotation computed from B after the rounds before it (B <- R^dag B R, U <- U R).
+// Writes U to Ug[coset].  What bounds it is the chain of rounds, and in a round the rotation (a hypot, three
+// divisions and two square roots, about 110 dependent instructions), so the rest is one entry pair per thread:
+// thread (i, l) forms the rotation of pair l itself, without waiting for another's, and rotates columns p, q of
+// row i of B and U; then thread (l, j) rotates rows p, q of column j of B.  B has two copies, one per half round,
+// so that a round needs two barriers (of a single warp at G = 8).  With a warp per coset looping over the entries
+// the kernel took 7.0 us at G = 8 and 20.3 us at G = 16, TIMES now.
+template <class R, int G>
+__global__ void __launch_bounds__(G * G / 2) k_coset_unitaries(const cx_t<R>* A, int d, JacobiPass p,
+                                                               cx_t<R>* __restrict__ Ug) {
+  using V = cx_t<R>;
+  __shared__ V B[G][G + 1], C[G][G + 1], U[G][G + 1];
+  __shared__ Rot2<R> rot[G / 2];
+  auto sync = [] {
+    if constexpr (G * G / 2 <= 32) __syncwarp();
+    else __syncthreads();
+  };
+  const int c = blockIdx.x, t = threadIdx.x;
+  const int i = t / (G / 2), l = t % (G / 2);  // first half of a round
+  const int l2 = t / G, j2 = t % G;            // second half
+  const int rep = coset_rep(c, p);
+  grid_dep_wait();  // the pass before
+  after_wait(A, Ug);
+  asm volatile("griddepcontrol.launch_dependents;");  // the block kernel's loads of A do not depend on U
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int r = t / G + h * (G / 2);
+    B[r][j2] = ld_after_wait(A + (long long)coset_element(rep, r, p) * d + coset_element(rep, j2, p));
+    U[r][j2] = cmake<V>(r == j2 ? R(1) : R(0), R(0));
+  }
+  sync();
+#pragma unroll 1
+  for (int s = 1; s < G; ++s) {
+    const int hb = 31 - __clz(s);
+    {
+      const int pp = insert_zero(l, hb), q = pp ^ s;
+      const V bp = B[i][pp], bq = B[i][q], up = U[i][pp], uq = U[i][q];
+      const Rot2<R> r = rotation_for<R>(B[pp][pp].x, B[q][q].x, B[pp][q]);
+      const V rqp = cmake<V>(-r.emph.x * r.sn, -r.emph.y * r.sn), rqq = cmake<V>(r.emph.x * r.cs, r.emph.y * r.cs);
+      C[i][pp] = rot_col(r.cs, bp, bq, rqp);
+      C[i][q] = rot_col(r.sn, bp, bq, rqq);
+      U[i][pp] = rot_col(r.cs, up, uq, rqp);
+      U[i][q] = rot_col(r.sn, up, uq, rqq);
+      if (i == 0) rot[l] = r;
+    }
+    sync();
+    {
+      const int pp = insert_zero(l2, hb), q = pp ^ s;
+      const Rot2<R> r = rot[l2];
+      const V rqp = cmake<V>(-r.emph.x * r.sn, -r.emph.y * r.sn), rqq = cmake<V>(r.emph.x * r.cs, r.emph.y * r.cs);
+      const V bp = C[pp][j2], bq = C[q][j2];
+      B[pp][j2] = rot_row(r.cs, bp, rqp, bq);
+      B[q][j2] = rot_row(r.sn, bp, rqq, bq);
+    }
+    sync();
+  }
+  V* out = Ug + (size_t)c * G * G;
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    const int e = t + h * (G * G / 2);
+    out[e] = U[e / G][e % G];
+  }
 }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // RB consecutive unitary entries from shared memory: FP32 two per 16-byte load, as the broadcast pairs
 // (u.x, u.x) in ux and (u.y, u.y) in uy that the packed products take; FP64 as they are (uy unused).
@@ -490,7 +501,8 @@ template <class R, int G, int TS> struct TileSmem {
 // column cosets x TS / G .. in shared memory (loaded before waiting for the pass's unitaries), computes
 // T = A U_l and V' = V U_l (U block-diagonal over the cosets), then A' = U_k^dag T, each thread an RB x RB
 // block of outputs, and writes both tiles back.  Every entry is read and written once per pass.
-template <class R, int G, int TS>
+// HASV: eigenvectors are accumulated (Vi, Vo); without, V takes no shared memory traffic and no arithmetic.
+template <class R, int G, int TS, bool HASV>
 __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__ A, cx_t<R>* __restrict__ Ao,
                                                       const cx_t<R>* __restrict__ Vi, cx_t<R>* __restrict__ Vo,
                                                       cx_t<R>* __restrict__ phi, int d, JacobiPass p,
@@ -505,16 +517,33 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
   if (t < TS) S.ridx[t] = coset_element(coset_rep(k0 + t / G, p), t % G, p);
   else if (t < 2 * TS) S.cidx[t - TS] = coset_element(coset_rep(l0 + (t - TS) / G, p), (t - TS) % G, p);
   __syncthreads();
-  for (int e = t; e < TS * TS; e += 256) {  // every copy of the tiles in flight at once
-    const int r = e / TS, c = e % TS;
-    const long long off = (long long)S.ridx[r] * d + S.cidx[c];
-    cp_async_entry(&S.a[r][c + c / G], A + off);
-    if (Vi != nullptr) cp_async_entry(&S.v[r][c + c / G], Vi + off);
+  // this thread's column and rows of the tiles (t / TS and every 256 / TS after it)
+  const int tc = t % TS, tr = t / TS, tcs = tc + tc / G;
+  constexpr int kStep = 256 / TS;
+  const int gc = S.cidx[tc];
+  {
+    // Every load of the tiles in flight at once, before the wait for this pass's unitaries: the pass before was
+    // complete when their kernel let this one start.  Through L2 only (a line of the same buffer may be left in L1
+    // from two passes ago).
+    constexpr int kPer = TS / kStep;
+    V ra[kPer], rv[HASV ? kPer : 1];
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      const long long off = (long long)S.ridx[tr + k * kStep] * d + gc;
+      ra[k] = ld_after_wait(A + off);
+      if (HASV) rv[k] = ld_after_wait(Vi + off);
+    }
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      S.a[tr + k * kStep][tcs] = ra[k];
+      if (HASV) S.v[tr + k * kStep][tcs] = rv[k];
+    }
   }
-  const bool with_phi = phi != nullptr && blockIdx.x == 0;
-  if (with_phi && t < TS) S.ph[t] = phi[S.ridx[t]];
   grid_dep_wait();  // the unitaries of this pass
   after_wait(Ug);
+  asm volatile("griddepcontrol.launch_dependents;");
+  const bool with_phi = phi != nullptr && blockIdx.x == 0;
+  if (with_phi && t < TS) S.ph[t] = ld_after_wait(phi + S.ridx[t]);
   for (int e = t; e < TPC * G * G; e += 256) {
     const int cc = e / (G * G), rc = (e / G) % G, jc = e % G;
     const V ul = ld_after_wait(Ug + (size_t)(l0 + cc) * G * G + rc * G + jc);
@@ -522,7 +551,6 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
     S.ul[cc][rc][jc] = ul;
     S.uk[cc][rc][jc] = uk;
   }
-  cp_async_wait_all();
   __syncthreads();
   if (with_phi && t < TS) {  // phi <- U_k^dag phi on the row cosets
     const int rc = t / G, i = t % G;
@@ -551,19 +579,19 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
 #pragma unroll
       for (int i = 0; i < RB; ++i) {
         const V m = S.a[rr + 16 * i][cc * (G + 1) + q];
-        const V w = Vi != nullptr ? S.v[rr + 16 * i][cc * (G + 1) + q] : cmake<V>(R(0), R(0));
+        const V w = HASV ? S.v[rr + 16 * i][cc * (G + 1) + q] : cmake<V>(R(0), R(0));
         if constexpr (kF32) {
           const float2 msw = make_float2(-m.y, m.x), wsw = make_float2(-w.y, w.x);  // i m, i w
 #pragma unroll
           for (int j = 0; j < RB; ++j) {  // m u = u.x m + u.y (i m)
             acc[i][j] = __ffma2_rn(uy[j], msw, __ffma2_rn(ux[j], m, acc[i][j]));
-            accv[i][j] = __ffma2_rn(uy[j], wsw, __ffma2_rn(ux[j], w, accv[i][j]));
+            if (HASV) accv[i][j] = __ffma2_rn(uy[j], wsw, __ffma2_rn(ux[j], w, accv[i][j]));
           }
         } else {
 #pragma unroll
           for (int j = 0; j < RB; ++j) {
             acc[i][j] = cadd(acc[i][j], cmul(m, ux[j]));
-            accv[i][j] = cadd(accv[i][j], cmul(w, ux[j]));
+            if (HASV) accv[i][j] = cadd(accv[i][j], cmul(w, ux[j]));
           }
         }
       }
@@ -574,10 +602,15 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
 #pragma unroll
       for (int j = 0; j < RB; ++j) {
         S.a[rr + 16 * i][c0 + j + cc] = acc[i][j];
-        S.v[rr + 16 * i][c0 + j + cc] = accv[i][j];
+        if (HASV) S.v[rr + 16 * i][c0 + j + cc] = accv[i][j];
       }
   }
   __syncthreads();
+  if (HASV) {  // V' leaves while A' is formed
+    V* vc = Vo + gc;
+#pragma unroll 4
+    for (int r = tr; r < TS; r += kStep) vc[(long long)S.ridx[r] * d] = S.v[r][tcs];
+  }
   {  // A' = U_k^dag T: lane l of warp w takes the RB rows of row block rb = 2 w + l / 16 (inside row coset rc)
      // and columns cs + 16 j (cs = l % 16)
     const int cs = lane % 16, rb = 2 * warp + lane / 16;
@@ -615,12 +648,10 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
       }
   }
   __syncthreads();
+  {
+    V* ac = Ao + gc;
 #pragma unroll 4
-  for (int e = t; e < TS * TS; e += 256) {
-    const int r = e / TS, c = e % TS;
-    const long long off = (long long)S.ridx[r] * d + S.cidx[c];
-    Ao[off] = S.a[r][c + c / G];
-    if (Vi != nullptr) Vo[off] = S.v[r][c + c / G];
+    for (int r = tr; r < TS; r += kStep) ac[(long long)S.ridx[r] * d] = S.a[r][tcs];
   }
 }
 
@@ -821,12 +852,15 @@ cudaError_t tile_pass(int d, const JacobiPass& p, const cx_t<R>* A, cx_t<R>* Ao,
                       cx_t<R>* phi, cx_t<R>* ucos, cudaStream_t s) {
   constexpr int TS = sizeof(R) == 4 ? 64 : 32;
   const size_t smem = sizeof(TileSmem<R, G, TS>);
-  cudaError_t e = ensure_dynamic_smem((const void*)k_jacobi_tile<R, G, TS>, smem);
+  const void* fn = Vi ? (const void*)k_jacobi_tile<R, G, TS, true> : (const void*)k_jacobi_tile<R, G, TS, false>;
+  cudaError_t e = ensure_dynamic_smem(fn, smem);
   if (e != cudaSuccess) return e;
-  k_coset_unitaries<R, G><<<d / G, 32, 0, s>>>(A, d, p, ucos);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  return launch_dep(k_jacobi_tile<R, G, TS>, dim3(d / TS, d / TS), dim3(256), smem, s, A, Ao, Vi, Vo, phi, d, p,
-                    (const cx_t<R>*)ucos);
+  e = launch_dep(k_coset_unitaries<R, G>, dim3(d / G), dim3(G * G / 2), 0, s, A, d, p, ucos);
+  if (e != cudaSuccess) return e;
+  const dim3 grid(d / TS, d / TS);
+  const cx_t<R>* U = ucos;
+  return Vi ? launch_dep(k_jacobi_tile<R, G, TS, true>, grid, dim3(256), smem, s, A, Ao, Vi, Vo, phi, d, p, U)
+            : launch_dep(k_jacobi_tile<R, G, TS, false>, grid, dim3(256), smem, s, A, Ao, Vi, Vo, phi, d, p, U);
 }
 
 // One sweep: every pass of the schedule, ping-ponging (Ain, Aout) and (Vin, Vout).  Passes over cosets of 8
