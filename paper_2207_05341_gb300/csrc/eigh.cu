@@ -407,7 +407,7 @@ template <class R, class V> __device__ __forceinline__ V rot_row(R s, V p, V z, 
 // thread (i, l) forms the rotation of pair l itself, without waiting for another's, and rotates columns p, q of
 // row i of B and U; then thread (l, j) rotates rows p, q of column j of B.  B has two copies, one per half round,
 // so that a round needs two barriers (of a single warp at G = 8).  With a warp per coset looping over the entries
-// the kernel took 7.0 us at G = 8 and 20.3 us at G = 16, TIMES now.
+// the kernel took 7.0 us at G = 8 and 20.3 us at G = 16, 5.9 and 10.2 us now.
 template <class R, int G>
 __global__ void __launch_bounds__(G * G / 2) k_coset_unitaries(const cx_t<R>* A, int d, JacobiPass p,
                                                                cx_t<R>* __restrict__ Ug) {
@@ -847,10 +847,9 @@ std::vector<JacobiPass> build_schedule(int N) {
 
 constexpr int kMaxScheduleN = 14;
 
-template <class R, int G>
-cudaError_t tile_pass(int d, const JacobiPass& p, const cx_t<R>* A, cx_t<R>* Ao, const cx_t<R>* Vi, cx_t<R>* Vo,
-                      cx_t<R>* phi, cx_t<R>* ucos, cudaStream_t s) {
-  constexpr int TS = sizeof(R) == 4 ? 64 : 32;
+template <class R, int G, int TS>
+cudaError_t tile_pass_sized(int d, const JacobiPass& p, const cx_t<R>* A, cx_t<R>* Ao, const cx_t<R>* Vi, cx_t<R>* Vo,
+                            cx_t<R>* phi, cx_t<R>* ucos, cudaStream_t s) {
   const size_t smem = sizeof(TileSmem<R, G, TS>);
   const void* fn = Vi ? (const void*)k_jacobi_tile<R, G, TS, true> : (const void*)k_jacobi_tile<R, G, TS, false>;
   cudaError_t e = ensure_dynamic_smem(fn, smem);
@@ -861,6 +860,15 @@ cudaError_t tile_pass(int d, const JacobiPass& p, const cx_t<R>* A, cx_t<R>* Ao,
   const cx_t<R>* U = ucos;
   return Vi ? launch_dep(k_jacobi_tile<R, G, TS, true>, grid, dim3(256), smem, s, A, Ao, Vi, Vo, phi, d, p, U)
             : launch_dep(k_jacobi_tile<R, G, TS, false>, grid, dim3(256), smem, s, A, Ao, Vi, Vo, phi, d, p, U);
+}
+
+// 64 x 64 tiles; 32 x 32 where those would be 64 CTAs at most (N = 9: two A_P iterations and rho 5.57 -> 5.09 ms; at
+// N = 10, 256 CTAs, the small tiles are 7 % slower) and for FP64.
+template <class R, int G>
+cudaError_t tile_pass(int d, const JacobiPass& p, const cx_t<R>* A, cx_t<R>* Ao, const cx_t<R>* Vi, cx_t<R>* Vo,
+                      cx_t<R>* phi, cx_t<R>* ucos, cudaStream_t s) {
+  if (sizeof(R) == 4 && d > 512) return tile_pass_sized<R, G, sizeof(R) == 4 ? 64 : 32>(d, p, A, Ao, Vi, Vo, phi, ucos, s);
+  return tile_pass_sized<R, G, 32>(d, p, A, Ao, Vi, Vo, phi, ucos, s);
 }
 
 // One sweep: every pass of the schedule, ping-ponging (Ain, Aout) and (Vin, Vout).  Passes over cosets of 8

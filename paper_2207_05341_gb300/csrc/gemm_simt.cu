@@ -1,13 +1,14 @@
 // Complex d x d products on the CUDA cores (FP64, and FP32 where gemm_tc_fp32.cu does not run them):
 //   X = T T   (Sec. 3.2 eq. unified_DP, Hermitian: only tiles I >= J are computed)
 //   Y = G T   (backward of X = T T)
-// Row-major complex operands.  Classic register-blocked tiling: a CTA computes a
-// BM x BN tile, each thread a TM x TN block; the next K slice is prefetched into
-// registers while the current one is multiplied.  Shared-memory layout: A is
-// stored transposed with rows of BM + 4 entries, so that the stores of a warp
-// (8 k by 4 m) fall in distinct bank groups; a thread's TN columns of B are
-// 16-byte chunks (CW complex each) spaced by the chunks of the other threads of
-// its row, so that the 16 threads of a row read consecutive chunks.
+// Row-major complex operands.
+//
+// FP32 (k_cgemm): packed FMAs and 16-byte shared loads only in the inner loop: A is staged as (x, x, -y, y) and B
+// as (x, y, y, x), the operand pairs of the two FMAs of a complex product (packing them in registers cost more than
+// the shorter loads saved: 63 against 54 us at d = 512), and a thread's 4 x 4 entries take 32 FMAs from 8 loads.
+// What bounds it below d = 1024 is latency, two warps to a tile and one or two tiles to an SM (8 x 4 entries a
+// thread, half the warps: 101 us).  The next K slice is loaded into registers meanwhile.  Every entry is the sum
+// over k in order, re: a.x b.x then -a.y b.y, im: a.x b.y then a.y b.x, whatever the tile.
 //
 // FP64 has its own kernel (k_cgemm_f64): this part does 2 FP64 FMAs per clock and SM, a fortieth of its FP32
 // rate, so what counts is that every SM gets the same share of them, not the operand traffic.
@@ -17,12 +18,80 @@
 
 namespace qst {
 
-template <class R, int BM, int BN, int BK, int TM, int TN>
-__global__ void __launch_bounds__((BM / TM) * (BN / TN)) k_cgemm(int d, const cx_t<R>* __restrict__ A,
-                                                                 const cx_t<R>* __restrict__ B,
-                                                                 cx_t<R>* __restrict__ C, int lower,
-                                                                 const void* const* tab) {
-  using V = cx_t<R>;
+// BM x BM tile by (BM / 4)^2 threads: thread (ty, tx) the rows ty + BM / 4 i and columns tx + BM / 4 j.
+template <int BM, int BK>
+__global__ void __launch_bounds__((BM / 4) * (BM / 4)) k_cgemm(int d, const float2* __restrict__ A,
+                                                               const float2* __restrict__ B, float2* __restrict__ C,
+                                                               int lower, const void* const* tab) {
+  rebind(tab, A, B, C);
+  constexpr int TX = BM / 4, NT = TX * TX, L = BM * BK / NT;
+  __shared__ float4 As[2][BK][BM + 1];
+  __shared__ float4 Bs[2][BK][BM];
+  int I, J;
+  if (lower) tri_decode(blockIdx.x, I, J);
+  else { I = blockIdx.y; J = blockIdx.x; }
+  const int m0 = I * BM, n0 = J * BM, tid = threadIdx.x, tx = tid % TX, ty = tid / TX;
+  float2 ra[L], rb[L];
+  auto gload = [&](int k0) {
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      const int e = tid + l * NT;
+      ra[l] = A[(long long)(m0 + e / BK) * d + k0 + e % BK];
+      rb[l] = B[(long long)(k0 + e / BM) * d + n0 + e % BM];
+    }
+  };
+  auto sstore = [&](int buf) {
+#pragma unroll
+    for (int l = 0; l < L; ++l) {
+      const int e = tid + l * NT;
+      As[buf][e % BK][e / BK] = make_float4(ra[l].x, ra[l].x, -ra[l].y, ra[l].y);
+      Bs[buf][e / BM][e % BM] = make_float4(rb[l].x, rb[l].y, rb[l].y, rb[l].x);
+    }
+  };
+  float2 acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  const int nk = d / BK;
+  gload(0);
+  sstore(0);
+  __syncthreads();
+  for (int kt = 0; kt < nk; ++kt) {
+    const int buf = kt & 1;
+    if (kt + 1 < nk) gload((kt + 1) * BK);
+#pragma unroll
+    for (int k = 0; k < BK; ++k) {
+      float4 a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = As[buf][k][ty + TX * i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = Bs[buf][k][tx + TX * j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          acc[i][j] = __ffma2_rn(make_float2(a[i].z, a[i].w), make_float2(b[j].z, b[j].w),
+                                 __ffma2_rn(make_float2(a[i].x, a[i].y), make_float2(b[j].x, b[j].y), acc[i][j]));
+    }
+    if (kt + 1 < nk) {
+      sstore(buf ^ 1);
+      __syncthreads();
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) C[(long long)(m0 + ty + TX * i) * d + n0 + tx + TX * j] = acc[i][j];
+}
+
+// d >= 2048, where tiles abound: 128 x 128 tiles, 8 x 8 entries a thread (half the shared loads per FMA; X = T T at
+// d = 2048 in 914 us against 1035 with k_cgemm's 64 x 64 tiles, Y = G T in 1778 against 1838).  Same order of sums.
+__global__ void __launch_bounds__(256) k_cgemm_large(int d, const float2* __restrict__ A, const float2* __restrict__ B,
+                                                     float2* __restrict__ C, int lower, const void* const* tab) {
+  using V = float2;
+  using R = float;
+  constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
   rebind(tab, A, B, C);
   constexpr int NTX = BN / TN, NTY = BM / TM, NT = NTX * NTY;
   constexpr int LA = BM * BK / NT, LB = BK * BN / NT;
@@ -213,25 +282,32 @@ __global__ void k_cgemm_small(int d, const cx_t<R>* A, const cx_t<R>* B, cx_t<R>
   }
 }
 
-template <class R, int BM, int BN, int BK, int TM, int TN>
-static cudaError_t run_tiled(int d, const cx_t<R>* A, const cx_t<R>* B, cx_t<R>* C, bool lower, cudaStream_t s) {
-  constexpr int NT = (BM / TM) * (BN / TN);
+template <int BM, int BK>
+static cudaError_t run_tiled(int d, const float2* A, const float2* B, float2* C, bool lower, cudaStream_t s) {
+  constexpr int NT = (BM / 4) * (BM / 4);
   const int nt = d / BM;
   BatchArgs ba;
   if (batch_take(ba, {A, B, C})) return cudaSuccess;
-  if (lower) {
-    k_cgemm<R, BM, BN, BK, TM, TN><<<dim3((unsigned)(nt * (nt + 1) / 2), 1, ba.nz), NT, 0, s>>>(d, A, B, C, 1, ba.tab);
-  } else {
-    k_cgemm<R, BM, BN, BK, TM, TN><<<dim3(d / BN, d / BM, ba.nz), NT, 0, s>>>(d, A, B, C, 0, ba.tab);
-  }
+  const dim3 grid = lower ? dim3((unsigned)(nt * (nt + 1) / 2), 1, ba.nz) : dim3(nt, nt, ba.nz);
+  k_cgemm<BM, BK><<<grid, NT, 0, s>>>(d, A, B, C, lower ? 1 : 0, ba.tab);
   return cudaGetLastError();
 }
 
+// 64 x 64 tiles at d = 1024 (136 and 256 of them on 152 SMs); 32 x 32 tiles of two warps below, where 64-wide ones
+// would be 64 CTAs at most (d = 512: 54 us, 231 with 128 x 128 tiles).  A lower result covers the diagonal tiles
+// whole; its readers take entries on or below the diagonal only.
 template <>
 cudaError_t cgemm_simt<float>(int d, const float2* A, const float2* B, float2* C, bool lower, cudaStream_t s) {
-  if (d >= 128) return run_tiled<float, 128, 128, 8, 8, 8>(d, A, B, C, lower, s);
-  if (d == 64) return run_tiled<float, 64, 64, 8, 4, 4>(d, A, B, C, lower, s);
-  if (d == 32) return run_tiled<float, 32, 32, 8, 2, 2>(d, A, B, C, lower, s);
+  if (d >= 2048) {
+    const int nt = d / 128;
+    BatchArgs ba;
+    if (batch_take(ba, {A, B, C})) return cudaSuccess;
+    k_cgemm_large<<<lower ? dim3((unsigned)(nt * (nt + 1) / 2), 1, ba.nz) : dim3(nt, nt, ba.nz), 256, 0, s>>>(
+        d, A, B, C, lower ? 1 : 0, ba.tab);
+    return cudaGetLastError();
+  }
+  if (d == 1024) return run_tiled<64, 8>(d, A, B, C, lower, s);
+  if (d >= 32) return run_tiled<32, 16>(d, A, B, C, lower, s);
   k_cgemm_small<float><<<1, 256, 0, s>>>(d, A, B, C, lower ? 1 : 0);
   return cudaGetLastError();
 }
