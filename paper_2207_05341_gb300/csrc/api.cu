@@ -159,6 +159,7 @@ struct qst_ctx {
   size_t P = 0;           // parameters: qst_theta_size_net(N, network)
   bool cnn = false;       // the App. A CNN head instead of the 3-layer FNN
   unsigned long long* samp = nullptr;  // scratch of qst_sample_counts, allocated on first use
+  int* guide = nullptr;                // its guide table, where the budget has room for one
   long long oa_refinements = 0;  // tensor-core refinements taken (QST_MIXED A_P), Jacobi fallbacks
   long long oa_fallbacks = 0;
   double oa_last[2] = {0.0, 0.0};  // max |E| and the unresolved coupling of the latest refinement
@@ -242,6 +243,12 @@ template <class T> cudaError_t dalloc(qst_ctx* c, T** p, size_t count) {
   c->allocs.push_back(q);
   *p = reinterpret_cast<T*>(q);
   return cudaSuccess;
+}
+
+// What a context may still allocate on first use: the sampler's and the sampled fidelity's running sums, the state
+// fidelity's eigenvalue workspace and scratch.
+size_t lazy_scratch_bytes(const Dims& D) {
+  return 8 * (2 * (size_t)D.n + (size_t)D.n / 512) + 40 * (size_t)D.d * D.d + 512 * (size_t)D.d + 65536;
 }
 
 // An allocation the context can do without: skipped where it fails, or where it would leave less of the
@@ -362,7 +369,7 @@ template <class R> qst_status alloc_work(qst_ctx* c) {
   }
   // FP32 products on tensor cores where their operand planes fit (else on the CUDA cores)
   if (c->prec == QST_FP32 && c->opt.mapping != QST_MAP_ABS_P && tc32_ok(D.d)) {
-    const size_t later = 8 * (2 * (size_t)D.n + (size_t)D.n / 512) + 24 * nn + 512 * (size_t)D.d + 65536;
+    const size_t later = lazy_scratch_bytes(D);
     unsigned short *p9 = nullptr, *p6 = nullptr;
     dalloc_optional(c, &p9, 9 * nn, 12 * nn + later);
     if (p9) dalloc_optional(c, &p6, 6 * nn, later);
@@ -396,6 +403,7 @@ template <class R> qst_status check_f_begin(qst_ctx* c, const void* fdev) {
   QST_CU(net_check_f<R>(c->D.n, (const R*)fdev, w->partials, w->counters + CNT_CHECK, w->scal + kCheckF, c->stream));
   QST_CU(cudaMemcpyAsync(c->h_scal + kCheckF, w->scal + kCheckF, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
   QST_CU(cudaEventRecord(c->ev_check, c->stream));
+  c->launches += 1;
   return QST_OK;
 }
 qst_status check_f_end(qst_ctx* c) {
@@ -1531,7 +1539,10 @@ qst_status qst_sample_counts(qst_ctx* c, const double* P, long long shots, unsig
   if (!c || !P || !counts || shots < 0) return QST_E_INVAL;
   if (!is_device_ptr(P) || !is_device_ptr(counts) || (f && !is_device_ptr(f))) return QST_E_INVAL;
   const long long n = c->D.n;
-  if (!c->samp) QST_CU(dalloc(c, &c->samp, (size_t)sampler_scratch_words(n)));
+  if (!c->samp) {
+    QST_CU(dalloc(c, &c->samp, (size_t)sampler_scratch_words(n)));
+    dalloc_optional(c, &c->guide, (size_t)(n / 4 + 16), lazy_scratch_bytes(c->D));  // draws do without it
+  }
   unsigned int* flags = c->prec == QST_FP64 ? W<double>(c)->flags : W<float>(c)->flags;
   QST_CU(cudaMemsetAsync(flags + 2, 0, sizeof(unsigned int), c->stream));
   QST_CU(multinomial_prepare(n, P, c->samp, counts, flags + 2, c->stream));
@@ -1542,8 +1553,9 @@ qst_status qst_sample_counts(qst_ctx* c, const double* P, long long shots, unsig
   QST_CU(cudaStreamSynchronize(c->stream));
   c->launches += 3;
   if (c->h_flags[2] != 0u || W == 0ull) return QST_E_INPUT;
-  QST_CU(multinomial_draw(n, shots, seed, c->samp, counts, c->stream));
-  c->launches += shots > 0 ? 1 : 0;
+  int kernels = 0;
+  QST_CU(multinomial_draw(n, shots, seed, W, c->samp, c->guide, counts, &kernels, c->stream));
+  c->launches += kernels;
   if (f && shots > 0) {
     cudaError_t e = c->prec == QST_FP64 ? counts_to_frequencies<double>(n, counts, shots, (double*)f, c->stream)
                                         : counts_to_frequencies<float>(n, counts, shots, (float*)f, c->stream);

@@ -448,8 +448,10 @@ template <class R> cudaError_t make_test_state(int N, int kind, double w, cx_t<R
 long long sampler_scratch_words(long long n);
 cudaError_t multinomial_prepare(long long n, const double* P, unsigned long long* scratch, long long* counts,
                                 unsigned int* bad, cudaStream_t s);
-cudaError_t multinomial_draw(long long n, long long shots, unsigned long long seed, const unsigned long long* scratch,
-                             long long* counts, cudaStream_t s);
+// W: the total weight; guide: scratch of n / 4 + 1 ints, or NULL; *kernels: the launches made.
+cudaError_t multinomial_draw(long long n, long long shots, unsigned long long seed, unsigned long long W,
+                             const unsigned long long* scratch, int* guide, long long* counts, int* kernels,
+                             cudaStream_t s);
 template <class R> cudaError_t counts_to_frequencies(long long n, const long long* counts, long long shots, R* f,
                                                      cudaStream_t s);
 

@@ -52,44 +52,86 @@ __global__ void __launch_bounds__(256) k_test_state(cx_t<R>* __restrict__ rho, i
   }
 }
 
-// Integer weights and a block-local inclusive scan; block totals to tops.  A bad probability
-// (not finite, or above 1) raises *bad.
-__global__ void __launch_bounds__(256) k_weights_scan(const double* __restrict__ P, long long n,
-                                                       unsigned long long* __restrict__ C,
-                                                       unsigned long long* __restrict__ tops, unsigned int* bad) {
+// floor(max(p, 0) 2^52) from the bits of p (FP64 arithmetic is two operations per clock and SM here); a bad
+// probability (not finite, or above 1) raises *bad.
+__device__ __forceinline__ unsigned long long weight_of(double p, unsigned int* bad) {
+  const unsigned long long b = (unsigned long long)__double_as_longlong(p), mag = b & 0x7FFFFFFFFFFFFFFFull;
+  if (mag >= 0x7FF0000000000000ull || (b == mag && mag > 0x3FF0000000000000ull)) {
+    atomicOr(bad, 1u);
+    return 0;
+  }
+  if (b != mag) return 0;  // negative (or -0)
+  const int sh = 1023 - (int)(mag >> 52);  // p = m 2^(-52 - sh), m in [2^52, 2^53): the weight is m >> sh
+  return sh > 52 ? 0 : ((mag & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull) >> sh;
+}
+
+// The weights of a block's kBlockElems outcomes, summed (SCAN false: their total to tops[block]) or as running
+// sums on top of tops[block] (SCAN true: C, and counts cleared).  Two passes over P instead of a pass over P and
+// one over C: nothing is written before it is final (10 and 16 us at N = 11, 46 and 14 before).
+template <bool SCAN>
+__global__ void __launch_bounds__(256) k_weights(const double* __restrict__ P, long long n,
+                                                  unsigned long long* __restrict__ C,
+                                                  unsigned long long* __restrict__ tops,
+                                                  long long* __restrict__ counts, unsigned int* bad) {
   __shared__ unsigned long long wsum[8];
-  const long long base = (long long)blockIdx.x * kBlockElems + (long long)threadIdx.x * kPer;
-  unsigned long long v[kPer];
-  unsigned long long run = 0;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const long long i = base + k;
-    unsigned long long wk = 0;
-    if (i < n) {
-      const double p = P[i];
-      if (!(p <= 1.0) || !isfinite(p)) atomicOr(bad, 1u);
-      else if (p > 0.0) wk = (unsigned long long)(p * 4503599627370496.0);  // floor(p 2^52)
-    }
-    run += wk;
-    v[k] = run;
-  }
+  // thread t takes the pairs t, t + 256, ... of the block: whole lines per warp and load
+  const long long base = (long long)blockIdx.x * kBlockElems;
+  const bool vec = ((reinterpret_cast<uintptr_t>(P) | reinterpret_cast<uintptr_t>(SCAN ? counts : nullptr)) & 15u) == 0 &&
+                   base + kBlockElems <= n;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  unsigned long long x = run;
+  unsigned long long before = SCAN ? tops[blockIdx.x] : 0;
+  unsigned long long total = 0;
+  double2 pv[kPer / 2];
 #pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
-    if (lane >= o) x += y;
+  for (int k = 0; k < kPer / 2; ++k) {
+    const long long i = base + 2 * (threadIdx.x + 256 * k);
+    if (vec) pv[k] = *reinterpret_cast<const double2*>(P + i);
+    else pv[k] = make_double2(i < n ? P[i] : 0.0, i + 1 < n ? P[i + 1] : 0.0);
   }
-  if (lane == 31) wsum[warp] = x;
-  __syncthreads();
-  unsigned long long off = x - run;
-  for (int w = 0; w < warp; ++w) off += wsum[w];
 #pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const long long i = base + k;
-    if (i < n) C[i] = v[k] + off;
+  for (int k = 0; k < kPer / 2; ++k) {
+    const unsigned long long w0 = weight_of(pv[k].x, bad), w1 = weight_of(pv[k].y, bad);
+    if (!SCAN) {
+      total += w0 + w1;
+      continue;
+    }
+    unsigned long long x = w0 + w1;  // inclusive scan of the pairs over the block
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    __syncthreads();  // the slice before has read wsum
+    if (lane == 31) wsum[warp] = x;
+    __syncthreads();
+    unsigned long long off = before, all = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      off += w < warp ? wsum[w] : 0;
+      all += wsum[w];
+    }
+    before += all;
+    const long long i = base + 2 * (threadIdx.x + 256 * k);
+    const unsigned long long c1 = off + x, c0 = c1 - w1;
+    if (vec) {
+      *reinterpret_cast<ulonglong2*>(C + i) = make_ulonglong2(c0, c1);
+      *reinterpret_cast<longlong2*>(counts + i) = make_longlong2(0, 0);
+    } else {
+      if (i < n) { C[i] = c0; counts[i] = 0; }
+      if (i + 1 < n) { C[i + 1] = c1; counts[i + 1] = 0; }
+    }
   }
-  if (threadIdx.x == 255) tops[blockIdx.x] = off + run;
+  if (!SCAN) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
+    if (lane == 0) wsum[warp] = total;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned long long t = 0;
+      for (int w = 0; w < 8; ++w) t += wsum[w];
+      tops[blockIdx.x] = t;
+    }
+  }
 }
 
 __global__ void __launch_bounds__(1024) k_tops_scan(unsigned long long* tops, int nb) {
@@ -116,37 +158,55 @@ __global__ void __launch_bounds__(1024) k_tops_scan(unsigned long long* tops, in
   }
 }
 
-__global__ void __launch_bounds__(256) k_add_tops(unsigned long long* __restrict__ C, long long n,
-                                                   const unsigned long long* __restrict__ tops,
-                                                   long long* __restrict__ counts) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    C[i] += tops[i / kBlockElems];
-    counts[i] = 0;
+// smallest k in [lo, hi] with C[k] > t (C[hi] > t, or hi = n - 1)
+__device__ __forceinline__ long long first_above(const unsigned long long* __restrict__ C, unsigned long long t,
+                                                 long long lo, long long hi) {
+  while (lo < hi) {
+    const long long m = (lo + hi) >> 1;
+    if (C[m] > t) hi = m;
+    else lo = m + 1;
   }
+  return lo;
 }
 
+// start[b] = the outcome of the draw t = b 2^sh, b = 0 .. M: a draw t then lies between start[t >> sh] and the entry
+// after it.  Neighbouring buckets search neighbouring places, so this costs far less than as many draws.
+__global__ void __launch_bounds__(256) k_guide(const unsigned long long* __restrict__ C, long long n, int M, int sh,
+                                                int* __restrict__ start) {
+  for (int b = blockIdx.x * blockDim.x + threadIdx.x; b <= M; b += gridDim.x * blockDim.x)
+    start[b] = (int)first_above(C, (unsigned long long)b << sh, 0, n - 1);
+}
+
+// One draw: a bucket of the guide table and, within it, a search over the few outcomes that share it (about four at
+// n = 4 M; without the table every draw was 22 dependent loads over 33 MB, 600 us for 10^7 shots at N = 11; now 148 us, the
+// table 29, bound by the random sectors of C and the atomics on counts).
 __global__ void __launch_bounds__(256) k_draw(const unsigned long long* __restrict__ C, long long n, long long shots,
-                                               unsigned long long seed, long long* __restrict__ counts) {
+                                               unsigned long long seed, const int* __restrict__ start, int sh,
+                                               long long* __restrict__ counts) {
   const unsigned long long W = C[n - 1];
   for (long long s = (long long)blockIdx.x * blockDim.x + threadIdx.x; s < shots; s += (long long)gridDim.x * blockDim.x) {
     const unsigned long long a = splitmix64(seed, (unsigned long long)s) >> 11;  // < 2^53
     const unsigned long long hi = __umul64hi(a, W), lo = a * W;
     const unsigned long long t = (hi << 11) | (lo >> 53);                         // floor(a W / 2^53) < W
-    long long l = 0, h = n - 1;
-    while (l < h) {
-      const long long m = (l + h) >> 1;
-      if (C[m] > t) h = m;
-      else l = m + 1;
-    }
+    const int b = (int)(t >> sh);
+    const long long l = start ? first_above(C, t, start[b], start[b + 1]) : first_above(C, t, 0, n - 1);
     atomicAdd(reinterpret_cast<unsigned long long*>(counts + l), 1ull);
   }
 }
 
+// f = counts / shots, correctly rounded as on the host.  Nearly all counts are small and share few quotients, so a
+// block makes those once (one FP64 division per entry was 169 us at N = 11; this is 20).
+constexpr int kQuot = 256;
 template <class R>
 __global__ void __launch_bounds__(256) k_freq(const long long* __restrict__ counts, long long n, long long shots,
                                                R* __restrict__ f) {
-  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    f[i] = (R)((double)counts[i] / (double)shots);  // correctly rounded, as counts / shots on the host
+  __shared__ R quot[kQuot];
+  for (int c = threadIdx.x; c < kQuot; c += blockDim.x) quot[c] = (R)((double)c / (double)shots);
+  __syncthreads();
+  for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long c = counts[i];
+    f[i] = c >= 0 && c < kQuot ? quot[c] : (R)((double)c / (double)shots);
+  }
 }
 
 int grid_of(long long work, int sms_mult = 8) {
@@ -174,21 +234,33 @@ cudaError_t multinomial_prepare(long long n, const double* P, unsigned long long
   const int nb = (int)((n + kBlockElems - 1) / kBlockElems);
   unsigned long long* C = scratch;
   unsigned long long* tops = scratch + n;
-  k_weights_scan<<<nb, 256, 0, s>>>(P, n, C, tops, bad);
+  k_weights<false><<<nb, 256, 0, s>>>(P, n, C, tops, counts, bad);
   k_tops_scan<<<1, 1024, 0, s>>>(tops, nb);
-  k_add_tops<<<grid_of(n), 256, 0, s>>>(C, n, tops, counts);
+  k_weights<true><<<nb, 256, 0, s>>>(P, n, C, tops, counts, bad);
   return cudaGetLastError();
 }
 
-cudaError_t multinomial_draw(long long n, long long shots, unsigned long long seed, const unsigned long long* scratch,
-                             long long* counts, cudaStream_t s) {
-  if (shots > 0) k_draw<<<grid_of(shots), 256, 0, s>>>(scratch, n, shots, seed, counts);
+// The guide table has a bucket for every four outcomes, or every four shots where those are fewer (building it is then
+// a fraction of the draws); none below 4096 shots.
+cudaError_t multinomial_draw(long long n, long long shots, unsigned long long seed, unsigned long long W,
+                             const unsigned long long* scratch, int* guide, long long* counts, int* kernels,
+                             cudaStream_t s) {
+  *kernels = 0;
+  if (shots <= 0) return cudaSuccess;
+  int lm = 0, bits = 64;
+  while (lm < 30 && (1LL << (lm + 1)) <= shots / 4 && (1LL << (lm + 1)) <= n / 4) ++lm;
+  while (bits > 0 && !((W - 1) >> (bits - 1) & 1ull)) --bits;  // (W - 1) >> (bits - lm) < 2^lm
+  const int M = 1 << lm, sh = bits > lm ? bits - lm : 0;
+  const bool table = guide && shots >= 4096 && lm >= 4 && sh < 64;
+  if (table) k_guide<<<grid_of(M + 1), 256, 0, s>>>(scratch, n, M, sh, guide);
+  k_draw<<<grid_of(shots), 256, 0, s>>>(scratch, n, shots, seed, table ? guide : nullptr, table ? sh : 0, counts);
+  *kernels = table ? 2 : 1;
   return cudaGetLastError();
 }
 
 template <class R> cudaError_t counts_to_frequencies(long long n, const long long* counts, long long shots, R* f,
                                                      cudaStream_t s) {
-  k_freq<R><<<grid_of(n), 256, 0, s>>>(counts, n, shots, f);
+  k_freq<R><<<grid_of(n, 4), 256, 0, s>>>(counts, n, shots, f);
   return cudaGetLastError();
 }
 
