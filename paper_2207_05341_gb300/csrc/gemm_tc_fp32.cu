@@ -19,14 +19,17 @@
 // A complex product is one real product with the K axis doubled, A' = [A_re | A_im], and the N axis doubled:
 // with the planes P_re, P_im, P_nim = -P_im of B^dag, Re C uses [P_re | P_im] and Im C uses [P_nim | P_re].
 //
-// Kernel: one CTA per 128 x BN complex tile (N = 2 BN real columns), 10 warps.  Warp 8 streams K blocks with
-// TMA into a ring (A: 3 terms x 128 rows, B: 3 terms x 2 BN rows of 64 bytes, 64-byte swizzle), warp 9 issues
+// Kernel: one CTA, or below d = 2048 a cluster of ks CTAs that share the K blocks, per 128 x 128 complex tile
+// (N = 256 real columns), 10 warps.  Warp 8 streams K blocks with TMA into a ring (A: 3 terms x 128 rows, B:
+// 3 terms x 256 rows of 64 bytes, 64-byte swizzle: 47 bytes per clock; a 128 x 64 tile needs 62, at the limit of
+// what an SM takes from L2, and was twice as slow per product), warp 9 issues
 // the block's 12 MMAs into one of two TMEM accumulators, and warps 0-7 drain the other one into registers
 // (TMEM to FP32 adds), so the promotion runs beside the MMAs: 12 MMAs of N = 256 take about 1540 cycles, the
 // drain of 128 x 256 sums about 500.  Bound by the tensor pipe: at N = 11 X = T T takes 129 us and Y = G T 253 us
-// (206 and 412 GFLOP of BF16 products, 1.6 PFLOP/s; 914 and 1778 us on the CUDA cores), at N = 9 28 and 28 us
-// (231 and 232).  Every mbarrier wait is bounded; on timeout the kernel raises *err,
+// (206 and 412 GFLOP of BF16 products, 1.6 PFLOP/s; 914 and 1778 us on the CUDA cores), at N = 9 27 and 26 us
+// (231 and 232), there mostly fixed costs.  Every mbarrier wait is bounded; on timeout the kernel raises *err,
 // drains its copies, frees TMEM and returns.
+#include <cooperative_groups.h>
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -43,18 +46,18 @@ constexpr int kRow = kBK * 2;
 constexpr int kEpiWarps = 8;
 constexpr int kThreads32 = (kEpiWarps + 2) * 32;
 
-template <int BN> struct Cfg32 {
-  static constexpr int kA = kBM * kRow;       // bytes of one term of A in a stage
-  static constexpr int kB = BN * kRow;        // bytes of one term of one half of B
-  static constexpr int kStage = 3 * kA + 6 * kB;
-  static constexpr int kStages = BN == 128 ? 3 : 4;
-  static constexpr int kSmem = kStages * kStage + 1024 + 256;
-  static constexpr int kTmem = 4 * BN;        // two accumulators of 2 BN columns
-};
+constexpr int kBN = 128;                      // complex columns of a tile
+constexpr int kA = kBM * kRow;                // bytes of one term of A in a stage
+constexpr int kB = kBN * kRow;                // bytes of one term of one half of B
+constexpr int kStage = 3 * kA + 6 * kB;
+constexpr int kStages = 3;
+constexpr int kSmem = kStages * kStage + 1024 + 256;
+constexpr int kTmem = 4 * kBN;                // two accumulators of 256 columns
+static_assert(kBM * kBN * 8 <= kStages * kStage, "a partial tile fits in the ring");
 
 struct Maps32 {
   CUtensorMap a;  // 6 planes: re h, m, l; im h, m, l (box 32 x 128 x 3)
-  CUtensorMap b;  // 9 planes: re, im, -im, each h, m, l (box 32 x BN x 1)
+  CUtensorMap b;  // 9 planes: re, im, -im, each h, m, l (box 32 x 128 x 1)
 };
 
 __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
@@ -80,48 +83,45 @@ __device__ __forceinline__ uint64_t desc64(uint32_t addr) {
   return d;
 }
 
-// kind::f16, FP32 accumulators, BF16 operands, both K-major, M = 128, N = 2 BN
-template <int BN> __device__ constexpr uint32_t idesc32() {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * BN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
-}
+// kind::f16, FP32 accumulators, BF16 operands, both K-major, M = 128, N = 256
+constexpr uint32_t kIdesc32 = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(2 * kBN >> 3) << 17) | ((uint32_t)(kBM >> 4) << 24);
 
 // krange: 0 all of K; 1 only k >= the tile's first row (A and B^dag upper triangular, tiles I >= J);
 // 2 only k <= the tile's last row (A lower triangular).  What is left out is multiplied by zeros.
+// ks: CTAs of a cluster that share a tile (rank r takes the r-th part of the K blocks); their partial tiles meet in
+// distributed shared memory, rank r summing its rows over the ranks in order.
 // tab: a batched launch (grid z = tomography); row z holds the tensor maps' device copy, C, sA, sB, err, clear.
-template <int BN>
 __global__ void __launch_bounds__(kThreads32, 1)
-    k_tc_cgemm32(const __grid_constant__ Maps32 maps, float2* __restrict__ C, int d, int lower, int krange,
+    k_tc_cgemm32(const __grid_constant__ Maps32 maps, float2* __restrict__ C, int d, int lower, int krange, int ks,
                  const double* sA, const double* sB, unsigned int* err, unsigned int* clear, int no_loads,
                  const void* const* tab) {
-  using K = Cfg32<BN>;
   const Maps32* mp = &maps;
   rebind(tab, mp, C, sA, sB, err, clear);
   grid_dep_wait();
   after_wait(mp, C, sA, sB, err, clear);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + K::kStages * K::kStage);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
   const uint32_t full0 = smem_u32(bars);
-  const uint32_t empty0 = smem_u32(bars + K::kStages);
-  const uint32_t accf0 = smem_u32(bars + 2 * K::kStages);      // accumulator b complete
-  const uint32_t acce0 = smem_u32(bars + 2 * K::kStages + 2);  // accumulator b drained
-  const uint32_t done = smem_u32(bars + 2 * K::kStages + 4);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * K::kStages + 5);
+  const uint32_t empty0 = smem_u32(bars + kStages);
+  const uint32_t accf0 = smem_u32(bars + 2 * kStages);      // accumulator b complete
+  const uint32_t acce0 = smem_u32(bars + 2 * kStages + 2);  // accumulator b drained
+  const uint32_t done = smem_u32(bars + 2 * kStages + 4);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
 
-  int I, J;  // the tile: rows 128 I .., columns BN J ..
+  int I, J;  // the tile: rows 128 I .., columns 128 J ..
+  const int rank = (int)blockIdx.x % ks;
   if (lower) {
-    constexpr int kSub = kBM / BN;
-    tri_decode(blockIdx.x / kSub, I, J);
-    J = J * kSub + (int)(blockIdx.x % kSub);
+    tri_decode(blockIdx.x / ks, I, J);
   } else {
     I = blockIdx.y;
-    J = blockIdx.x;
+    J = (int)blockIdx.x / ks;
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
   if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0u;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < K::kStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
     }
@@ -135,7 +135,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
   __syncwarp();
   if (warp == 0) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)),
-                 "r"(K::kTmem)
+                 "r"(kTmem)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
@@ -143,7 +143,8 @@ __global__ void __launch_bounds__(kThreads32, 1)
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
   const int kbeg = krange == 1 ? I * kBM : 0, kend = krange == 2 ? (I + 1) * kBM : d;
-  const int half = (kend - kbeg) / kBK, nkb = 2 * half;
+  const int half = (kend - kbeg) / kBK;                       // K blocks of the real part, and of the imaginary part
+  const int kb0 = 2 * half * rank / ks, nkb = 2 * half * (rank + 1) / ks - kb0;  // this CTA's
 
   if (warp == kEpiWarps) {
     if (lane == 0) {  // ---------------- TMA producer
@@ -153,28 +154,28 @@ __global__ void __launch_bounds__(kThreads32, 1)
       }
       int issued = 0;
       for (int kb = 0; kb < (no_loads ? 0 : nkb); ++kb) {
-        const int s = kb % K::kStages, it = kb / K::kStages;
-        if (kb >= K::kStages && !mbar_wait(empty0 + 8 * s, (uint32_t)((it - 1) & 1))) {
+        const int s = kb % kStages, it = kb / kStages;
+        if (kb >= kStages && !mbar_wait(empty0 + 8 * s, (uint32_t)((it - 1) & 1))) {
           atomicOr(err, 1u);
           break;
         }
         const uint32_t fb = full0 + 8 * s;
-        mbar_expect_tx(fb, K::kStage);
-        const int part = kb < half ? 0 : 1;
-        const int col = kbeg + (kb - part * half) * kBK;
-        const uint32_t base = smem_u32(smem + s * K::kStage), bb = base + 3 * K::kA;
+        mbar_expect_tx(fb, kStage);
+        const int part = kb0 + kb < half ? 0 : 1;
+        const int col = kbeg + (kb0 + kb - part * half) * kBK;
+        const uint32_t base = smem_u32(smem + s * kStage), bb = base + 3 * kA;
         tma_load_3d(base, &mp->a, col, I * kBM, 3 * part, fb);
         const int z1 = part == 0 ? 0 : 3, z2 = part == 0 ? 6 : 0;  // Re: re | im; Im: -im | re
 #pragma unroll
         for (int t = 0; t < 3; ++t) {
-          tma_load_3d(bb + (2 * t) * K::kB, &mp->b, col, J * BN, z1 + t, fb);
-          tma_load_3d(bb + (2 * t + 1) * K::kB, &mp->b, col, J * BN, z2 + t, fb);
+          tma_load_3d(bb + (2 * t) * kB, &mp->b, col, J * kBN, z1 + t, fb);
+          tma_load_3d(bb + (2 * t + 1) * kB, &mp->b, col, J * kBN, z2 + t, fb);
         }
         ++issued;
       }
       // every stage issued must have landed before the CTA may exit
-      for (int kb = (issued > K::kStages ? issued - K::kStages : 0); kb < issued; ++kb) {
-        if (!mbar_wait(full0 + 8 * (kb % K::kStages), (uint32_t)((kb / K::kStages) & 1))) {
+      for (int kb = (issued > kStages ? issued - kStages : 0); kb < issued; ++kb) {
+        if (!mbar_wait(full0 + 8 * (kb % kStages), (uint32_t)((kb / kStages) & 1))) {
           atomicOr(err, 1u);
           break;
         }
@@ -185,19 +186,19 @@ __global__ void __launch_bounds__(kThreads32, 1)
     if (lane == 0) {  // ---------------- MMA issuer
       bool ok = true;
       for (int kb = 0; kb < nkb; ++kb) {
-        const int s = kb % K::kStages, b = kb & 1;
-        if (!mbar_wait(full0 + 8 * s, (uint32_t)((kb / K::kStages) & 1))) { ok = false; break; }
+        const int s = kb % kStages, b = kb & 1;
+        if (!mbar_wait(full0 + 8 * s, (uint32_t)((kb / kStages) & 1))) { ok = false; break; }
         if (kb >= 2 && !mbar_wait(acce0 + 8 * b, (uint32_t)(((kb >> 1) - 1) & 1))) { ok = false; break; }
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t base = smem_u32(smem + s * K::kStage), bb = base + 3 * K::kA;
-        const uint32_t acc = tmem + (uint32_t)(b * 2 * BN);
+        const uint32_t base = smem_u32(smem + s * kStage), bb = base + 3 * kA;
+        const uint32_t acc = tmem + (uint32_t)(b * 2 * kBN);
         constexpr int ta[6] = {2, 0, 1, 1, 0, 0}, tb[6] = {0, 2, 1, 0, 1, 0};  // lh hl mm mh hm hh
 #pragma unroll
         for (int p = 0; p < 6; ++p) {
 #pragma unroll
           for (int kk = 0; kk < kBK / 16; ++kk)
-            mma_f16(acc, desc64(base + ta[p] * K::kA + kk * 32), desc64(bb + 2 * tb[p] * K::kB + kk * 32),
-                    idesc32<BN>(), p > 0 || kk > 0 ? 1u : 0u);
+            mma_f16(acc, desc64(base + ta[p] * kA + kk * 32), desc64(bb + 2 * tb[p] * kB + kk * 32),
+                    kIdesc32, p > 0 || kk > 0 ? 1u : 0u);
         }
         mma_commit(empty0 + 8 * s);
         mma_commit(accf0 + 8 * b);
@@ -208,7 +209,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
     __syncwarp();
   } else {
     // ---------------- promotion: warp w drains TMEM lanes 32 (w % 4) .. and half w / 4 of the columns
-    constexpr int CH = BN / 2;  // complex columns of this warp
+    constexpr int CH = kBN / 2;  // complex columns of this warp
     const int q = warp & 3, hf = warp >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(hf * CH);
     float re[CH], im[CH];
@@ -220,12 +221,12 @@ __global__ void __launch_bounds__(kThreads32, 1)
       ok = __all_sync(0xffffffffu, mbar_wait(accf0 + 8 * b, (uint32_t)((kb >> 1) & 1)));
       if (!ok) break;
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t src = lane_base + (uint32_t)(b * 2 * BN);
+      const uint32_t src = lane_base + (uint32_t)(b * 2 * kBN);
 #pragma unroll
       for (int c = 0; c < CH; c += 16) {
         uint32_t r[16], i[16];
         tmem_ld16(src + (uint32_t)c, r);
-        tmem_ld16(src + (uint32_t)(BN + c), i);
+        tmem_ld16(src + (uint32_t)(kBN + c), i);
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
         for (int u = 0; u < 16; ++u) {
@@ -237,11 +238,17 @@ __global__ void __launch_bounds__(kThreads32, 1)
       __syncwarp();
       if (lane == 0) mbar_arrive(acce0 + 8 * b);
     }
-    if (ok) {
+    if (ok && ks > 1) {  // the partial tile to shared memory (every operand has been used), 16-byte chunks swizzled
+      const int row = q * 32 + lane;
+      float4* part = reinterpret_cast<float4*>(smem) + row * (kBN / 2);
+#pragma unroll
+      for (int c = 0; c < CH; c += 2)
+        part[(hf * (CH / 2) + c / 2) ^ (row & (kBN / 2 - 1))] = make_float4(re[c], im[c], re[c + 1], im[c + 1]);
+    } else if (ok) {
       // C = acc / (sA sB), both powers of two; the smaller factor first (no overflow on the way)
       const float ua = (float)(1.0 / *sA), ub = (float)(1.0 / *sB);
       const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
-      float2* out = C + (long long)(I * kBM + q * 32 + lane) * d + (long long)J * BN + hf * CH;
+      float2* out = C + (long long)(I * kBM + q * 32 + lane) * d + (long long)J * kBN + hf * CH;
 #pragma unroll
       for (int c = 0; c < CH; c += 2)
         *reinterpret_cast<float4*>(out + c) = make_float4(re[c] * u1 * u2, im[c] * u1 * u2, re[c + 1] * u1 * u2,
@@ -250,11 +257,33 @@ __global__ void __launch_bounds__(kThreads32, 1)
       atomicOr(err, 1u);
     }
   }
+  if (ks > 1) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
+    __syncwarp();
+    cl.sync();
+    const float ua = (float)(1.0 / *sA), ub = (float)(1.0 / *sB);
+    const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
+    const int rows = kBM / ks;
+    constexpr int kChunks = kBN / 2;
+    for (int e = threadIdx.x; e < rows * kChunks; e += kThreads32) {
+      const int row = rank * rows + e / kChunks, ch = e % kChunks;
+      float4* at = reinterpret_cast<float4*>(smem) + row * kChunks + (ch ^ (row & (kChunks - 1)));
+      float4 v = *cl.map_shared_rank(at, 0);
+      for (int r = 1; r < ks; ++r) {
+        const float4 w = *cl.map_shared_rank(at, r);
+        v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+      }
+      *reinterpret_cast<float4*>(C + (long long)(I * kBM + row) * d + (long long)J * kBN + 2 * ch) =
+          make_float4(v.x * u1 * u2, v.y * u1 * u2, v.z * u1 * u2, v.w * u1 * u2);
+    }
+    cl.sync();  // no CTA leaves while its part may still be read
+  }
   if (warp == 0) mbar_wait(done, 0u);  // no MMA in flight when TMEM is freed
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (warp == 0) {
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(K::kTmem) : "memory");
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmem) : "memory");
   }
 }
 
@@ -449,23 +478,6 @@ bool planes_map(CUtensorMap* m, const void* base, int d, int planes, int rows, i
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int BN>
-cudaError_t launch32(int d, const void* Ap, const void* Bp, const double* sA, const double* sB, float2* C, bool lower,
-                     int krange, unsigned int* err, unsigned int* clear, cudaStream_t s) {
-  using K = Cfg32<BN>;
-  cudaError_t e = ensure_dynamic_smem((const void*)k_tc_cgemm32<BN>, K::kSmem);
-  if (e != cudaSuccess) return e;
-  Maps32 M;
-  if (!planes_map(&M.a, Ap, d, 6, kBM, 3) || !planes_map(&M.b, Bp, d, 9, BN, 1)) return cudaErrorInvalidValue;
-  BatchArgs ba;
-  if (batch_take(ba, {C, sA, sB, err, clear}, &M, sizeof(Maps32))) return cudaSuccess;
-  const int no_loads = inject_take(INJ_TC_LOADS) ? 1 : 0;
-  const int nt = d / kBM;
-  const dim3 grid = lower ? dim3((unsigned)(nt * (nt + 1) / 2 * (kBM / BN)), 1, ba.nz) : dim3(d / BN, nt, ba.nz);
-  return launch_dep(k_tc_cgemm32<BN>, grid, dim3(kThreads32), (size_t)K::kSmem, s, M, C, d, lower ? 1 : 0, krange, sA,
-                    sB, err, clear, no_loads, ba.tab);
-}
-
 }  // namespace
 
 bool tc32_ok(int d) { return d >= 128 && d % 128 == 0 && tc_available(); }
@@ -493,13 +505,37 @@ cudaError_t tc32_split(int d, const float2* A, void* P, int planes, bool keep_sc
                     partials, counter, flags, ba.tab);
 }
 
-// 128-wide tiles where they fill the GPU (136 or 256 of them on 152 SMs at d = 2048); half as wide below,
-// where the 128-wide grid (at most 64 tiles) would leave most SMs idle.
+// CTAs per tile: one from d = 2048 on (136 and 256 tiles on 152 SMs); below, K shared so that a single product
+// reaches more SMs (the order of the sums depends on d alone, so a batch has the bits of its members).
+static int k_split(int d) { return d >= 2048 ? 1 : d >= 512 ? 2 : 4; }
+
 cudaError_t tc32_product(int d, const void* Ap, const void* Bp, const double* sA, const double* sB, float2* C,
                          bool lower, int krange, unsigned int* err, unsigned int* clear, cudaStream_t s) {
   if (d < kBM || d % kBM) return cudaErrorInvalidValue;
-  if (d >= 2048) return launch32<128>(d, Ap, Bp, sA, sB, C, lower, krange, err, clear, s);
-  return launch32<64>(d, Ap, Bp, sA, sB, C, lower, krange, err, clear, s);
+  cudaError_t e = ensure_dynamic_smem((const void*)k_tc_cgemm32, kSmem);
+  if (e != cudaSuccess) return e;
+  Maps32 M;
+  if (!planes_map(&M.a, Ap, d, 6, kBM, 3) || !planes_map(&M.b, Bp, d, 9, kBN, 1)) return cudaErrorInvalidValue;
+  BatchArgs ba;
+  if (batch_take(ba, {C, sA, sB, err, clear}, &M, sizeof(Maps32))) return cudaSuccess;
+  const int no_loads = inject_take(INJ_TC_LOADS) ? 1 : 0;
+  const int nt = d / kBM, ks = k_split(d);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = lower ? dim3((unsigned)(nt * (nt + 1) / 2 * ks), 1, ba.nz) : dim3(nt * ks, nt, ba.nz);
+  cfg.blockDim = dim3(kThreads32);
+  cfg.dynamicSmemBytes = kSmem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)ks;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  return cudaLaunchKernelEx(&cfg, k_tc_cgemm32, M, C, d, lower ? 1 : 0, krange, ks, sA, sB, err, clear, no_loads,
+                            ba.tab);
 }
 
 }  // namespace qst
