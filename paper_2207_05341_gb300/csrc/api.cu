@@ -421,7 +421,8 @@ unsigned int* amax_slot(qst_ctx* c, int slot) {
 template <class R> struct Engine {
   using V = cx_t<R>;
 
-  // X = T T (lower tiles) from the hidden activation already in w->hid; Tr X -> scal[0]
+  // X = T T (lower tiles) from the hidden activation already in w->hid; Tr X -> scal[0] where the POVM map does not
+  // form it
   static qst_status forward_state(qst_ctx* c, const R* theta, bool own_params = true) {
     Work<R>* w = W<R>(c);
     const Dims& D = c->D;
@@ -542,8 +543,11 @@ template <class R> struct Engine {
     } else {
       QST_CU(cgemm_simt<R>(D.d, delta ? w->Y : w->T, w->T, w->X, true, c->stream));
     }
-    QST_CU(trace_X<R>(D, w->X, w->scal, c->stream));
-    c->launches += 2;
+    if (!fast_povm(c)) {  // (the fast POVM map's first pass forms the trace beside its tiles)
+      QST_CU(trace_X<R>(D, w->X, w->scal, c->stream));
+      c->launches += 1;
+    }
+    c->launches += 1;
     tmark(c, QST_PH_XFWD);
     return QST_OK;
   }
@@ -568,7 +572,7 @@ template <class R> struct Engine {
           }
           fl = w->fperm;
         }
-        QST_CU(povm_lo_fwd_fast(D, w->X, w->Wlo, c->plan, c->stream));
+        QST_CU(povm_lo_fwd_fast(D, w->X, w->Wlo, c->plan, w->scal, c->stream));
         tmark(c, QST_PH_POVM_LO);
         QST_CU(povm_hi_nll_fast(D, w->Wlo, fl, w->scal, w->Whi, w->partials, w->counters + CNT_NLL, w->flags,
                                 c->plan, backward, c->stream));
@@ -964,6 +968,8 @@ template <class R> struct Engine {
     bool done = false;
     if constexpr (std::is_same<R, float>::value) {
       if (fast_povm(c)) {
+        QST_CU(trace_X<R>(D, w->X, w->scal, c->stream));
+        c->launches += 1;
         QST_CU(povm_fwd_fast(D, w->X, w->Wlo, w->Whi, c->plan, c->stream));  // q, unnormalised, in Whi
         done = true;
       }
@@ -1084,6 +1090,10 @@ template <class R> struct Engine {
     }
     if ((st = forward_state(c, w->theta)) != QST_OK) return st;
     if (rho_out) {
+      if (fast_povm(c)) {
+        QST_CU(trace_X<R>(D, w->X, w->scal, c->stream));
+        c->launches += 1;
+      }
       QST_CU(hermitian_complete<R>(D, w->X, dst, w->scal, c->stream));
       c->launches += 1;
       if (!dev) {

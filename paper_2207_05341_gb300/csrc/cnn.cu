@@ -199,11 +199,11 @@ __global__ void __launch_bounds__(256) k_cnn_conv_tiles(const R* __restrict__ f,
   for (int a = 0; a < kRowsPer + 2; ++a)
 #pragma unroll
     for (int b = 0; b < kColsPer + 2; ++b) v[a][b] = tile[rg * kRowsPer + a][cx + b];
-  double fs = 0.0;
+  typename SumOf<R>::T fsum;
 #pragma unroll
   for (int rr = 0; rr < kRowsPer; ++rr)
 #pragma unroll
-    for (int cc = 0; cc < kColsPer; ++cc) fs += (double)v[rr + 1][cc + 1];
+    for (int cc = 0; cc < kColsPer; ++cc) fsum.add(v[rr + 1][cc + 1]);
 #pragma unroll 1
   for (int c = 0; c < kMaps; ++c) {
     R w[9];
@@ -241,7 +241,7 @@ __global__ void __launch_bounds__(256) k_cnn_conv_tiles(const R* __restrict__ f,
       ri[warp][c] = idx;
     }
   }
-  fs = warp_sum(fs);
+  const double fs = warp_sum(fsum.value());
   if (lane == 0) rf[warp] = fs;
   __syncthreads();
   if (threadIdx.x < kMaps) {

@@ -83,9 +83,11 @@ __host__ __device__ __forceinline__ uint32_t interleave_ij(uint32_t i, uint32_t 
 __host__ __device__ __forceinline__ uint32_t row_of(uint32_t a) { return compact_bits(a >> 1); }
 __host__ __device__ __forceinline__ uint32_t col_of(uint32_t a) { return compact_bits(a); }
 
-// Row index I of the t-th lower-triangular tile pair (I >= J), t = I(I+1)/2 + J.
+// Row index I of the t-th lower-triangular tile pair (I >= J), t = I(I+1)/2 + J.  (Every thread of a tile kernel
+// comes through here: an FP64 square root cost each 256-thread CTA about 1.6 us of the SM's FP64 pipe, and
+// k_symmetrize, with 2080 CTAs at N = 11, spent 17 us where 8.8 are left.)
 __device__ __forceinline__ void tri_decode(uint32_t t, int& I, int& J) {
-  int i = (int)((sqrt(8.0 * (double)t + 1.0) - 1.0) * 0.5);
+  int i = (int)((sqrtf(8.f * (float)t + 1.f) - 1.f) * 0.5f);  // FP32: put right below wherever it is off
   while ((uint32_t)((i + 1) * (i + 2) / 2) <= t) ++i;
   while ((uint32_t)(i * (i + 1) / 2) > t) --i;
   I = i;
@@ -134,6 +136,31 @@ __device__ __forceinline__ double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   return v;
 }
+
+// A sum kept as an FP32 pair s + e (Knuth's two-sum; a product's rounding error by FMA), so that a thread's terms
+// keep about 48 bits without the FP64 pipe (two operations per clock and SM).
+struct PairSum {
+  float s = 0.f, e = 0.f;
+  __device__ __forceinline__ void add(float v) {
+    const float t = __fadd_rn(s, v), b = __fsub_rn(t, s);
+    e = __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, b)), __fsub_rn(v, b)));
+    s = t;
+  }
+  __device__ __forceinline__ void add_product(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    e = __fadd_rn(e, __fmaf_rn(a, b, -p));
+    add(p);
+  }
+  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+};
+// The same in FP64 arithmetic for FP64 terms.
+struct WideSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <class R> struct SumOf { using T = PairSum; };
+template <> struct SumOf<double> { using T = WideSum; };
 
 // Sums of M values each over a warp: out(j, sum) is called once per j, by one lane.  Step by step a lane hands half
 // of the values it still carries to its partner, which hands over the other half, so M = 11 takes 16 FP64 adds

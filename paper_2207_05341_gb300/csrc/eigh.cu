@@ -664,7 +664,9 @@ __global__ void k_identity(cx_t<R>* V, int d) {
 }
 
 // Spectrum: lam_i = Re A_ii, s_i = |lambda_i|^P (|lambda| floored at eps max|lambda| for P <= 1),
-// s'_i = d s_i / d lambda_i (0 on the floor).  One block.
+// s'_i = d s_i / d lambda_i (0 on the floor).  Every block finds max |lambda|, and block b does the entries
+// kSpec b .. of s (two FP64 powers each, which one block took 25 us for at d = 512).
+constexpr int kSpec = 64;
 template <class R>
 __global__ void __launch_bounds__(1024) k_absp_spectrum(const cx_t<R>* __restrict__ A, R* lam, R* s, R* sp, int d,
                                                          double P, double eps) {
@@ -681,7 +683,8 @@ __global__ void __launch_bounds__(1024) k_absp_spectrum(const cx_t<R>* __restric
   }
   __syncthreads();
   const double floor_v = P <= 1.0 ? eps * (double)red[0] : 0.0;
-  for (int i = threadIdx.x; i < d; i += blockDim.x) {
+  const int i = (int)blockIdx.x * kSpec + (int)threadIdx.x;
+  if (threadIdx.x < kSpec && i < d) {
     const double li = (double)A[(long long)i * d + i].x;
     const double ai = fabs(li);
     const double ui = ai > floor_v ? ai : floor_v;
@@ -938,7 +941,7 @@ cudaError_t abs_p_forward(int d, const cx_t<R>* T, AbsPWork<R>& w, int sweeps, b
   }
   w.A = Ain;  // diagonalised
   w.Q = Vin;  // eigenvectors in columns (V0)
-  k_absp_spectrum<R><<<1, 1024, 0, s>>>(w.A, w.lam, w.s, w.sp, d, P, sizeof(R) == 4 ? 1e-7 : 1e-15);
+  k_absp_spectrum<R><<<(d + kSpec - 1) / kSpec, 256, 0, s>>>(w.A, w.lam, w.s, w.sp, d, P, sizeof(R) == 4 ? 1e-7 : 1e-15);
   k_scale_cols<R><<<blocks_for(nn), 256, 0, s>>>(w.Q, w.s, w.W, d);
   const int TS = d < 32 ? d : 32;
   k_conj_transpose<R><<<dim3(d / TS, d / TS), 256, 0, s>>>(w.Q, w.Qh, d);
@@ -960,7 +963,7 @@ cudaError_t jacobi_values_project(int d, const cx_t<R>* T, AbsPWork<R>& w, int s
   for (int sw = 0; sw < sweeps; ++sw)
     if ((e = jacobi_sweep<R>(d, Ain, Aout, Vin, Vout, phi, w.ucos, s)) != cudaSuccess) return e;
   w.A = Ain;
-  k_absp_spectrum<R><<<1, 1024, 0, s>>>(w.A, w.lam, w.s, w.sp, d, P, sizeof(R) == 4 ? 1e-7 : 1e-15);
+  k_absp_spectrum<R><<<(d + kSpec - 1) / kSpec, 256, 0, s>>>(w.A, w.lam, w.s, w.sp, d, P, sizeof(R) == 4 ? 1e-7 : 1e-15);
   return cudaGetLastError();
 }
 
@@ -1322,7 +1325,7 @@ cudaError_t abs_p_forward_tc_warm(int d, const void* Tb, const double* sT, AbsPW
     return e;
   if (Ain != w.A0 && (e = cudaMemcpyAsync(w.A0, Ain, nn * sizeof(float2), cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
     return e;
-  k_absp_spectrum<float><<<1, 1024, 0, s>>>(w.A0, w.lam, w.s, w.sp, d, P, 1e-7);
+  k_absp_spectrum<float><<<(d + kSpec - 1) / kSpec, 256, 0, s>>>(w.A0, w.lam, w.s, w.sp, d, P, 1e-7);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // X = Q |Lambda|^P Q^dag on tensor cores (lower tiles), and Q^dag
   return abs_p_tc_finish(d, w, fmt, X, err, s);

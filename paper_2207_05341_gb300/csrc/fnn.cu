@@ -5,6 +5,8 @@
 // width H = 2N is a template parameter so that the H running sums live in
 // registers.  Sums over the 4^N axis are reduced per block and then by the last
 // block to arrive, in a fixed order (deterministic, no floating-point atomics).
+#include <algorithm>
+
 #include "impl.h"
 
 namespace qst {
@@ -504,7 +506,7 @@ __global__ void __launch_bounds__(256) k_tri_grad(const cx_t<R>* __restrict__ Z,
 // ------------------------------------------------------------------ input check, Rprop reset
 // *out = sum f in FP64, or NaN when an entry is negative or not finite (a fixed order: per-thread sums, then the
 // blocks in turn).  One read of f, where the check on the host cost a copy of f to pageable memory and a serial
-// loop (3 ms of a 3.8 ms loss and gradient at N = 11; this pass takes about 10 us there, bound by FP64 adds).
+// loop (3 ms of a 3.8 ms loss and gradient at N = 11; this pass takes 12 us there, cold).
 template <class R>
 __global__ void __launch_bounds__(256) k_check_f(const R* __restrict__ f, long long n, double* partials,
                                                   unsigned int* counter, double* out) {
@@ -512,7 +514,7 @@ __global__ void __launch_bounds__(256) k_check_f(const R* __restrict__ f, long l
   constexpr int VW = VV::W;
   const bool vec = (reinterpret_cast<uintptr_t>(f) & 15u) == 0 && n % VW == 0;
   const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x, nt = (long long)gridDim.x * blockDim.x;
-  double s = 0.0;
+  typename SumOf<R>::T sum;
   bool bad = false;
   if (vec) {
     for (long long i = tid; i < n / VW; i += nt) {
@@ -521,16 +523,17 @@ __global__ void __launch_bounds__(256) k_check_f(const R* __restrict__ f, long l
 #pragma unroll
       for (int u = 0; u < VW; ++u) {
         bad |= !(v[u] >= R(0)) || !isfinite(v[u]);
-        s += (double)v[u];
+        sum.add(v[u]);
       }
     }
   } else {
     for (long long i = tid; i < n; i += nt) {
       const R v = f[i];
       bad |= !(v >= R(0)) || !isfinite(v);
-      s += (double)v;
+      sum.add(v);
     }
   }
+  double s = sum.value();
   if (bad) s = nan("");
   __shared__ double red[8];
   s = warp_sum(s);
@@ -583,7 +586,7 @@ template <class R> static RpropCfg<R> rcfg(const NetCfg& c) {
 
 template <class R>
 cudaError_t net_check_f(long long n, const R* f, double* partials, unsigned int* counter, double* out, cudaStream_t s) {
-  const int grid = stream_grid(k_check_f<R>, n / Vec<R>::W);
+  const int most = 2 * 152, grid = std::min(stream_grid(k_check_f<R>, n / Vec<R>::W), most);
   k_check_f<R><<<grid, 256, 0, s>>>(f, n, partials, counter, out);
   return cudaGetLastError();
 }

@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_cgemm(const __grid_constant__ TcM
   const bool ready = mbar_wait(done, 0u);
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   if (ready && !s_fail) {
-    const float unscale = (float)(1.0 / (*sA * *sB));  // exact: both scales are powers of two
+    const float unscale = pow2f(-(exponent_of(*sA) + exponent_of(*sB)));  // 1 / (sA sB), both powers of two
     const int row = I * kBM + warp * 32 + lane;
     float2* out = C + (long long)row * d + (long long)J * kBN;
     const uint32_t lane_base = tmem + ((uint32_t)(warp * 32) << 16);
@@ -247,7 +247,7 @@ template <class H> __device__ __forceinline__ void hi_lo(float v, H& hi, H& lo) 
   lo = to16<H>(v - from16(hi));
 }
 
-// Complex FP32 matrix -> 16-bit hi / lo planes of s * x (G: re, im (hi), re, im (lo)); s = split_scale(amax),
+// Complex FP32 matrix -> 16-bit hi / lo planes of s * x (G: re, im (hi), re, im (lo)); s = 2^split_exponent(amax),
 // written to *s_slot.  Each thread converts 8 consecutive entries (four 16-byte loads, one 16-byte store
 // per plane); nn is a multiple of 8.
 template <class H>
@@ -256,9 +256,9 @@ __global__ void __launch_bounds__(256) k_split(const float2* __restrict__ A, H* 
   rebind(tab, A, P, amax, s_slot);
   grid_dep_wait();
   after_wait(A, P, amax, s_slot);
-  const double sd = split_scale(amax);
-  const float sc = (float)sd;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = sd;
+  const int se = split_exponent(amax);
+  const float sc = pow2f(se);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
   union Pack {
     uint4 v;
     H h[8];
@@ -284,7 +284,7 @@ __global__ void __launch_bounds__(256) k_split(const float2* __restrict__ A, H* 
 
 // The Hermitian T of t (R = t as d x d row-major; T_ii = R_ii, T_ij = R_ij + i R_ji for i > j,
 // T_ji = conj T_ij), written straight into the 6 planes of s * T: re, im, -im (hi), then (lo);
-// s = split_scale(amax) (max |t| folded in by the kernel that wrote t), written to *s_slot.  One CTA
+// s = 2^split_exponent(amax) (max |t| folded in by the kernel that wrote t), written to *s_slot.  One CTA
 // per 32 x 32 tile pair (I, J), I >= J (d >= 32): each thread loads one float4 of each tile, and
 // writes 8 adjacent columns of one row of every plane with one 16-byte store (threads 0-127 the
 // tile (I, J), 128-255 the tile (J, I)).
@@ -295,9 +295,9 @@ __global__ void __launch_bounds__(256) k_hermitian_planes(const float* __restric
   rebind(tab, t, P, amax, s_slot);
   __shared__ float Ra[32][33];
   __shared__ float Rb[32][33];
-  const double sd = split_scale(amax);
-  const float sc = (float)sd;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = sd;
+  const int se = split_exponent(amax);
+  const float sc = pow2f(se);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
   const long long nn = (long long)d * d;
   int I, J;
   tri_decode(blockIdx.x, I, J);
@@ -352,9 +352,9 @@ __global__ void __launch_bounds__(256) k_hermitian_planes64(const float* __restr
   after_wait(t, P, amax, s_slot);
   __shared__ float Ra[64][65];
   __shared__ float Rb[64][65];
-  const double sd = split_scale(amax);
-  const float sc = (float)sd;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = sd;
+  const int se = split_exponent(amax);
+  const float sc = pow2f(se);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
   const long long nn = (long long)d * d;
   int I, J;
   tri_decode(blockIdx.x, I, J);
@@ -421,15 +421,15 @@ __global__ void __launch_bounds__(256) k_amax(const float2* __restrict__ M, long
 
 // 16-bit hi / lo planes of s * Z for a general product operand, Z = M (op 0) or M^dag (op 1), d x d
 // row-major: 4 planes (re, im; hi then lo: the left operand A of C = A B) or 6 planes (re, im, -im; hi
-// then lo: the right operand given as B^dag, which k_tc_cgemm reads row by row).  s = split_scale(amax),
+// then lo: the right operand given as B^dag, which k_tc_cgemm reads row by row).  s = 2^split_exponent(amax),
 // written to *s_slot.  One CTA per 32 x 32 tile of Z; the transpose goes through shared memory.
 template <class H>
 __global__ void __launch_bounds__(256) k_planes_op(const float2* __restrict__ M, int d, int op, int six,
                                                     H* __restrict__ P, const unsigned int* amax, double* s_slot) {
   __shared__ float2 tile[32][33];
-  const double sd = split_scale(amax);
-  const float sc = (float)sd;
-  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *s_slot = sd;
+  const int se = split_exponent(amax);
+  const float sc = pow2f(se);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
   const long long nn = (long long)d * d;
   const int bi = blockIdx.y, bj = blockIdx.x;  // tile (bi, bj) of Z
   // Z tile (bi, bj) = M tile (bi, bj) (op 0) or the conjugate transpose of M tile (bj, bi) (op 1)

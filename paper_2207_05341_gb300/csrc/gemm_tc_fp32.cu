@@ -246,7 +246,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
         part[(hf * (CH / 2) + c / 2) ^ (row & (kBN / 2 - 1))] = make_float4(re[c], im[c], re[c + 1], im[c + 1]);
     } else if (ok) {
       // C = acc / (sA sB), both powers of two; the smaller factor first (no overflow on the way)
-      const float ua = (float)(1.0 / *sA), ub = (float)(1.0 / *sB);
+      const float ua = pow2f(-exponent_of(*sA)), ub = pow2f(-exponent_of(*sB));
       const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
       float2* out = C + (long long)(I * kBM + q * 32 + lane) * d + (long long)J * kBN + hf * CH;
 #pragma unroll
@@ -262,7 +262,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
     cg::cluster_group cl = cg::this_cluster();
     __syncwarp();
     cl.sync();
-    const float ua = (float)(1.0 / *sA), ub = (float)(1.0 / *sB);
+    const float ua = pow2f(-exponent_of(*sA)), ub = pow2f(-exponent_of(*sB));
     const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
     const int rows = kBM / ks;
     constexpr int kChunks = kBN / 2;
@@ -307,7 +307,7 @@ union Pack8 {
 };
 
 // Planes of a complex matrix, 8 consecutive entries per thread: re, im (and, with nine, -im), each h, m, l.
-// *s_slot: the scale, split_scale(amax), written here; with keep, the scale already there.
+// *s_slot: the scale, 2^split_exponent(amax), written here; with keep, the scale already there.
 // X (may be NULL; A is then G = dL/dX of Chol_H): X's lower 128 x 128 tiles.  L does not change with the scale
 // of T, so Tr(G X) = 0; rounding of G's identity component (one scalar of about 2^-25 of sum f / Tr X) breaks
 // that, and its product with T is most of the gradient's error (2.4e-6 of its norm at N = 9, 3.5e-7 without).
@@ -321,11 +321,11 @@ __global__ void __launch_bounds__(256) k_split3(const float2* __restrict__ A, __
   rebind(tab, A, P, amax, s_slot, X, scal, partials, counter, flags);
   grid_dep_wait();
   after_wait(A, P, amax, s_slot, X, scal, partials, counter, flags);
-  const double sd = keep ? *s_slot : split_scale(amax);
-  const float sc = (float)sd;
-  if (!keep && blockIdx.x == 0 && threadIdx.x == 0) *s_slot = sd;
+  const int se = keep ? exponent_of(*s_slot) : split_exponent(amax);
+  const float sc = pow2f(se);
+  if (!keep && blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
   const long long n8 = nn / 8;
-  double dot = 0.0;
+  PairSum dsum;
   for (long long q = (long long)blockIdx.x * blockDim.x + threadIdx.x; q < n8; q += (long long)gridDim.x * blockDim.x) {
     const float4* src = reinterpret_cast<const float4*>(A + 8 * q);
     Pack8 r[3], i[3];
@@ -342,7 +342,7 @@ __global__ void __launch_bounds__(256) k_split3(const float2* __restrict__ A, __
           const float4 x = xs[u];
           p = fmaf(av[u].x, x.x, fmaf(av[u].y, x.y, fmaf(av[u].z, x.z, fmaf(av[u].w, x.w, p))));
         }
-        dot += (ti > tj ? 2.0 : 1.0) * (double)p;
+        dsum.add(ti > tj ? 2.f * p : p);
       }
     }
 #pragma unroll
@@ -371,7 +371,7 @@ __global__ void __launch_bounds__(256) k_split3(const float2* __restrict__ A, __
   }
   if (!X) return;
   __shared__ double red[8];
-  dot = warp_sum(dot);
+  const double dot = warp_sum(dsum.value());
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = dot;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -403,9 +403,9 @@ __global__ void __launch_bounds__(256) k_hermitian_planes3(const float* __restri
   after_wait(t, P, amax, s_slot);
   __shared__ float Ra[64][65];
   __shared__ float Rb[64][65];
-  const double sd = split_scale(amax);
-  const float sc = (float)sd;
-  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = sd;
+  const int se = split_exponent(amax);
+  const float sc = pow2f(se);
+  if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
   const long long nn = (long long)d * d;
   int I, J;
   tri_decode(blockIdx.x, I, J);
@@ -497,7 +497,7 @@ cudaError_t tc32_split(int d, const float2* A, void* P, int planes, bool keep_sc
   const long long nn = (long long)d * d;
   if (nn % 1024 || (planes != 6 && planes != 9)) return cudaErrorInvalidValue;
   long long blocks = (nn / 8 + 255) / 256;
-  if (blocks > 2048) blocks = 2048;
+  if (blocks > (X ? 608 : 2048)) blocks = X ? 608 : 2048;  // with X: four per SM, fewer FP64 sums
   BatchArgs ba;
   if (batch_take(ba, {A, P, amax, s_slot, X, scal, partials, counter, flags})) return cudaSuccess;
   return launch_dep(k_split3, dim3((unsigned)blocks, 1, ba.nz), dim3(256), 0, s, A, (__nv_bfloat16*)P, nn,

@@ -111,7 +111,7 @@ template <class R> struct Work {
   R* fstage;           // staging copy of a host f, n reals
   R* fperm;            // f in the order of the structured likelihood pass (FP32 fast path), n reals
   double* scal;        // [0] Tr X, [1] sum f, [2] loss, [3] scale of T, [4] scale of G, [5] F_c,
-                       // [8..10] state fidelity (sum g, bracket bound, F_q), [12] kGauge, [13] kCheckF
+                       // [8..10] state fidelity (sum g, bracket bound, F_q), [12] kGauge, [13] kCheckF, [14], [15] kConst64, kConst32
   double* partials;    // per-block partial sums
   unsigned int* counters;  // last-block counters, one per reduction site
   unsigned int* flags;     // [0] clamp count, [1] device-side wait timeouts, [2] sampler's bad input, [4] the
@@ -148,6 +148,7 @@ constexpr int kScaleT = 3;  // scal slot of the power-of-two scale of T (mixed p
 constexpr int kScaleG = 4;  // scal slot of the scale of G
 constexpr int kGauge = 12;  // scal slot of the multiple of T that makes Tr(G X) = 0 (FP32 tensor-core products)
 constexpr int kCheckF = 13;  // scal slot of the sum of a new f, NaN for a bad entry
+constexpr int kConst64 = 14, kConst32 = 15;  // scal slots of sum f / Tr X as FP64 and as FP32 (a float in the slot)
 constexpr int kPartialBlocks = 1024;   // max blocks of a reducing kernel
 constexpr int kPartialStride = 32;     // doubles per block in `partials` (>= H + 1)
 
@@ -173,7 +174,7 @@ template <class R> cudaError_t povm_hi_fwd_pauli(const Dims& D, const R* W, R* p
 template <class R> cudaError_t povm_hi_nll_pauli(const Dims& D, const R* W, const R* f, double* scal, R* Wadj,
                                                  double* partials, unsigned int* counter, unsigned int* flags,
                                                  const PovmB<R>& B, bool adjoint, cudaStream_t s);
-// scal[0] = Tr X = sum_i Re X_ii of the computed X (fixed-order FP64 sum)
+// scal[0] = Tr X = sum_i Re X_ii of the computed X (fixed-order FP64 sum), and sum f / Tr X from scal[1]
 template <class R> cudaError_t trace_X(const Dims& D, const cx_t<R>* X, double* scal, cudaStream_t s);
 // full Hermitian matrix from its lower tiles, scaled by 1 / scal[0] (rho = X / Tr X)
 template <class R> cudaError_t hermitian_complete(const Dims& D, const cx_t<R>* Xlow, cx_t<R>* rho,
@@ -198,7 +199,8 @@ bool povm_fast_ok(const Dims& D);
 // row-major tile pairs otherwise).  Pass 2 (high qubits): the structured path's own kernels, else the
 // Pauli-basis kernels of povm_pauli.cu on the row-major layout.
 cudaError_t povm_fwd_fast(const Dims& D, const float2* X, float* W, float* p, const PovmPlan& P, cudaStream_t s);
-cudaError_t povm_lo_fwd_fast(const Dims& D, const float2* X, float* W, const PovmPlan& P, cudaStream_t s);
+// scal (may be NULL): one more CTA beside the tiles forms Tr X (trace_X's sum) for the likelihood pass
+cudaError_t povm_lo_fwd_fast(const Dims& D, const float2* X, float* W, const PovmPlan& P, double* scal, cudaStream_t s);
 // The structured likelihood pass reads f permuted into its own consumption order (povm_permute_f,
 // n reals): f is constant while its pointer is, so the copy is made once per new f.
 bool povm_needs_fperm(const PovmPlan& P);

@@ -22,6 +22,7 @@
 
 #include "impl.h"
 #include "modes.cuh"
+#include "trace.cuh"
 
 namespace qst {
 
@@ -260,7 +261,7 @@ __global__ void __launch_bounds__(256) k_povm_hi_nll(const R* __restrict__ W, co
 
   // L = -sum_k f_k log q_k + (sum_k f_k) log Tr X;  g_k = dL/dq_k = -f_k / q_k + sum f / Tr X
   const double tX = scal[0], sumf = scal[1];
-  const R gconst = (R)(sumf / tX);
+  const R gconst = likelihood_const<R>(scal);  // (R)(sumf / tX)
   const R qmin = min_normal<R>();
   double acc = 0.0;
   unsigned int nclamp = 0;
@@ -323,30 +324,10 @@ __global__ void __launch_bounds__(256) k_povm_hi_nll(const R* __restrict__ W, co
 template <class R>
 __global__ void __launch_bounds__(256) k_trace(const cx_t<R>* __restrict__ X, int d, double* scal,
                                                 const void* const* tab) {
-  __shared__ double red[8];
   rebind(tab, X, scal);
   grid_dep_wait();
   after_wait(X, scal);
-  // every diagonal load of a thread is issued before the first add (one memory latency, not d / 256)
-  constexpr int kPer = 16;  // d <= 4096 = 16 x 256
-  R v[kPer];
-#pragma unroll
-  for (int k = 0; k < kPer; ++k) {
-    const int i = threadIdx.x + k * 256;
-    v[k] = i < d ? X[(long long)i * d + i].x : R(0);
-  }
-  double acc = 0.0;
-#pragma unroll
-  for (int k = 0; k < kPer; ++k)
-    if (threadIdx.x + k * 256 < d) acc += (double)v[k];
-  acc = warp_sum(acc);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    scal[0] = t;
-  }
+  block_trace<R>(X, d, scal);
 }
 
 // ---------------------------------------------------------------- rho = X / Tr X from lower tiles
@@ -357,7 +338,8 @@ __global__ void __launch_bounds__(256) k_herm_complete(const cx_t<R>* __restrict
   __shared__ V tile[32][33];
   const int TS = d < 32 ? d : 32;
   const int bi = blockIdx.y, bj = blockIdx.x;  // output tile (row block, col block)
-  const R s = (R)(1.0 / scal[0]);
+  __shared__ R s_inv;
+  if (threadIdx.x == 0) s_inv = (R)(1.0 / scal[0]);  // one FP64 division per CTA, not per thread (20 us at N = 11)
   // load the tile of the lower triangle that covers this output tile
   const int lr = bi >= bj ? bi : bj, lc = bi >= bj ? bj : bi;
   for (int e = threadIdx.x; e < TS * TS; e += blockDim.x) {
@@ -365,6 +347,7 @@ __global__ void __launch_bounds__(256) k_herm_complete(const cx_t<R>* __restrict
     tile[r][c] = X[(long long)(lr * TS + r) * d + lc * TS + c];
   }
   __syncthreads();
+  const R s = s_inv;
   for (int e = threadIdx.x; e < TS * TS; e += blockDim.x) {
     const int r = e / TS, c = e % TS;
     const int gi = bi * TS + r, gj = bj * TS + c;

@@ -26,6 +26,7 @@
 #include <float.h>
 
 #include "impl.h"
+#include "trace.cuh"
 
 namespace qst {
 
@@ -182,12 +183,20 @@ __device__ __forceinline__ float4 ld4(const float2* p) {
 }
 
 // ---------------------------------------------------------------- pass 1, forward
-template <class MAP, bool XOR>
+// TRACE: one CTA beside the tiles forms Tr X (an instantiation of its own: the plain map keeps its registers).
+template <class MAP, bool XOR, bool TRACE>
 __global__ void __launch_bounds__(kLoThreads, 4) k_lo_fwd_fast(const float2* __restrict__ X, float* __restrict__ W,
-                                                                 int N, MAP m, Out4 outmap, const void* const* tab) {
+                                                                 int N, MAP m, Out4 outmap, double* scal,
+                                                                 const void* const* tab) {
   __shared__ float2 Z[kTile * kTile];
-  rebind(tab, X, W);
+  rebind(tab, X, W, scal);
   pdl_trigger();
+  if (TRACE && blockIdx.x == gridDim.x - 1) {  // the trace, beside the tiles instead of in a launch of its own
+    pdl_wait();
+    after_wait(X, scal);
+    block_trace<float>(X, 1 << N, scal);
+    return;
+  }
   const long long d = 1LL << N;
   const int nb = (int)(d >> 6);
   int I, J;
@@ -432,7 +441,7 @@ __global__ void __launch_bounds__(kCP * NB, (NB == 32 && kCP == 8) ? 2 : 1) k_hi
   }
   __syncthreads();
   pdl_wait();
-  after_wait(f);
+  after_wait(f, scal);
   // ---- thread (cp, x = wv): the sequence of the diagonal x, transformed r -> z -> zeta
   float2 w[NB];
   {
@@ -499,8 +508,7 @@ __global__ void __launch_bounds__(kCP * NB, (NB == 32 && kCP == 8) ? 2 : 1) k_hi
     return;
   }
   // L = -sum f log q + (sum f) log Tr X;  g_k = -f_k / q_k + sum f / Tr X
-  const double tX = scal[0], sumf = scal[1];
-  const float gconst = (float)(sumf / tX);
+  const float gconst = likelihood_const<float>(scal);
   float acc = 0.f;
   unsigned int nclamp = 0;
 #pragma unroll
@@ -539,7 +547,7 @@ __global__ void __launch_bounds__(kCP * NB, (NB == 32 && kCP == 8) ? 2 : 1) k_hi
       for (int b = t; b < (int)gridDim.x; b += 32) v += partials[b];
       v = warp_sum(v);
       if (t == 0) {
-        scal[2] = -v + sumf * log(tX);
+        scal[2] = -v + scal[1] * log(scal[0]);
         *counter = 0u;
       }
     }
@@ -704,24 +712,27 @@ PovmPlan make_povm_plan(const PovmB<double>& Bd) {
 
 bool povm_fast_ok(const Dims& D) { return D.g == 6 && D.N >= 7 && D.N <= 11 && D.C > 0; }
 
-cudaError_t povm_lo_fwd_fast(const Dims& D, const float2* X, float* W, const PovmPlan& P, cudaStream_t s) {
-  const unsigned tiles = (unsigned)(D.nb * (D.nb + 1) / 2);
+cudaError_t povm_lo_fwd_fast(const Dims& D, const float2* X, float* W, const PovmPlan& P, double* scal,
+                             cudaStream_t s) {
+  const unsigned tiles = (unsigned)(D.nb * (D.nb + 1) / 2) + (scal ? 1u : 0u);
   const Out4 o = out_of(P);
   BatchArgs ba;
-  if (batch_take(ba, {X, W})) return cudaSuccess;
+  if (batch_take(ba, {X, W, scal})) return cudaSuccess;
   if (P.structured) {
     const MapStruct m = map_struct(P);
-    return launch_dep(k_lo_fwd_fast<MapStruct, true>, dim3(tiles, 1, ba.nz), dim3(kLoThreads), 0, s, X, W, D.N, m, o,
-                      ba.tab);
+    return launch_dep(scal ? k_lo_fwd_fast<MapStruct, true, true> : k_lo_fwd_fast<MapStruct, true, false>,
+                      dim3(tiles, 1, ba.nz), dim3(kLoThreads), 0, s, X, W, D.N, m, o,
+                      scal, ba.tab);
   } else {
     const MapGeneric m = map_generic(P);
-    return launch_dep(k_lo_fwd_fast<MapGeneric, false>, dim3(tiles, 1, ba.nz), dim3(kLoThreads), 0, s, X, W, D.N, m,
-                      o, ba.tab);
+    return launch_dep(scal ? k_lo_fwd_fast<MapGeneric, false, true> : k_lo_fwd_fast<MapGeneric, false, false>,
+                      dim3(tiles, 1, ba.nz), dim3(kLoThreads), 0, s, X, W, D.N, m,
+                      o, scal, ba.tab);
   }
 }
 
 cudaError_t povm_fwd_fast(const Dims& D, const float2* X, float* W, float* p, const PovmPlan& P, cudaStream_t s) {
-  cudaError_t e = povm_lo_fwd_fast(D, X, W, P, s);
+  cudaError_t e = povm_lo_fwd_fast(D, X, W, P, nullptr, s);
   if (e != cudaSuccess) return e;
   if (P.structured)
     return dispatch_hi<0>(D, W, p, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, P, false, s);

@@ -23,6 +23,7 @@
 #include <float.h>
 
 #include "impl.h"
+#include "trace.cuh"
 
 namespace qst {
 
@@ -189,7 +190,7 @@ __global__ void __launch_bounds__(32 * pauli_warps<R, NB>()) k_povm_hi_pauli(con
 
   // L = -sum f log q + (sum f) log Tr X;  g_k = -f_k / q_k + sum f / Tr X
   const double tX = scal[0], sumf = scal[1];
-  const R gconst = (R)(sumf / tX);
+  const R gconst = likelihood_const<R>(scal);  // (R)(sumf / tX)
   const R qmin = min_norm<R>();
   R accr = R(0);  // a lane's terms in R (FP64 arithmetic is a slow pipe on this part); lanes, blocks in FP64
   unsigned int nclamp = 0;

@@ -74,14 +74,24 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "memory");
 }
 
-// Scale of an operand split: 2^-e for the largest |re|, |im| in [2^e, 2^(e+1)) (*amax, float bits, folded
-// in by the kernel that wrote the matrix), i.e. the power of two that brings it into [1, 2); 1 without amax.
-__device__ __forceinline__ double split_scale(const unsigned int* amax) {
-  if (!amax) return 1.0;
-  const double m = (double)__uint_as_float(*reinterpret_cast<const volatile unsigned int*>(amax));
-  if (!(m > 0.0) || !isfinite(m)) return 1.0;
-  const int e = -ilogb(m);
-  return ldexp(1.0, e > 126 ? 126 : e);  // a finite FP32 factor for subnormal maxima too
+// Scale of an operand split: 2^k that brings the largest |re|, |im| (*amax, float bits, folded in by the kernel that
+// wrote the matrix) into [1, 2), k <= 126; 1 without amax, for 0 and for a maximum that is not finite.  By its
+// exponent alone (every thread of a split comes through here: no FP64 arithmetic).
+__device__ __forceinline__ int split_exponent(const unsigned int* amax) {
+  if (!amax) return 0;
+  const unsigned int b = *reinterpret_cast<const volatile unsigned int*>(amax);
+  const int e = (int)(b >> 23);
+  if (b == 0u || e >= 255) return 0;
+  const int k = e > 0 ? 127 - e : 118 + __clz((int)b);  // a subnormal maximum m = b 2^-149
+  return k > 126 ? 126 : k;
 }
+__device__ __forceinline__ float pow2f(int k) {  // 2^k, -149 <= k <= 127 (0 and infinity beyond)
+  if (k > 127) return __int_as_float(0x7F800000);
+  if (k >= -126) return __int_as_float((k + 127) << 23);
+  return k >= -149 ? __int_as_float(1 << (k + 149)) : 0.f;
+}
+__device__ __forceinline__ double pow2d(int k) { return __hiloint2double((1023 + k) << 20, 0); }  // |k| <= 1022
+// k of a scale 2^k kept as a double
+__device__ __forceinline__ int exponent_of(double s) { return ((__double2hiint(s) >> 20) & 0x7FF) - 1023; }
 
 }  // namespace qst

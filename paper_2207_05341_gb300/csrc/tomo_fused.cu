@@ -91,23 +91,6 @@ __device__ double block_sum1(double v, double* red) {
   return red[kTot];
 }
 
-// s + e: a sum kept as an FP32 pair (Knuth's two-sum; the products' rounding errors by FMA), so that a thread's
-// terms keep about 48 bits without the FP64 pipe (two operations per clock and SM)
-struct PairSum {
-  float s = 0.f, e = 0.f;
-  __device__ __forceinline__ void add(float v) {
-    const float t = s + v, b = t - s;
-    e += (s - (t - b)) + (v - b);
-    s = t;
-  }
-  __device__ __forceinline__ void add_product(float a, float b) {
-    const float p = a * b;
-    e += fmaf(a, b, -p);
-    add(p);
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
-};
-
 // C = A B in shared memory (pitch P): warp w takes rows RP w .., lane l the columns l + 32 c.
 template <int D, int RP, int CP> __device__ void smem_cgemm(const float2* A, const float2* B, float2* C) {
   constexpr int P = pitch_of(D);
@@ -275,7 +258,9 @@ __device__ void tomo_iteration(const TomoDesc& td, const PovmB<float>& Bm, const
   for (int i = tid; i < d; i += nth) tr += (double)X[i * P + i].x;
   const double tX = block_sum1(tr, sm.red);
   if (td.rho) {  // rho from the lower triangle of X
-    const float s = (float)(1.0 / tX);
+    if (tid == 0) sm.vec[62] = (float)(1.0 / tX);
+    __syncthreads();
+    const float s = sm.vec[62];
     for (int e = tid; e < n; e += nth) {
       const int i = e >> N, j = e & (d - 1);
       const float2 x = i >= j ? X[i * P + j] : cconj(X[j * P + i]);
@@ -288,7 +273,9 @@ __device__ void tomo_iteration(const TomoDesc& td, const PovmB<float>& Bm, const
   else block_modes<false>(X, N, Bm);
   // S6: likelihood, and g = dL/dq into G
   const double sumf = td.scal[1];
-  const float gconst = (float)(sumf / tX);
+  if (tid == 0) sm.vec[63] = (float)(sumf / tX);
+  __syncthreads();
+  const float gconst = sm.vec[63];
   PairSum acc;
   unsigned int nclamp = 0;
   for (int k = tid; k < n; k += nth) {
@@ -308,13 +295,15 @@ __device__ void tomo_iteration(const TomoDesc& td, const PovmB<float>& Bm, const
     G[e] = make_float2(gk, 0.f);
   }
   if (nclamp) atomicAdd(td.flags, nclamp);
-  const double ll = block_sum1(acc.value(), sm.red);
-  if (tid == 0) {
+  const double ll = block_sum1(acc.value(), sm.red);  // its barriers also order G
+  if (tid == nth - 32) {  // (the last warp sits out the POVM sweeps of N <= 6)
     td.scal[0] = tX;
     td.scal[2] = -ll + sumf * log(tX);
   }
-  __syncthreads();
-  if (td.rho) return;
+  if (td.rho) {
+    __syncthreads();
+    return;
+  }
   // S7: G = sum_k g_k M_k in place
   if (SM) apply_modes_tile<float, true>(G, N, P, Bm);
   else block_modes<true>(G, N, Bm);
