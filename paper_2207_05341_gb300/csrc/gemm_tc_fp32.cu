@@ -97,8 +97,6 @@ __global__ void __launch_bounds__(kThreads32, 1)
                  const void* const* tab) {
   const Maps32* mp = &maps;
   rebind(tab, mp, C, sA, sB, err, clear);
-  grid_dep_wait();
-  after_wait(mp, C, sA, sB, err, clear);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStage);
@@ -119,8 +117,12 @@ __global__ void __launch_bounds__(kThreads32, 1)
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0u;
+  // barriers, TMEM and descriptors before the wait for the kernel that makes the planes
   if (threadIdx.x == 0) {
+    if (!tab) {
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mp->a)) : "memory");
+      asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&mp->b)) : "memory");
+    }
     for (int s = 0; s < kStages; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
@@ -142,6 +144,9 @@ __global__ void __launch_bounds__(kThreads32, 1)
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
+  grid_dep_wait();
+  after_wait(mp, C, sA, sB, err, clear);
+  if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0u;
   const int kbeg = krange == 1 ? I * kBM : 0, kend = krange == 2 ? (I + 1) * kBM : d;
   const int half = (kend - kbeg) / kBK;                       // K blocks of the real part, and of the imaginary part
   const int kb0 = 2 * half * rank / ks, nkb = 2 * half * (rank + 1) / ks - kb0;  // this CTA's
@@ -265,17 +270,33 @@ __global__ void __launch_bounds__(kThreads32, 1)
     const float ua = pow2f(-exponent_of(*sA)), ub = pow2f(-exponent_of(*sB));
     const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
     const int rows = kBM / ks;
-    constexpr int kChunks = kBN / 2;
-    for (int e = threadIdx.x; e < rows * kChunks; e += kThreads32) {
-      const int row = rank * rows + e / kChunks, ch = e % kChunks;
-      float4* at = reinterpret_cast<float4*>(smem) + row * kChunks + (ch ^ (row & (kChunks - 1)));
-      float4 v = *cl.map_shared_rank(at, 0);
-      for (int r = 1; r < ks; ++r) {
-        const float4 w = *cl.map_shared_rank(at, r);
-        v.x += w.x; v.y += w.y; v.z += w.z; v.w += w.w;
+    constexpr int kChunks = kBN / 2, kFly = 4;  // a thread's chunks in flight together
+    for (int e0 = threadIdx.x; e0 < rows * kChunks; e0 += kFly * kThreads32) {
+      float4 v[kFly];
+      for (int r = 0; r < ks; ++r) {
+        float4 w[kFly];
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) {
+          const int e = e0 + u * kThreads32;
+          if (e < rows * kChunks) {
+            const int row = rank * rows + e / kChunks, ch = e % kChunks;
+            w[u] = *cl.map_shared_rank(reinterpret_cast<float4*>(smem) + row * kChunks + (ch ^ (row & (kChunks - 1))), r);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kFly; ++u) {
+          if (r == 0) { v[u] = w[u]; continue; }
+          v[u].x += w[u].x; v[u].y += w[u].y; v[u].z += w[u].z; v[u].w += w[u].w;
+        }
       }
-      *reinterpret_cast<float4*>(C + (long long)(I * kBM + row) * d + (long long)J * kBN + 2 * ch) =
-          make_float4(v.x * u1 * u2, v.y * u1 * u2, v.z * u1 * u2, v.w * u1 * u2);
+#pragma unroll
+      for (int u = 0; u < kFly; ++u) {
+        const int e = e0 + u * kThreads32;
+        if (e >= rows * kChunks) continue;
+        const int row = rank * rows + e / kChunks, ch = e % kChunks;
+        *reinterpret_cast<float4*>(C + (long long)(I * kBM + row) * d + (long long)J * kBN + 2 * ch) =
+            make_float4(v[u].x * u1 * u2, v[u].y * u1 * u2, v[u].z * u1 * u2, v[u].w * u1 * u2);
+      }
     }
     cl.sync();  // no CTA leaves while its part may still be read
   }
@@ -321,6 +342,7 @@ __global__ void __launch_bounds__(256) k_split3(const float2* __restrict__ A, __
   rebind(tab, A, P, amax, s_slot, X, scal, partials, counter, flags);
   grid_dep_wait();
   after_wait(A, P, amax, s_slot, X, scal, partials, counter, flags);
+  asm volatile("griddepcontrol.launch_dependents;");  // the product's prologue may start
   const int se = keep ? exponent_of(*s_slot) : split_exponent(amax);
   const float sc = pow2f(se);
   if (!keep && blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
@@ -401,6 +423,7 @@ __global__ void __launch_bounds__(256) k_hermitian_planes3(const float* __restri
   rebind(tab, t, P, amax, s_slot);
   grid_dep_wait();
   after_wait(t, P, amax, s_slot);
+  asm volatile("griddepcontrol.launch_dependents;");  // the product's prologue may start
   __shared__ float Ra[64][65];
   __shared__ float Rb[64][65];
   const int se = split_exponent(amax);
