@@ -719,9 +719,18 @@ template <class R> struct Engine {
   }
 
   static qst_status read_loss(qst_ctx* c, double* loss) {
+    const qst_status st = loss_begin(c);
+    return st == QST_OK ? loss_end(c, loss) : st;
+  }
+  // The copies of the loss and the flags are enqueued; loss_end waits for them.
+  static qst_status loss_begin(qst_ctx* c) {
     Work<R>* w = W<R>(c);
     QST_CU(cudaMemcpyAsync(c->h_scal, w->scal, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
     QST_CU(cudaMemcpyAsync(c->h_flags, w->flags, 2 * sizeof(unsigned int), cudaMemcpyDeviceToHost, c->stream));
+    return QST_OK;
+  }
+  static qst_status loss_end(qst_ctx* c, double* loss) {
+    Work<R>* w = W<R>(c);
     QST_CU(cudaStreamSynchronize(c->stream));
     *loss = c->h_scal[2];
     if (c->h_flags[1] != 0u) {
@@ -1061,7 +1070,8 @@ template <class R> struct Engine {
     return QST_OK;
   }
 
-  static qst_status get_rho(qst_ctx* c, const void* f_user, void* rho_out, double* loss) {
+  // want_loss: the loss is on its way when this returns (loss_end)
+  static qst_status rho_begin(qst_ctx* c, const void* f_user, void* rho_out, bool want_loss) {
     Work<R>* w = W<R>(c);
     const Dims& D = c->D;
     qst_status st;
@@ -1085,12 +1095,13 @@ template <class R> struct Engine {
           QST_CU(cudaMemcpyAsync(rho_out, dst, (size_t)D.d * D.d * sizeof(V), cudaMemcpyDeviceToHost, c->stream));
           QST_CU(cudaStreamSynchronize(c->stream));
         }
-        return loss ? read_loss(c, loss) : QST_OK;
+        return want_loss ? loss_begin(c) : QST_OK;
       }
     }
     if ((st = forward_state(c, w->theta)) != QST_OK) return st;
+    if (want_loss && (st = povm_likelihood(c, f, false)) != QST_OK) return st;
     if (rho_out) {
-      if (fast_povm(c)) {
+      if (fast_povm(c) && !want_loss) {
         QST_CU(trace_X<R>(D, w->X, w->scal, c->stream));
         c->launches += 1;
       }
@@ -1101,11 +1112,12 @@ template <class R> struct Engine {
         QST_CU(cudaStreamSynchronize(c->stream));
       }
     }
-    if (loss) {
-      if ((st = povm_likelihood(c, f, false)) != QST_OK) return st;
-      return read_loss(c, loss);
-    }
-    return QST_OK;
+    return want_loss ? loss_begin(c) : QST_OK;
+  }
+
+  static qst_status get_rho(qst_ctx* c, const void* f_user, void* rho_out, double* loss) {
+    const qst_status st = rho_begin(c, f_user, rho_out, loss != nullptr);
+    return st == QST_OK && loss ? loss_end(c, loss) : st;
   }
 };
 
@@ -1939,10 +1951,18 @@ qst_status qst_batch_reconstruct(qst_batch* bt, const void* const* f, int iters,
     if (st < 0) return st;
   }
   QST_CU(cudaStreamSynchronize(bt->root));
+  if (!rho_out && !final_losses) return QST_OK;
+  // every tomography's state and loss are enqueued on its own stream before the first loss is waited for
   for (int b = 0; b < bt->B; ++b) {
-    if (!rho_out && !final_losses) break;
-    const qst_status st = qst_get_rho(bt->ctx[b], f[b], rho_out ? rho_out[b] : nullptr,
-                                      final_losses ? final_losses + b : nullptr);
+    qst_ctx* c = bt->ctx[b];
+    if (!f[b]) return QST_E_INVAL;
+    if (!c->params_set) return QST_E_STATE;
+    const qst_status st = QST_DISPATCH(c, rho_begin(c, f[b], rho_out ? rho_out[b] : nullptr, final_losses != nullptr));
+    if (st < 0) return st;
+  }
+  for (int b = 0; final_losses && b < bt->B; ++b) {
+    qst_ctx* c = bt->ctx[b];
+    const qst_status st = QST_DISPATCH(c, loss_end(c, final_losses + b));
     if (st < 0) return st;
   }
   return QST_OK;
