@@ -331,10 +331,11 @@ qst_status qst_graph_enable(qst_ctx* ctx, int enable);
 
 /* Launch parameters of the library, process-wide (instrumentation of the library, not part of the
  * method; the shipped defaults were chosen by the package's autotuner on the target GPU).
- *   bulk_chunks_per_cta  least number of 256-column chunks that one CTA of an FP32 weight pass (and of
- *                        the layer-1 forward that shares its partition) streams, >= 1; the grid is at
- *                        most one CTA per SM.  It fixes how the passes' sums over 4^N terms are split,
- *                        so results change in the last bits with it.
+ *   bulk_chunks_per_cta  least number of 256-column chunks in a group of an FP32 weight pass (and of
+ *                        the layer-1 forward that shares its partition), >= 1; there are at most as many
+ *                        groups as SMs.  A single tomography runs a CTA per group, a batch CTAs that walk
+ *                        several.  The groups fix how the passes' sums over 4^N terms are split, so results
+ *                        change in the last bits with it.
  *   fused_ctas_per_sm    resident CTAs per SM of the persistent launch of a batch's fused tomographies
  *                        (1 or 2); results do not depend on it.
  *   fused_max_qubits     the limit qst_options.fused_max_qubits = 0 stands for (0..7; 0 = never).

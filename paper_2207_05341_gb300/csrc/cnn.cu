@@ -416,7 +416,7 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
 #pragma unroll
   for (int j0 = 0; j0 < H; j0 += 4) {  // H = 4 N: four rows at a time
     const R a4[4] = {acc[j0], acc[j0 + 1], acc[j0 + 2], acc[j0 + 3]};
-    warp_sums<4>(a4, [&](int j, double x) { red[wp][j0 + j] = x; });
+    warp_sums<4>(a4, [&](int j, typename SumOf<R>::T x) { red[wp][j0 + j] = x.value(); });
   }
   __syncthreads();
   for (int j = threadIdx.x; j < H; j += blockDim.x) {

@@ -162,39 +162,65 @@ struct WideSum {
 template <class R> struct SumOf { using T = PairSum; };
 template <> struct SumOf<double> { using T = WideSum; };
 
-// Sums of M values each over a warp: out(j, sum) is called once per j, by one lane.  Step by step a lane hands half
-// of the values it still carries to its partner, which hands over the other half, so M = 11 takes 16 FP64 adds
-// where M butterflies take 55 (an FP64 add is 64 issue cycles of a scheduler here: two per clock and SM).  The
-// pairs added are warp_sum's, so every sum has its bits.
+// The sum of two pairs.
+__device__ __forceinline__ PairSum pair_add(PairSum a, PairSum b) {
+  PairSum r = a;
+  r.add(b.s);
+  r.e = __fadd_rn(r.e, b.e);
+  return r;
+}
+__device__ __forceinline__ WideSum pair_add(WideSum a, WideSum b) {
+  a.s += b.s;
+  return a;
+}
+__device__ __forceinline__ PairSum pair_xor(PairSum a, int o) {
+  PairSum r;
+  r.s = __shfl_xor_sync(0xffffffffu, a.s, o);
+  r.e = __shfl_xor_sync(0xffffffffu, a.e, o);
+  return r;
+}
+__device__ __forceinline__ WideSum pair_xor(WideSum a, int o) {
+  a.s = __shfl_xor_sync(0xffffffffu, a.s, o);
+  return a;
+}
+
+// Sums of M values each over a warp: out(j, sum) is called once per j, by one lane, with an FP32 pair (or, for FP64
+// values, an FP64 sum).  Step by step a lane hands half of the values it still carries to its partner, which hands
+// over the other half: M = 11 takes 16 additions where M butterflies take 55; and the additions are FP32 two-sums,
+// 10 issue slots each, where an FP64 add with its conversions takes 64 to 192 (two operations per clock and SM).
 template <int M, class R, class F> __device__ __forceinline__ void warp_sums(const R (&v)[M], F out) {
   static_assert(M >= 1 && M <= 32, "at most one value per lane");
+  using S = typename SumOf<R>::T;
   constexpr int L = M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : M <= 16 ? 4 : 5, P = 1 << L;
   const int lane = threadIdx.x & 31;
-  double a[P > 1 ? P / 2 : 1];
+  S a[P > 1 ? P / 2 : 1];
+  int o = 16;
   if constexpr (P == 1) {
-    a[0] = warp_sum((double)v[0]);
+    a[0].add(v[0]);
   } else {
     const bool up = (lane & 16) != 0;
 #pragma unroll
     for (int k = 0; k < P / 2; ++k) {
       const R lo = k < M ? v[k < M ? k : 0] : R(0), hi = k + P / 2 < M ? v[k + P / 2 < M ? k + P / 2 : 0] : R(0);
       const R keep = up ? hi : lo, send = up ? lo : hi;
-      a[k] = (double)keep + (double)__shfl_xor_sync(0xffffffffu, send, 16);
+      a[k].s = keep;
+      a[k].add(__shfl_xor_sync(0xffffffffu, send, 16));
     }
+    o = 8;
+  }
 #pragma unroll
-    for (int o = 8, c = P / 2; o > 0; o >>= 1) {
-      if (c > 1) {
-        c >>= 1;
-        const bool u = (lane & o) != 0;
+  for (int c = P / 2; o > 0; o >>= 1) {
+    if (c > 1) {
+      c >>= 1;
+      const bool u = (lane & o) != 0;
 #pragma unroll
-        for (int k = 0; k < P / 4; ++k) {
-          if (k >= c) break;
-          const double keep = u ? a[k + c] : a[k], send = u ? a[k] : a[k + c];
-          a[k] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-        }
-      } else {
-        a[0] += __shfl_xor_sync(0xffffffffu, a[0], o);
+      for (int k = 0; k < P / 4; ++k) {
+        if (k >= c) break;
+        const S keep = u ? a[k + c] : a[k], send = u ? a[k] : a[k + c];
+        a[k] = pair_add(keep, pair_xor(send, o));
       }
+    } else {
+      a[0] = pair_add(a[0], pair_xor(a[0], o));
     }
   }
   const int j = lane >> (5 - L);

@@ -32,15 +32,16 @@ constexpr int kRowBatch = 4;
 // Reduce M per-thread values over the block; thread 0 writes them (as double) to out[0..M).
 template <int M, class R>
 __device__ __forceinline__ void block_reduce_to(const R (&v)[M], double* out) {
-  __shared__ double red[8][M];
+  using S = typename SumOf<R>::T;
+  __shared__ S red[8][M];
   const int w = threadIdx.x >> 5;
-  warp_sums<M>(v, [&](int j, double x) { red[w][j] = x; });
+  warp_sums<M>(v, [&](int j, S x) { red[w][j] = x; });
   __syncthreads();
   const int nw = blockDim.x >> 5;
   for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    double s = 0.0;
-    for (int q = 0; q < nw; ++q) s += red[q][j];
-    out[j] = s;
+    S s;
+    for (int q = 0; q < nw; ++q) s = pair_add(s, red[q][j]);
+    out[j] = s.value();
   }
 }
 

@@ -1,7 +1,11 @@
 // Rprop weight passes of the Sec. 3.1 network (FP32, in-place update) with bulk-copy staging.
 //
-// Each CTA walks chunks of kCols consecutive columns of the 4^N axis (chunk c to CTA
-// c mod grid, one CTA per SM).  The CTA is warp-specialised: one producer thread issues,
+// The 4^N axis is cut into chunks of kCols consecutive columns and the chunks into groups (chunk c to group
+// c mod groups); a group is what the sums over the axis are split by, whatever the launch: a single tomography
+// runs a CTA per group (at most one per SM), and a batch, whose members fill the GPU together, CTAs that walk
+// several groups one after another without letting the ring run dry.  (With at least 32 chunks to a CTA, as the
+// batch liked it, an N = 7 pass was 2 CTAs and took 45 us, 12 now; N = 8 49 and 14, N = 9 59 and 25, N = 10 79 and
+// 70 us, against 5, 11 and 48 us for the bytes of N = 8, 9 and 10.)  The CTA is warp-specialised: one producer thread issues,
 // per chunk, one 2-D tensor copy (cp.async.bulk.tensor, box kCols x H) of each parameter
 // array (weights, Rprop state words: H rows n apart) and 1-D bulk copies of the
 // chunk of dt (W2 pass) or f (W1 pass) and of b2's state, all counted on the stage's
@@ -54,6 +58,8 @@ __device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// barrier of the consumer warps alone (the producer warp goes on issuing copies)
+__device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"r"(kConsumers) : "memory"); }
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   if (bar_try(bar, parity)) return true;
   const unsigned long long t0 = clock64();
@@ -124,23 +130,24 @@ template <class R> __device__ __forceinline__ R leaky_b(R x, R slope) { return x
 // thread of the block calls it (the producer warp contributes nothing).
 template <int M>
 __device__ __forceinline__ void block_sum_to(const float (&v)[M], double* out) {
-  __shared__ double red[kConsumerWarps][M];
+  __shared__ PairSum red[kConsumerWarps][M];
   const int w = threadIdx.x >> 5;
-  if (w < kConsumerWarps) warp_sums<M>(v, [&](int j, double x) { red[w][j] = x; });
+  if (w < kConsumerWarps) warp_sums<M>(v, [&](int j, PairSum x) { red[w][j] = x; });
   __syncthreads();
   for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    double s = 0.0;
-    for (int q = 0; q < kConsumerWarps; ++q) s += red[q][j];
-    out[j] = s;
+    PairSum s;
+    for (int q = 0; q < kConsumerWarps; ++q) s = pair_add(s, red[q][j]);
+    out[j] = s.value();
   }
 }
 
+// The sums over the `groups` partial rows, row j by one warp; fin(j, sum) on its lane 0.
 template <class F>
-__device__ __forceinline__ void final_sum(const double* partials, int M, F fin) {
+__device__ __forceinline__ void final_sum(const double* partials, int groups, int M, F fin) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = blockDim.x >> 5;
   for (int j = w; j < M; j += nw) {
     double s = 0.0;
-    for (int b = lane; b < (int)gridDim.x; b += 32) s += partials[(size_t)b * kPartialStride + j];
+    for (int b = lane; b < groups; b += 32) s += partials[(size_t)b * kPartialStride + j];
     s = warp_sum(s);
     if (lane == 0) fin(j, s);
   }
@@ -156,7 +163,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
                                                           long long n, long long ob2, long long ob1,
                                                           double* partials, unsigned int* counter,
                                                           unsigned int* flags, RpropCfg<float> rc, float slope,
-                                                          int no_loads, const void* const* tab) {
+                                                          int groups, int per_cta, int no_loads,
+                                                          const void* const* tab) {
   using S = Stage<H, W2>;
   const WMaps* mp = &maps;
   rebind(tab, mp, theta, step, vec, hidv, pre, dpre_io, pre_out, hid_out, scal, partials, counter, flags);
@@ -167,13 +175,19 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
   constexpr int kStages = S::kStages;
   __shared__ __align__(8) uint64_t full[kMaxStages], empty[kMaxStages];
   __shared__ float hs[H];
-  __shared__ int s_fail;
+  __shared__ volatile int s_fail;
+  __shared__ int s_stop;
+  constexpr int RPT = (H + kGroups - 1) / kGroups;  // rows per consumer thread
+  __shared__ PairSum red[kGroups * kConsumerWarps][RPT + 1];
   // ob2: offset of b2 in theta and step, < 0 when this launch leaves b2 alone (W2 pass);
   // ob1: offset of b1, < 0 when the W2 pass only writes dpre (the caller updates b1)
   const bool with_b2 = W2 && ob2 >= 0;
   const uint32_t tx = with_b2 ? S::kTx : (uint32_t)S::kBw;  // bytes one chunk's copies bring in
-  const long long nchunks = n / kCols;
-  const long long nk = blockIdx.x < nchunks ? (nchunks - 1 - blockIdx.x) / gridDim.x + 1 : 0;  // chunks of this CTA
+  const int nchunks = (int)(n / kCols);
+  const int g0 = (int)blockIdx.x * per_cta, g1 = min(g0 + per_cta, groups);  // this CTA's groups
+  auto chunks_of = [&](int g) { return (nchunks - 1 - g) / groups + 1; };      // groups <= nchunks
+  int nk = 0;
+  for (int g = g0; g < g1; ++g) nk += chunks_of(g);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid < H) hs[tid] = W2 ? hidv[tid] : dpre_io[tid];  // W2: h; W1: dpre
   if (tid == 0) {
@@ -186,7 +200,6 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
   }
   __syncthreads();
 
-  constexpr int RPT = (H + kGroups - 1) / kGroups;  // rows per consumer thread
   const int col = tid % kCols, rg = tid / kCols;      // column of a chunk, row group
   float acc[RPT], accf = 0.f, hr[RPT];
 #pragma unroll
@@ -201,10 +214,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
         tensormap_acquire(&mp->w);
         tensormap_acquire(&mp->st);
       }
-      auto issue_loads = [&](long long k) {
-        const int q = (int)(k % kStages);
+      // the CTA's chunks in order: group by group, each group's chunks `groups` apart
+      struct Walk {
+        int g, c;
+      } wl{g0, g0}, ws{g0, g0};
+      auto next = [&](Walk& w) {
+        const long long c0 = (long long)w.c * kCols;
+        w.c += groups;
+        if (w.c >= nchunks) w.c = ++w.g;
+        return c0;
+      };
+      auto issue_loads = [&](int k) {
+        const int q = k % kStages;
         uint8_t* st = smem + q * S::kBytes;
-        const long long c0 = (blockIdx.x + k * gridDim.x) * kCols;
+        const long long c0 = next(wl);
         const uint32_t bar = s_u32(&full[q]);
         bar_expect(bar, tx);
         tma_load_box(st + S::kW, &mp->w, (int)c0, bar);
@@ -215,10 +238,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
           bulk_load(st + S::kBst, step + ob2 + c0, kCols * 4, bar);
         }
       };
-      auto issue_stores = [&](long long k) {
-        const int q = (int)(k % kStages);
+      auto issue_stores = [&](int k) {
+        const int q = k % kStages;
         uint8_t* st = smem + q * S::kBytes;
-        const long long c0 = (blockIdx.x + k * gridDim.x) * kCols;
+        const long long c0 = next(ws);
         tma_store_box(&mp->w, (int)c0, st + S::kW);
         tma_store_box(&mp->st, (int)c0, st + S::kSt);
         if (with_b2) {
@@ -227,11 +250,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
         }
         bulk_commit();
       };
-      long long loaded = 0;  // chunks [0, loaded) have been issued
+      int loaded = 0;  // chunks [0, loaded) have been issued
       // no_loads (qst_inject_wait_timeout): issue nothing, so that every bounded wait of the pass runs out
-      const long long nload = no_loads ? 0 : nk;
+      const int nload = no_loads ? 0 : nk;
       for (; loaded < nload && loaded < kStages; ++loaded) issue_loads(loaded);
-      for (long long k = 0; k < nk; ++k) {
+      for (int k = 0; k < nk; ++k) {
         if (!bar_wait(s_u32(&empty[k % kStages]), (uint32_t)((k / kStages) & 1))) {
           atomicOr(flags, 4u);
           s_fail = 1;
@@ -247,8 +270,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
       bulk_wait_all();
       if (s_fail) {  // drain: wait (bounded) for the last load issued into every stage
         for (int q = 0; q < kStages; ++q) {
-          long long last = -1;
-          for (long long k = loaded - 1; k >= 0 && k >= loaded - kStages; --k)
+          int last = -1;
+          for (int k = loaded - 1; k >= 0 && k >= loaded - kStages; --k)
             if (k % kStages == q) last = k;
           if (last >= 0) bar_wait(s_u32(&full[q]), (uint32_t)((last / kStages) & 1));
         }
@@ -257,75 +280,81 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
     __syncwarp();
   } else {
     // ---------------- consumers: column col, rows rg * RPT + l, of every chunk
-    for (long long k = 0; k < nk; ++k) {
-      const int q = (int)(k % kStages);
-      if (!bar_wait(s_u32(&full[q]), (uint32_t)((k / kStages) & 1))) {
-        if (tid == 0) atomicOr(flags, 4u);
-        s_fail = 1;
-        break;
-      }
-      uint8_t* st = smem + q * S::kBytes;
-      float* w = reinterpret_cast<float*>(st + S::kW);
-      float* sp = reinterpret_cast<float*>(st + S::kSt);
-      const float v = reinterpret_cast<const float*>(st + S::kVec)[col];  // dt_i or f_i
-      if (rg == 0) {
-        if (with_b2) {
-          float* bw = reinterpret_cast<float*>(st + S::kBw);
-          float* bst = reinterpret_cast<float*>(st + S::kBst);
-          float bs = bst[col];
-          bw[col] = rprop1(bw[col], v, bs, rc);
-          bst[col] = bs;
-        } else if (!W2) {
-          accf += v;
+    // A thread whose wait runs out takes no more chunks but comes to the group's barriers like the others; the group
+    // is the last one then (s_stop, set between the two barriers, so that all leave together).
+    int k = 0;
+    bool late = false;
+    for (int g = g0; g < g1; ++g) {
+      for (int c = g; c < nchunks; c += groups, ++k) {
+        const int q = k % kStages;
+        if (late || !bar_wait(s_u32(&full[q]), (uint32_t)((k / kStages) & 1))) {
+          if (!late && tid == 0) atomicOr(flags, 4u);
+          late = true;
+          s_fail = 1;
+          continue;
         }
-      }
+        uint8_t* st = smem + q * S::kBytes;
+        float* w = reinterpret_cast<float*>(st + S::kW);
+        float* sp = reinterpret_cast<float*>(st + S::kSt);
+        const float v = reinterpret_cast<const float*>(st + S::kVec)[col];  // dt_i or f_i
+        if (rg == 0) {
+          if (with_b2) {
+            float* bw = reinterpret_cast<float*>(st + S::kBw);
+            float* bst = reinterpret_cast<float*>(st + S::kBst);
+            float bs = bst[col];
+            bw[col] = rprop1(bw[col], v, bs, rc);
+            bst[col] = bs;
+          } else if (!W2) {
+            accf += v;
+          }
+        }
 #pragma unroll
-      for (int l = 0; l < RPT; ++l) {
-        const int j = rg * RPT + l;
-        if (RPT * kGroups != H && j >= H) continue;
-        const int e = j * kCols + col;
-        float wj = w[e];
-        float sj = sp[e];
-        if (W2) {
-          acc[l] += wj * v;  // dh_j with the old weights
-          wj = rprop1(wj, hr[l] * v, sj, rc);
-        } else {
-          wj = rprop1(wj, hr[l] * v, sj, rc);
-          acc[l] += wj * v;  // next pre-activation with the new weights
+        for (int l = 0; l < RPT; ++l) {
+          const int j = rg * RPT + l;
+          if (RPT * kGroups != H && j >= H) continue;
+          const int e = j * kCols + col;
+          float wj = w[e];
+          float sj = sp[e];
+          if (W2) {
+            acc[l] += wj * v;  // dh_j with the old weights
+            wj = rprop1(wj, hr[l] * v, sj, rc);
+          } else {
+            wj = rprop1(wj, hr[l] * v, sj, rc);
+            acc[l] += wj * v;  // next pre-activation with the new weights
+          }
+          w[e] = wj;
+          sp[e] = sj;
         }
-        w[e] = wj;
-        sp[e] = sj;
+        fence_async_smem();  // the producer's tensor stores read what this thread wrote
+        bar_arrive(s_u32(&empty[q]));
       }
-      fence_async_smem();  // the producer's tensor stores read what this thread wrote
-      bar_arrive(s_u32(&empty[q]));
+      // the group's sums: per row the thread partials of its kCols columns, per warp, then over the row group's
+      // kConsumerWarps warps in order (the partition of k_l1_forward_cols)
+      warp_sums<RPT>(acc, [&](int l, PairSum x) { red[warp][l] = x; });
+      if (!W2 && rg == 0) {
+        const float one[1] = {accf};
+        warp_sums<1>(one, [&](int, PairSum x) { red[warp][RPT] = x; });
+      }
+      consumers_sync();
+      if (tid == 0) s_stop = s_fail;
+      if (tid < (W2 ? H : H + 1)) {
+        const int gr = tid < H ? tid / RPT : 0, l = tid < H ? tid % RPT : RPT;
+        PairSum sum;
+        for (int q = 0; q < kConsumerWarps; ++q) sum = pair_add(sum, red[gr * kConsumerWarps + q][l]);
+        partials[(size_t)g * kPartialStride + tid] = sum.value();
+      }
+      consumers_sync();
+      if (s_stop) break;
+#pragma unroll
+      for (int l = 0; l < RPT; ++l) acc[l] = 0.f;
+      accf = 0.f;
     }
   }
   __syncthreads();
   if (s_fail) return;
-
-  // per row j: the thread partials of its group's kCols columns, summed per warp (FP64) and over the
-  // group's kConsumerWarps warps in order (the partition of k_l1_forward_cols)
-  {
-    __shared__ double red[kGroups * kConsumerWarps][RPT + 1];
-    if (warp < kConsumers / 32) {
-      warp_sums<RPT>(acc, [&](int l, double x) { red[warp][l] = x; });
-      if (!W2 && rg == 0) {
-        const double x = warp_sum((double)accf);
-        if (lane == 0) red[warp][RPT] = x;
-      }
-    }
-    __syncthreads();
-    double* out = partials + (size_t)blockIdx.x * kPartialStride;
-    for (int j = tid; j < (W2 ? H : H + 1); j += blockDim.x) {
-      const int g = j < H ? j / RPT : 0, l = j < H ? j % RPT : RPT;
-      double sum = 0.0;
-      for (int q = 0; q < kConsumerWarps; ++q) sum += red[g * kConsumerWarps + q][l];
-      out[j] = sum;
-    }
-  }
   if (last_block_arrived(counter)) {
     if (W2) {
-      final_sum(partials, H, [&](int j, double sum) {
+      final_sum(partials, groups, H, [&](int j, double sum) {
         const float p = pre[j];
         const float dp = (float)sum * (p > 0.f ? 1.f : slope);
         dpre_io[j] = dp;
@@ -336,7 +365,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
         }
       });
     } else {
-      final_sum(partials, H + 1, [&](int j, double sum) {
+      final_sum(partials, groups, H + 1, [&](int j, double sum) {
         if (j < H) {
           const float p = (float)(sum + (double)theta[ob1 + j]);
           pre_out[j] = p;
@@ -351,8 +380,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
   }
 }
 
-// Layer-1 forward with exactly the partition of the bulk W1 pass (chunk c of the 4^N axis to block
-// c mod grid, column t of a chunk to thread t), so that the hidden layer it gives is bit-identical to
+// Layer-1 forward with exactly the partition of the bulk W1 pass (block g the chunks of group g, column t of a chunk to thread t), so that the hidden layer it gives is bit-identical to
 // the one the W1 pass leaves for the next iteration (checkpoint resume depends on this).
 template <int H>
 __global__ void __launch_bounds__(kCols, 2) k_l1_forward_cols(const float* __restrict__ theta,
@@ -373,7 +401,7 @@ __global__ void __launch_bounds__(kCols, 2) k_l1_forward_cols(const float* __res
   }
   block_sum_to<H + 1>(acc, partials + (size_t)blockIdx.x * kPartialStride);
   if (last_block_arrived(counter)) {
-    final_sum(partials, H + 1, [&](int j, double sum) {
+    final_sum(partials, (int)gridDim.x, H + 1, [&](int j, double sum) {
       if (j < H) {
         const float p = (float)(sum + (double)theta[ob1 + j]);
         pre[j] = p;
@@ -387,14 +415,13 @@ __global__ void __launch_bounds__(kCols, 2) k_l1_forward_cols(const float* __res
   }
 }
 
-long long bulk_grid(long long n) {
+// Groups of the 4^N axis: at most one per SM, of at least bulk_chunks_per_cta chunks.
+long long bulk_groups(long long n) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   long long grid = (long long)kCtasPerSm * sms;
   const long long nchunks = n / kCols;
-  // at least bulk_chunks_per_cta chunks per CTA: a CTA's ring fill and store drain are then a small
-  // share of its time, and a batch of small tomographies keeps few CTAs per tomography
   const long long per = tuning().bulk_chunks_per_cta;
   const long long want = nchunks / per < 1 ? 1 : nchunks / per;
   if (grid > want) grid = want;
@@ -438,15 +465,21 @@ template <int H, bool W2> cudaError_t launch_bulk(float* theta, float* step, con
   WMaps maps;
   if (!make_rows_map(&maps.w, theta + rowoff, n, H) || !make_rows_map(&maps.st, step + rowoff, n, H))
     return cudaErrorInvalidValue;
-  const long long grid = bulk_grid(n);
+  const int groups = (int)bulk_groups(n);
   BatchArgs ba;
   if (batch_take(ba, {theta, step, vec, hid, pre, dpre, pre_out, hid_out, scal, partials, counter, flags}, &maps,
                  sizeof(WMaps)))
     return cudaSuccess;
   const int no_loads = inject_take(INJ_WPASS_LOADS) ? 1 : 0;
-  return launch_dep(k_wpass_bulk<H, W2>, dim3((unsigned)grid, 1, ba.nz), dim3(kThreads), (size_t)smem, s, maps, theta,
-                    step, vec, hid, pre, dpre, pre_out, hid_out, scal, n, ob2, ob1, partials, counter, flags, rc,
-                    slope, no_loads, ba.tab);
+  // A batch's members share the GPU: about two CTAs per SM in all, each with several groups (a CTA's ring fill and
+  // store drain are then a small share of its time).
+  int per_cta = 1;
+  if (ba.nz > 1) per_cta = (int)((long long)groups * ba.nz + 2 * 152 - 1) / (2 * 152);
+  if (per_cta > groups) per_cta = groups;
+  const unsigned grid = (unsigned)((groups + per_cta - 1) / per_cta);
+  return launch_dep(k_wpass_bulk<H, W2>, dim3(grid, 1, ba.nz), dim3(kThreads), (size_t)smem, s, maps, theta, step, vec,
+                    hid, pre, dpre, pre_out, hid_out, scal, n, ob2, ob1, partials, counter, flags, rc, slope, groups,
+                    per_cta, no_loads, ba.tab);
 }
 
 }  // namespace
@@ -492,7 +525,7 @@ cudaError_t w2_rows_pass_bulk(long long n, int rows, float* theta, float* step, 
 
 cudaError_t l1_forward_bulk(const Dims& D, const float* theta, const float* f, float* pre, float* hid, double* scal,
                             double* partials, unsigned int* counter, const NetCfg& c, cudaStream_t s) {
-  const long long grid = bulk_grid(D.n);
+  const long long grid = bulk_groups(D.n);
   QST_BULK_SWITCH(D.H, k_l1_forward_cols<HH><<<(unsigned)grid, kCols, 0, s>>>(theta, f, D.n, pre, hid, scal, partials,
                                                                               counter, (float)c.slope));
   return cudaGetLastError();

@@ -66,13 +66,14 @@ static_assert(sizeof(Smem) % 16 == 0 && 2 * (kFusedSmem + 1024) <= 227 * 1024, "
 constexpr int kTot = 31 * 16;
 template <int M> __device__ void block_sum(const float (&v)[M], double* red) {
   static_assert(M <= 16, "at most 16 values per reduction");
+  PairSum* pr = reinterpret_cast<PairSum*>(red);  // (a pair has the size of a double)
   const int warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-  warp_sums<M>(v, [&](int j, double s) { red[warp * 16 + j] = s; });
+  warp_sums<M>(v, [&](int j, PairSum s) { pr[warp * 16 + j] = s; });
   __syncthreads();
   if (threadIdx.x < M) {
-    double s = 0.0;
-    for (int w = 0; w < nw; ++w) s += red[w * 16 + threadIdx.x];
-    red[kTot + threadIdx.x] = s;  // warps <= 16 leave the last row free
+    PairSum s;
+    for (int w = 0; w < nw; ++w) s = pair_add(s, pr[w * 16 + threadIdx.x]);
+    red[kTot + threadIdx.x] = s.value();  // warps <= 16 leave the last row free
   }
   __syncthreads();
 }
