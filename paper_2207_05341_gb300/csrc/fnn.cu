@@ -219,7 +219,9 @@ __global__ void __launch_bounds__(256, 2) k_w2_pass(R* __restrict__ theta, R* __
                                                   RpropCfg<R> rc, R slope) {
   using VV = Vec<R>;
   constexpr int VW = VV::W;
-  constexpr int JB = kRowBatch;  // rows whose loads are issued together, ahead of their updates
+  // rows whose loads are issued together, ahead of their updates; the gradient form, which loads no state words,
+  // takes half of them at once
+  constexpr int JB = UPD ? kRowBatch : (H + 1) / 2;
   const long long o2 = (long long)H * n, ob2 = 2LL * H * n, ob1 = 2LL * H * n + n;
   __shared__ R hs[H];
   if (threadIdx.x < H) hs[threadIdx.x] = hid[threadIdx.x];

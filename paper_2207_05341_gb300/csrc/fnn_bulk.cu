@@ -388,12 +388,28 @@ __global__ void __launch_bounds__(kCols, 2) k_l1_forward_cols(const float* __res
                                                               float* hid, double* scal, double* partials,
                                                               unsigned int* counter, float slope) {
   const long long ob1 = 2LL * H * n + n;
-  const long long nchunks = n / kCols;
   float acc[H + 1];
 #pragma unroll
   for (int j = 0; j <= H; ++j) acc[j] = 0.f;
-  for (long long chunk = blockIdx.x; chunk < nchunks; chunk += gridDim.x) {
-    const long long c = chunk * kCols + threadIdx.x;
+  // two chunks' loads in flight per thread (one left 3.6 TB/s of latency-bound reads); added one after the other
+  const long long step = (long long)gridDim.x * kCols;
+  long long c = (long long)blockIdx.x * kCols + threadIdx.x;
+  for (; c + step < n; c += 2 * step) {
+    float w0[H], w1[H];
+    const float v0 = f[c], v1 = f[c + step];
+#pragma unroll
+    for (int j = 0; j < H; ++j) {
+      w0[j] = theta[(long long)j * n + c];
+      w1[j] = theta[(long long)j * n + c + step];
+    }
+    acc[H] += v0;
+#pragma unroll
+    for (int j = 0; j < H; ++j) acc[j] += w0[j] * v0;
+    acc[H] += v1;
+#pragma unroll
+    for (int j = 0; j < H; ++j) acc[j] += w1[j] * v1;
+  }
+  if (c < n) {
     const float v = f[c];
     acc[H] += v;
 #pragma unroll
