@@ -334,7 +334,7 @@ qst_status qst_graph_enable(qst_ctx* ctx, int enable);
  *   bulk_chunks_per_cta  least number of 256-column chunks in a group of an FP32 weight pass (and of
  *                        the layer-1 forward that shares its partition), >= 1; there are at most as many
  *                        groups as SMs.  A single tomography runs a CTA per group, a batch CTAs that walk
- *                        several.  The groups fix how the passes' sums over 4^N terms are split, so results
+ *                        several.  (QST_MAP_ABS_P: at least 32 chunks.)  The groups fix how the passes' sums over 4^N terms are split, so results
  *                        change in the last bits with it.
  *   fused_ctas_per_sm    resident CTAs per SM of the persistent launch of a batch's fused tomographies
  *                        (1 or 2); results do not depend on it.

@@ -1467,6 +1467,9 @@ qst_status qst_init(qst_ctx** out, int N, const double* povm, int K, const qst_o
   c->net.eta_plus = o.eta_plus;
   c->net.step_min = o.step_min;
   c->net.step_max = o.step_max;
+  // The A_P map carries the last bit of a hidden unit to about 2e-5 of rho at N = 9 (FP32 eigenvectors of close
+  // eigenvalues): the split of its layer-1 sums stays as long as it has been, whatever suits the other maps.
+  if (o.mapping == QST_MAP_ABS_P) c->net.least_chunks = 32;
   cudaGetDevice(&c->device);
   cudaError_t e = cudaMallocHost((void**)&c->h_scal, 16 * sizeof(double));
   if (e == cudaSuccess) e = cudaMallocHost((void**)&c->h_flags, 8 * sizeof(unsigned int));

@@ -431,14 +431,14 @@ __global__ void __launch_bounds__(kCols, 2) k_l1_forward_cols(const float* __res
   }
 }
 
-// Groups of the 4^N axis: at most one per SM, of at least bulk_chunks_per_cta chunks.
-long long bulk_groups(long long n) {
+// Groups of the 4^N axis: at most one per SM, of at least bulk_chunks_per_cta (and `least`) chunks.
+long long bulk_groups(long long n, int least) {
   int dev = 0, sms = 152;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   long long grid = (long long)kCtasPerSm * sms;
   const long long nchunks = n / kCols;
-  const long long per = tuning().bulk_chunks_per_cta;
+  const long long per = tuning().bulk_chunks_per_cta > least ? tuning().bulk_chunks_per_cta : least;
   const long long want = nchunks / per < 1 ? 1 : nchunks / per;
   if (grid > want) grid = want;
   if (grid > kPartialBlocks) grid = kPartialBlocks;
@@ -469,7 +469,7 @@ template <int H, bool W2> cudaError_t launch_bulk(float* theta, float* step, con
                                                    float* hid_out, double* scal, long long n, long long rowoff,
                                                    long long ob2, long long ob1, double* partials,
                                                    unsigned int* counter, unsigned int* flags,
-                                                   const RpropCfg<float>& rc, float slope, cudaStream_t s) {
+                                                   const RpropCfg<float>& rc, float slope, int least, cudaStream_t s) {
   using S = Stage<H, W2>;
   const int smem = S::kStages * S::kBytes + 128;
   static bool set = false;
@@ -481,7 +481,7 @@ template <int H, bool W2> cudaError_t launch_bulk(float* theta, float* step, con
   WMaps maps;
   if (!make_rows_map(&maps.w, theta + rowoff, n, H) || !make_rows_map(&maps.st, step + rowoff, n, H))
     return cudaErrorInvalidValue;
-  const int groups = (int)bulk_groups(n);
+  const int groups = (int)bulk_groups(n, least);
   BatchArgs ba;
   if (batch_take(ba, {theta, step, vec, hid, pre, dpre, pre_out, hid_out, scal, partials, counter, flags}, &maps,
                  sizeof(WMaps)))
@@ -525,7 +525,7 @@ cudaError_t w2_pass_bulk(const Dims& D, float* theta, float* step, const float* 
   const long long n = D.n, H = D.H;  // theta = [W1 | W2^T | b2 | b1]
   QST_BULK_SWITCH(D.H, return (launch_bulk<HH, true>(theta, step, dt, hid, pre, dpre, nullptr, nullptr, nullptr,
                                                      n, H * n, 2 * H * n, 2 * H * n + n, partials, counter, flags, rc,
-                                                     (float)c.slope, s)));
+                                                     (float)c.slope, 0, s)));
   return cudaSuccess;
 }
 
@@ -535,13 +535,13 @@ cudaError_t w2_rows_pass_bulk(long long n, int rows, float* theta, float* step, 
   RpropCfg<float> rc{(float)c.eta_minus, (float)c.eta_plus, (float)c.step_min, (float)c.step_max};
   QST_BULK_SWITCH(rows, return (launch_bulk<HH, true>(theta, step, dt, hid, pre, dpre, nullptr, nullptr, nullptr, n,
                                                       rowoff, ob2, -1, partials, counter, flags, rc, (float)c.slope,
-                                                      s)));
+                                                      0, s)));
   return cudaSuccess;
 }
 
 cudaError_t l1_forward_bulk(const Dims& D, const float* theta, const float* f, float* pre, float* hid, double* scal,
                             double* partials, unsigned int* counter, const NetCfg& c, cudaStream_t s) {
-  const long long grid = bulk_groups(D.n);
+  const long long grid = bulk_groups(D.n, c.least_chunks);
   QST_BULK_SWITCH(D.H, k_l1_forward_cols<HH><<<(unsigned)grid, kCols, 0, s>>>(theta, f, D.n, pre, hid, scal, partials,
                                                                               counter, (float)c.slope));
   return cudaGetLastError();
@@ -554,7 +554,7 @@ cudaError_t w1_pass_bulk(const Dims& D, float* theta, float* step, const float* 
   const long long n = D.n, H = D.H;
   QST_BULK_SWITCH(D.H, return (launch_bulk<HH, false>(theta, step, f, nullptr, nullptr, dpre, pre, hid, scal, n, 0,
                                                       -1, 2 * H * n + n, partials, counter, flags, rc,
-                                                      (float)c.slope, s)));
+                                                      (float)c.slope, c.least_chunks, s)));
   return cudaSuccess;
 }
 

@@ -155,6 +155,7 @@ constexpr int kPartialStride = 32;     // doubles per block in `partials` (>= H 
 struct NetCfg {
   double slope;
   double eta_minus, eta_plus, step_min, step_max;
+  int least_chunks = 0;  // a group of the layer-1 sums has at least this many chunks (and the tuned least)
 };
 
 // ---- POVM map (povm.cu) ----
