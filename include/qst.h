@@ -277,8 +277,9 @@ long long qst_iterations(const qst_ctx* ctx);
  * coupling relative to max |lambda|. */
 qst_status qst_eig_counts(const qst_ctx* ctx, long long* refinements, long long* fallbacks, double* last);
 
-/* The ordering of the Jacobi eigensolver behind QST_MAP_ABS_P and qst_state_fidelity (Sec. 3.2,
- * eq. abs_P; inspection only, no GPU needed): for d = 2^N, round m of a sweep rotates the index pairs
+/* The ordering of the Jacobi eigensolver behind QST_MAP_ABS_P (Sec. 3.2, eq. abs_P) and, but for N = 9, 10
+ * and 11, where it takes another partition of the same rounds, qst_state_fidelity (inspection only, no GPU
+ * needed): for d = 2^N, round m of a sweep rotates the index pairs
  * {x, x ^ m}, m = 1 .. d - 1, and each pass applies the 2^k - 1 rounds of one k-dimensional subspace of
  * GF(2)^N (its nonzero elements; they act within the subspace's cosets of 2^k indices), k = 1 .. 4: a
  * partition of GF(2)^N \ {0} into such subspaces is one sweep.  count = passes per sweep; for the first
@@ -334,8 +335,9 @@ qst_status qst_graph_enable(qst_ctx* ctx, int enable);
  *   bulk_chunks_per_cta  least number of 256-column chunks in a group of an FP32 weight pass (and of
  *                        the layer-1 forward that shares its partition), >= 1; there are at most as many
  *                        groups as SMs.  A single tomography runs a CTA per group, a batch CTAs that walk
- *                        several.  (QST_MAP_ABS_P: at least 32 chunks.)  The groups fix how the passes' sums over 4^N terms are split, so results
- *                        change in the last bits with it.
+ *                        several.  The groups fix how the passes' sums over 4^N terms are split, so
+ *                        results change in the last bits with it.  (A QST_MAP_ABS_P context has at least
+ *                        32 chunks in a group of its layer-1 sums.)
  *   fused_ctas_per_sm    resident CTAs per SM of the persistent launch of a batch's fused tomographies
  *                        (1 or 2); results do not depend on it.
  *   fused_max_qubits     the limit qst_options.fused_max_qubits = 0 stands for (0..7; 0 = never).

@@ -1058,7 +1058,7 @@ template <class R> struct Engine {
     if (!absp) {
       const int sw = (sweeps > 0 ? sweeps : c->sweeps) + ((sweeps > 0 ? sweeps : c->sweeps) & 1);
       QST_CU(jacobi_values_project<R>(D.d, w->T, ap, sw, 2.0, psi, phi, c->stream));
-      c->launches += 1 + (long long)sw * jacobi_kernels_per_sweep(D.d);
+      c->launches += 1 + (long long)sw * jacobi_kernels_per_sweep(D.d, true);
     }
     double* out = w->scal + 8;
     QST_CU(state_fidelity_from_decomposition<R>(D.d, absp ? ap.Qh : nullptr, phi, ap.s, psi, wgt, c->fq, out,

@@ -752,8 +752,9 @@ int blocks_for(long long n) {
 // N >= 6 subspaces of dimension 3 and 4 (8- and 16-index cosets), the lift sizes chosen for the fewest passes.
 using Basis = std::vector<int>;
 
-int gf_mul(int k, int a, int b) {  // GF(2^k), moduli x^2 + x + 1, x^3 + x + 1, x^4 + x + 1
-  static const int kMod[5] = {0, 0, 0x7, 0xB, 0x13};
+// GF(2^k), moduli x^2 + x + 1, x^3 + x + 1, x^4 + x + 1, x^5 + x^2 + 1, x^6 + x + 1, x^7 + x + 1
+int gf_mul(int k, int a, int b) {
+  static const int kMod[8] = {0, 0, 0x7, 0xB, 0x13, 0x25, 0x43, 0x83};
   int r = 0;
   for (int i = 0; i < k; ++i)
     if ((b >> i) & 1) r ^= a << i;
@@ -848,6 +849,29 @@ std::vector<JacobiPass> build_schedule(int N) {
   return out;
 }
 
+// The partition used where no eigenvectors are wanted, 9 <= N <= 11: the graphs u -> (u, c iota(u)) of V(4) in
+// GF(2^k), k = N - 4 (dimension 4, one for each c), and V(k) partitioned as above, so nearly every pass applies 15
+// rounds: 41, 73 and 145 passes a sweep where the lifts by at most 4 dimensions above take 73, 145 and 273 (N = 8 and
+// 12 are 16-index passes throughout either way).  A pass is a chain of latencies (launch, loads, the rounds' rotations
+// one after another) more than work, so half the passes at twice the work each is faster: a state fidelity at FP32
+// N = 9, 10 and 11 7.5, 21.2 and 108.5 ms with A_P's partition, 6.4, 19.0 and 90.2 ms with this one.  A_P keeps its
+// order: its FP32 states follow the last bit of every rotation.
+std::vector<JacobiPass> build_values_schedule(int N) {
+  if (N < 9 || N > 11) return build_schedule(N);
+  const int k = N - 4;
+  std::vector<JacobiPass> out;
+  for (int c = 0; c < (1 << k); ++c) {
+    Basis b;
+    for (int i = 0; i < 4; ++i) b.push_back((1 << i) | (gf_mul(k, c, 1 << i) << 4));
+    out.push_back(make_pass(b));
+  }
+  for (Basis b : subspace_partition(k, 4)) {
+    for (int& v : b) v <<= 4;
+    out.push_back(make_pass(b));
+  }
+  return out;
+}
+
 constexpr int kMaxScheduleN = 14;
 
 template <class R, int G, int TS>
@@ -879,7 +903,7 @@ cudaError_t tile_pass(int d, const JacobiPass& p, const cx_t<R>* A, cx_t<R>* Ao,
 template <class R>
 cudaError_t jacobi_sweep(int d, cx_t<R>*& Ain, cx_t<R>*& Aout, cx_t<R>*& Vin, cx_t<R>*& Vout, cx_t<R>* phi,
                          cx_t<R>* ucos, cudaStream_t s) {
-  const std::vector<JacobiPass>& sched = jacobi_schedule(top_bit(d));
+  const std::vector<JacobiPass>& sched = jacobi_schedule(top_bit(d), Vin == nullptr);
   const int n4 = d / 4, n2 = d / 2;
   const dim3 g4((n4 + 15) / 16, (n4 + 15) / 16), g2((n2 + 15) / 16, (n2 + 15) / 16);
   for (const JacobiPass& p : sched) {
@@ -900,20 +924,23 @@ cudaError_t jacobi_sweep(int d, cx_t<R>*& Ain, cx_t<R>*& Aout, cx_t<R>*& Vin, cx
 
 }  // namespace
 
-const std::vector<JacobiPass>& jacobi_schedule(int N) {
+const std::vector<JacobiPass>& jacobi_schedule(int N, bool values) {
   static const std::vector<std::vector<JacobiPass>> all = [] {
-    std::vector<std::vector<JacobiPass>> v(kMaxScheduleN + 1);
-    for (int n = 1; n <= kMaxScheduleN; ++n) v[n] = build_schedule(n);
+    std::vector<std::vector<JacobiPass>> v(2 * (kMaxScheduleN + 1));
+    for (int n = 1; n <= kMaxScheduleN; ++n) {
+      v[2 * n] = build_schedule(n);
+      v[2 * n + 1] = build_values_schedule(n);
+    }
     return v;
   }();
-  return all[N < 1 ? 1 : (N > kMaxScheduleN ? kMaxScheduleN : N)];
+  return all[2 * (N < 1 ? 1 : (N > kMaxScheduleN ? kMaxScheduleN : N)) + (values ? 1 : 0)];
 }
 
 long long jacobi_passes_per_sweep(int d) { return (long long)jacobi_schedule(top_bit(d)).size(); }
 
-long long jacobi_kernels_per_sweep(int d) {
+long long jacobi_kernels_per_sweep(int d, bool values) {
   long long k = 0;
-  for (const JacobiPass& p : jacobi_schedule(top_bit(d))) k += p.k >= 3 ? 2 : 1;
+  for (const JacobiPass& p : jacobi_schedule(top_bit(d), values)) k += p.k >= 3 ? 2 : 1;
   return k;
 }
 

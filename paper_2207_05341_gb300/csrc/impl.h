@@ -360,9 +360,10 @@ struct JacobiPass {
   int basis[4];
   int piv[4];
 };
-const std::vector<JacobiPass>& jacobi_schedule(int N);  // 1 <= N <= 14
+// values: the order of a decomposition without eigenvectors (other than A_P's for 9 <= N <= 11); 1 <= N <= 14
+const std::vector<JacobiPass>& jacobi_schedule(int N, bool values = false);
 long long jacobi_passes_per_sweep(int d);
-long long jacobi_kernels_per_sweep(int d);  // a pass over cosets of 8 or 16 indices is two kernels
+long long jacobi_kernels_per_sweep(int d, bool values = false);  // a pass over cosets of 8 or 16 indices is two kernels
 // A warm-started step of the mixed path on the Jacobi sweeps: A0 = Q^dag T Q (Q in V0, T as its 6 planes Tb
 // with scale *sT) and X = Q |Lambda|^P Q^dag (lower tiles) on tensor cores, `sweeps` (even) sweeps between;
 // leaves Q in V0 and Q^dag in Qh, as abs_p_forward does.
