@@ -178,6 +178,8 @@ __global__ void __launch_bounds__(256) k_cnn_conv_tiles(const R* __restrict__ f,
   __shared__ R rv[8][kMaps];
   __shared__ int ri[8][kMaps];
   __shared__ double rf[8];
+  grid_dep_wait();
+  after_wait(f, cW, cB, tv, ti, tf);
   const int d = 1 << N, p = d / kGrid;
   const int tx = p / kTW, per_win = tx * (p / kTH);
   const int win = blockIdx.x / per_win, r = blockIdx.x % per_win;
@@ -272,6 +274,8 @@ __global__ void __launch_bounds__(1024) k_cnn_pool(const R* __restrict__ tv, con
                                                    R* vals, const R* __restrict__ W1, const R* __restrict__ b1, int H,
                                                    R* pre, R* hid, R slope, double* scal, unsigned int* counter) {
   __shared__ R sf[kFeat];
+  grid_dep_wait();
+  after_wait(tv, ti, tf, feats, pos, vals, W1, b1, pre, hid, scal, counter);
   const int lane = threadIdx.x & 31, gw = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (gw < kFeat) {
     const int c = gw / (kGrid * kGrid), win = gw % (kGrid * kGrid);
@@ -314,47 +318,78 @@ __global__ void __launch_bounds__(1024) k_cnn_pool(const R* __restrict__ tv, con
   }
 }
 
-// Output layer: t = W2 h + b2, 4 columns per thread, rows in batches of 8 (loads before the FMAs).
-template <class R, int H>
+// Four consecutive reals.  VEC: 16-byte accesses (the pointers are multiples of 16 bytes); a caller's parameters may
+// lie at any real's address, and go one by one.
+template <bool VEC, class R> __device__ __forceinline__ void ld4(const R* p, R (&v)[4]) {
+  if constexpr (!VEC) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) v[u] = p[u];
+  } else if constexpr (sizeof(R) == 4) {
+    const float4 a = *reinterpret_cast<const float4*>(p);
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+  } else {
+    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
+    v[0] = a.x; v[1] = a.y; v[2] = b.x; v[3] = b.y;
+  }
+}
+template <bool VEC, class R> __device__ __forceinline__ void st4(R* p, const R (&v)[4]) {
+  if constexpr (!VEC) {
+#pragma unroll
+    for (int u = 0; u < 4; ++u) p[u] = v[u];
+  } else if constexpr (sizeof(R) == 4) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+    reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
+  }
+}
+bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
+
+// Output layer: t = W2 h + b2, 4 columns per thread, half the rows' loads in flight at once.  Bound by HBM (every
+// weight is read once): what counts is bytes in flight, so the loads are 16 bytes wide and the first batch is on its
+// way before h is staged.  N = 10 FP32 (H = 40, 172 MB): 28.0 us, 6.1 TB/s; 44.2 with 4-byte loads of 8 rows at a time.
+template <class R, int H, bool VEC>
 __global__ void __launch_bounds__(256) k_cnn_output(const R* __restrict__ W2T, const R* __restrict__ b2,
                                                      const R* __restrict__ hid, long long n, R* __restrict__ t,
                                                      unsigned int* amax) {
+  constexpr int JB = H / 2;
   __shared__ R hs[H];
+  grid_dep_wait();
+  after_wait(W2T, b2, hid, t, amax);
+  const long long i = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+  const bool in = i < n;
+  R acc[4], w[JB][4];
+  if (in) {
+    ld4<VEC>(b2 + i, acc);
+#pragma unroll
+    for (int jj = 0; jj < JB; ++jj) ld4<VEC>(W2T + (long long)jj * n + i, w[jj]);
+  }
   if (threadIdx.x < H) hs[threadIdx.x] = hid[threadIdx.x];
   __syncthreads();
   float m = 0.f;
-  for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n / 4; v += (long long)gridDim.x * blockDim.x) {
-    const long long i = v * 4;
-    R acc[4];
+  if (in) {
 #pragma unroll
-    for (int u = 0; u < 4; ++u) acc[u] = b2[i + u];
+    for (int h = 0; h < 2; ++h) {
 #pragma unroll
-    for (int j0 = 0; j0 < H; j0 += 8) {
-      R w[8][4];
+      for (int jj = 0; jj < JB; ++jj)
 #pragma unroll
-      for (int jj = 0; jj < 8; ++jj)
-        if (j0 + jj < H)
+        for (int u = 0; u < 4; ++u) acc[u] += w[jj][u] * hs[h * JB + jj];
+      if (h == 0)
 #pragma unroll
-          for (int u = 0; u < 4; ++u) w[jj][u] = W2T[(long long)(j0 + jj) * n + i + u];
-#pragma unroll
-      for (int jj = 0; jj < 8; ++jj)
-        if (j0 + jj < H)
-#pragma unroll
-          for (int u = 0; u < 4; ++u) acc[u] += w[jj][u] * hs[j0 + jj];
+        for (int jj = 0; jj < JB; ++jj) ld4<VEC>(W2T + (long long)(JB + jj) * n + i, w[jj]);
     }
+    st4<true>(t + i, acc);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      t[i + u] = acc[u];
-      m = fmaxf(m, fabsf((float)acc[u]));
-    }
+    for (int u = 0; u < 4; ++u) m = fmaxf(m, fabsf((float)acc[u]));
   }
   if (amax) block_absmax_to(m, amax);
 }
 
 // Output-layer backward (Sec. 3.1 layer 2 of the CNN head): db2 = dt, dW2^T[j][i] = h_j dt_i,
 // dh_j = sum_i W2^T[j][i] dt_i (old weights) -> dpre_j = dh_j LeakyReLU'(pre_j) by the last block.
-// UPD: Rprop in place; else the gradient goes to dW2T / db2.
-template <class R, int H, bool UPD>
+// UPD: Rprop in place; else the gradient goes to dW2T / db2 (stores and, with 8 rows of weights on their way at once,
+// loads bound it).
+template <class R, int H, bool UPD, bool VEC>
 __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R* __restrict__ S2T,
                                                           R* __restrict__ b2, R* __restrict__ Sb2,
                                                           const R* __restrict__ dt, const R* __restrict__ hid,
@@ -371,45 +406,50 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
   for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n / 4; v += (long long)gridDim.x * blockDim.x) {
     const long long i = v * 4;
     R g[4];
+    ld4<true>(dt + i, g);
+    if constexpr (UPD) {
+      R b[4], sb[4];
+      ld4<VEC>(b2 + i, b);
+      ld4<VEC>(Sb2 + i, sb);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) g[u] = dt[i + u];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      if (UPD) {
-        R s = Sb2[i + u];
-        b2[i + u] = rprop1(b2[i + u], g[u], s, rc);
-        Sb2[i + u] = s;
-      } else {
-        db2[i + u] = g[u];
-      }
+      for (int u = 0; u < 4; ++u) b[u] = rprop1(b[u], g[u], sb[u], rc);
+      st4<VEC>(b2 + i, b);
+      st4<VEC>(Sb2 + i, sb);
+    } else {
+      st4<VEC>(db2 + i, g);
     }
+    constexpr int JB = (UPD ? 16 : 32) / (int)sizeof(R);  // rows a batch
 #pragma unroll
-    for (int j0 = 0; j0 < H; j0 += 4) {
-      R w[4][4], s[4][4];
+    for (int j0 = 0; j0 < H; j0 += JB) {
+      R w[JB][4], s[UPD ? JB : 1][4];
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj)
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const long long o = (long long)(j0 + jj) * n + i + u;
-          w[jj][u] = W2T[o];
-          if (UPD) s[jj][u] = S2T[o];
+      for (int jj = 0; jj < JB; ++jj)
+        if (j0 + jj < H) {
+          const long long o = (long long)(j0 + jj) * n + i;
+          ld4<VEC>(W2T + o, w[jj]);
+          if constexpr (UPD) ld4<VEC>(S2T + o, s[jj]);
         }
 #pragma unroll
-      for (int jj = 0; jj < 4; ++jj) {
+      for (int jj = 0; jj < JB; ++jj) {
         const int j = j0 + jj;
+        if (j < H) {
+          const long long o = (long long)j * n + i;
+          R gw[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const long long o = (long long)j * n + i + u;
-          acc[j] += w[jj][u] * g[u];
-          const R gw = hs[j] * g[u];
-          if (UPD) {
-            W2T[o] = rprop1(w[jj][u], gw, s[jj][u], rc);
-            S2T[o] = s[jj][u];
+          for (int u = 0; u < 4; ++u) {
+            acc[j] += w[jj][u] * g[u];
+            gw[u] = hs[j] * g[u];
+            if constexpr (UPD) w[jj][u] = rprop1(w[jj][u], gw[u], s[jj][u], rc);
+          }
+          if constexpr (UPD) {
+            st4<VEC>(W2T + o, w[jj]);
+            st4<VEC>(S2T + o, s[jj]);
           } else {
-            dW2T[o] = gw;
+            st4<VEC>(dW2T + o, gw);
           }
         }
       }
+      if constexpr (sizeof(R) == 8) asm volatile("" ::: "memory");  // one batch's loads at a time (spills otherwise)
     }
   }
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
@@ -455,6 +495,8 @@ __global__ void __launch_bounds__(1024) k_cnn_head_grad(const R* __restrict__ f,
   __shared__ R dfeat[kFeat];
   __shared__ R dp[H];
   __shared__ R part[kMaps * 10][10];
+  grid_dep_wait();
+  after_wait(f, pos, vals, dpre, W1, b1, Sb1, cW, ScW, cB, ScB, db1, dcW, dcB);
   const int d = 1 << N, t = threadIdx.x;
   if (t < H) dp[t] = dpre[t];
   __syncthreads();
@@ -525,6 +567,8 @@ template <class R, bool UPD>
 __global__ void __launch_bounds__(256) k_cnn_w1_update(const R* __restrict__ feats, const R* __restrict__ dpre, int H,
                                                         R* __restrict__ W1, R* __restrict__ S1, R* __restrict__ dW1,
                                                         RpropCfg<R> rc) {
+  grid_dep_wait();
+  after_wait(feats, dpre, W1, S1, dW1);
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= H * kFeat) return;
   const R g = dpre[e / kFeat] * feats[e % kFeat];
@@ -608,10 +652,12 @@ cudaError_t cnn_hidden(const Dims& D, const R* theta, const R* f, R* feats, int*
     double* tf = part;
     R* tv = reinterpret_cast<R*>(tf + tiles);
     int* ti = reinterpret_cast<int*>(tv + tiles * kMaps);
-    k_cnn_conv_tiles<R><<<(unsigned)tiles, 256, 0, s>>>(f, D.N, p.cW, p.cB, tv, ti, tf);
+    cudaError_t e = launch_dep(k_cnn_conv_tiles<R>, dim3((unsigned)tiles), dim3(256), 0, s, f, D.N, p.cW, p.cB, tv, ti, tf);
+    if (e != cudaSuccess) return e;
     const int per_win = (int)(tiles / (kGrid * kGrid));
-    k_cnn_pool<R><<<(kFeat + 1 + 31) / 32, 1024, 0, s>>>(tv, ti, tf, per_win, feats, pos, vals, p.W1, p.b1, D.H, pre,
-                                                      hid, (R)slope, scal, counter);
+    e = launch_dep(k_cnn_pool<R>, dim3((kFeat + 1 + 31) / 32), dim3(1024), 0, s, tv, ti, tf, per_win, feats, pos, vals, p.W1,
+                   p.b1, D.H, pre, hid, (R)slope, scal, counter);
+    if (e != cudaSuccess) return e;
   } else {
     k_cnn_features<R><<<kFeat, 256, 0, s>>>(f, D.N, p.cW, p.cB, feats, pos, vals, partials, counter, scal);
     k_cnn_dense1<R><<<1, 1024, 0, s>>>(feats, p.W1, p.b1, D.H, pre, hid, (R)slope);
@@ -623,8 +669,10 @@ template <class R>
 cudaError_t cnn_output(const Dims& D, const R* theta, const R* hid, R* t, unsigned int* amax, cudaStream_t s) {
   CnnParams<R> p = cnn_params(const_cast<R*>(theta), D.H, D.n);
   QST_SWITCH_H4(D.H, {
-    const int grid = resident_grid(k_cnn_output<R, HH>, D.n / 4);
-    k_cnn_output<R, HH><<<grid, 256, 0, s>>>(p.W2T, p.b2, hid, D.n, t, amax);
+    // theta may be a caller's, at any real's address
+    const auto fn = aligned16(theta) ? k_cnn_output<R, HH, true> : k_cnn_output<R, HH, false>;
+    cudaError_t e = launch_dep(fn, dim3((unsigned)((D.n / 4 + 255) / 256)), dim3(256), 0, s, p.W2T, p.b2, hid, D.n, t, amax);
+    if (e != cudaSuccess) return e;
   });
   return cudaGetLastError();
 }
@@ -653,13 +701,15 @@ cudaError_t cnn_output_backward(const Dims& D, R* theta, R* state, R* dtheta, co
   RpropCfg<R> rc{(R)c.eta_minus, (R)c.eta_plus, (R)c.step_min, (R)c.step_max};
   QST_SWITCH_H4(D.H, {
     if (upd) {
-      const int grid = resident_grid(k_cnn_output_back<R, HH, true>, D.n / 4);
-      k_cnn_output_back<R, HH, true><<<grid, 256, 0, s>>>(p.W2T, q.W2T, p.b2, q.b2, dt, hid, pre, dpre, nullptr,
-                                                          nullptr, D.n, partials, counter, rc, (R)c.slope);
-    } else {
-      const int grid = resident_grid(k_cnn_output_back<R, HH, true>, D.n / 4);
-      k_cnn_output_back<R, HH, false><<<grid, 256, 0, s>>>(p.W2T, nullptr, p.b2, nullptr, dt, hid, pre, dpre, g.W2T,
-                                                           g.b2, D.n, partials, counter, rc, (R)c.slope);
+      const int grid = resident_grid(k_cnn_output_back<R, HH, true, true>, D.n / 4);
+      k_cnn_output_back<R, HH, true, true><<<grid, 256, 0, s>>>(p.W2T, q.W2T, p.b2, q.b2, dt, hid, pre, dpre, nullptr,
+                                                                nullptr, D.n, partials, counter, rc, (R)c.slope);
+    } else {  // theta and dtheta may be a caller's, at any real's address
+      const auto fn = aligned16(theta) && aligned16(dtheta) ? k_cnn_output_back<R, HH, false, true>
+                                                            : k_cnn_output_back<R, HH, false, false>;
+      const int grid = resident_grid(k_cnn_output_back<R, HH, true, true>, D.n / 4);
+      fn<<<grid, 256, 0, s>>>(p.W2T, nullptr, p.b2, nullptr, dt, hid, pre, dpre, g.W2T, g.b2, D.n, partials, counter, rc,
+                              (R)c.slope);
     }
   });
   return cudaGetLastError();
@@ -674,19 +724,16 @@ cudaError_t cnn_head_backward(const Dims& D, R* theta, R* state, R* dtheta, cons
   CnnParams<R> g = upd ? CnnParams<R>{} : cnn_params(dtheta, D.H, D.n);
   RpropCfg<R> rc{(R)c.eta_minus, (R)c.eta_plus, (R)c.step_min, (R)c.step_max};
   QST_SWITCH_H4(D.H, {
-    if (upd)
-      k_cnn_head_grad<R, HH, true><<<1, 1024, 0, s>>>(f, D.N, pos, vals, dpre, p.W1, p.b1, q.b1, p.cW, q.cW, p.cB,
-                                                      q.cB, nullptr, nullptr, nullptr, rc);
-    else
-      k_cnn_head_grad<R, HH, false><<<1, 1024, 0, s>>>(f, D.N, pos, vals, dpre, p.W1, p.b1, nullptr, p.cW, nullptr,
-                                                       p.cB, nullptr, g.b1, g.cW, g.cB, rc);
+    const cudaError_t e =
+        upd ? launch_dep(k_cnn_head_grad<R, HH, true>, dim3(1), dim3(1024), 0, s, f, D.N, pos, vals, dpre, p.W1, p.b1, q.b1,
+                         p.cW, q.cW, p.cB, q.cB, nullptr, nullptr, nullptr, rc)
+            : launch_dep(k_cnn_head_grad<R, HH, false>, dim3(1), dim3(1024), 0, s, f, D.N, pos, vals, dpre, p.W1, p.b1,
+                         nullptr, p.cW, nullptr, p.cB, nullptr, g.b1, g.cW, g.cB, rc);
+    if (e != cudaSuccess) return e;
   });
   const int blocks = (D.H * kFeat + 255) / 256;
-  if (upd)
-    k_cnn_w1_update<R, true><<<blocks, 256, 0, s>>>(feats, dpre, D.H, p.W1, q.W1, nullptr, rc);
-  else
-    k_cnn_w1_update<R, false><<<blocks, 256, 0, s>>>(feats, dpre, D.H, p.W1, nullptr, g.W1, rc);
-  return cudaGetLastError();
+  return upd ? launch_dep(k_cnn_w1_update<R, true>, dim3(blocks), dim3(256), 0, s, feats, dpre, D.H, p.W1, q.W1, nullptr, rc)
+             : launch_dep(k_cnn_w1_update<R, false>, dim3(blocks), dim3(256), 0, s, feats, dpre, D.H, p.W1, nullptr, g.W1, rc);
 }
 
 #define QST_CNN_INST(R)                                                                                          \
