@@ -83,8 +83,6 @@ __global__ void __launch_bounds__(128, 1) k_tc_cgemm(const __grid_constant__ TcM
                                                       int no_loads, const void* const* tab) {
   const TcMaps* mp = &maps;
   rebind(tab, mp, C, sA, sB, err, clear);
-  grid_dep_wait();
-  after_wait(mp, C, sA, sB, err, clear);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStages * kStageBytes);
@@ -99,8 +97,7 @@ __global__ void __launch_bounds__(128, 1) k_tc_cgemm(const __grid_constant__ TcM
   else { I = blockIdx.y; J = blockIdx.x; }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  // the max slot behind this product's operand scale was read by the kernel that made the planes
-  if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0u;
+  // barriers and TMEM while the kernel that makes the planes runs
   if (threadIdx.x == 0) {
     s_fail = 0;
     for (int s = 0; s < kStages; ++s) {
@@ -121,6 +118,10 @@ __global__ void __launch_bounds__(128, 1) k_tc_cgemm(const __grid_constant__ TcM
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *tmem_slot;
   const int nkb = 2 * d / kBK;
+  grid_dep_wait();
+  after_wait(mp, C, sA, sB, err, clear);
+  // the max slot behind this product's operand scale was read by the kernel that made the planes
+  if (clear && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *clear = 0u;
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer
@@ -256,6 +257,7 @@ __global__ void __launch_bounds__(256) k_split(const float2* __restrict__ A, H* 
   rebind(tab, A, P, amax, s_slot);
   grid_dep_wait();
   after_wait(A, P, amax, s_slot);
+  asm volatile("griddepcontrol.launch_dependents;");  // the product's prologue may start
   const int se = split_exponent(amax);
   const float sc = pow2f(se);
   if (blockIdx.x == 0 && threadIdx.x == 0) *s_slot = pow2d(se);
@@ -350,6 +352,7 @@ __global__ void __launch_bounds__(256) k_hermitian_planes64(const float* __restr
   rebind(tab, t, P, amax, s_slot);
   grid_dep_wait();
   after_wait(t, P, amax, s_slot);
+  asm volatile("griddepcontrol.launch_dependents;");  // the product's prologue may start
   __shared__ float Ra[64][65];
   __shared__ float Rb[64][65];
   const int se = split_exponent(amax);
