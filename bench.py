@@ -38,8 +38,6 @@ THETA_SEED = 23
 COUNT_SEED = 24
 FID_TARGET = 0.99
 FALLBACK_PEAKS = {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}
-FP32_LANES_PER_SM = 128
-NUM_SMS = 152
 
 
 def workload_name(lam):
@@ -176,9 +174,9 @@ def phase_work(phase, N, mixed):
     if phase == "build_T":
         return "hbm", (H + 1) * 4 * n + (12 if mixed else 8) * n, "B"
     if phase == "x_fwd":
-        return ("tensor" if mixed else "alu"), 4 * d ** 3, "FLOP"
+        return "tensor", 4 * d ** 3, "FLOP"
     if phase == "gt":
-        return ("tensor" if mixed else "alu"), 8 * d ** 3, "FLOP"
+        return "tensor", 8 * d ** 3, "FLOP"
     if phase == "povm_lo":    # lower half of X read, packed intermediate written
         return "hbm", 4 * n + 4 * n, "B"
     if phase == "povm_hi":    # intermediate and f read, packed adjoint written
@@ -807,13 +805,8 @@ def main_ours(args):
         sec = ms / 1e3
         if bound == "hbm":
             achieved, peak, runit = amount / sec / 1e9, peaks["hbm_gbs"], "GB/s"
-        elif bound == "tensor":
-            achieved, peak, runit = amount / sec / 1e12, peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]), "TFLOP/s"
         else:
-            mhz = clk.get("sm_max_mhz") or 2070.0
-            achieved = amount / sec / 1e12
-            peak = NUM_SMS * FP32_LANES_PER_SM * 2 * mhz * 1e6 / 1e12
-            runit = "TFLOP/s"
+            achieved, peak, runit = amount / sec / 1e12, peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]), "TFLOP/s"
         return bound, achieved, peak, runit, achieved / peak
 
     bound, achieved, peak, runit, _ = roof(dom, per[dom])
@@ -858,7 +851,7 @@ def main_ours(args):
         "e2e": {"value": ws * e2e_rate, "unit": UNIT, "h2d_bytes_per_step": 4 * n, "d2h_bytes_per_step": 12},
         "gpu_launches": int(res[head]["launches"]),
         "roofline": {"kernel": dom, "bound": bound, "achieved": achieved, "peak": peak, "unit": runit,
-                     "frac": achieved / peak, "peak_source": peak_src if bound != "alu" else "derived: 152 SMs x 128 FP32 lanes x 2 x max SM clock",
+                     "frac": achieved / peak, "peak_source": peak_src,
                      "traffic": recorded_traffic(dom)},
         "rooflines": rooflines,
         "paths": {name: {"iters_per_s": ws * args.steps / (v["ms"] / 1e3), "ms_per_step": v["ms"] / args.steps,

@@ -77,11 +77,11 @@ typedef enum {
 enum { QST_MAP_CHOL_H = 0, QST_MAP_ABS_P = 1, QST_MAP_CHOL_DELTA = 2 };
 /* Precisions.  QST_FP32 runs the complex d x d products of QST_MAP_CHOL_H and QST_MAP_CHOL_DELTA with N >= 7
  * on tensor cores too, each operand as the exact sum of three BF16 terms (all 24 bits), summed in FP32;
- * where the device or device_memory_limit has no room for those operands, on the CUDA cores.  QST_MIXED runs the two complex d x d products on tensor cores
- * (tcgen05) with each FP32 operand split into FP16 hi + lo after a power-of-two
- * scaling (about 2^-21 relative error); QST_MIXED_BF16 uses a BF16 hi + lo split
- * without scaling (about 2^-16).  Everything else stays FP32 in both.  Mixed
- * modes need N >= 7 (d a multiple of 128). */
+ * where the device or device_memory_limit has no room for those operands, on the CUDA cores.  QST_MIXED
+ * runs the two complex d x d products on tensor cores (tcgen05) with each FP32 operand split into FP16
+ * hi + lo after a power-of-two scaling (about 2^-21 relative error); QST_MIXED_BF16 uses a BF16 hi + lo
+ * split without scaling (about 2^-16).  Everything else stays FP32 in both.  Mixed modes need N >= 7 (d a
+ * multiple of 128). */
 enum { QST_FP64 = 0, QST_FP32 = 1, QST_MIXED = 2, QST_MIXED_BF16 = 3 };
 
 typedef struct qst_options {
@@ -251,7 +251,9 @@ qst_status qst_test_state(qst_ctx* ctx, int kind, double w, void* rho);
  * qst_classical_fidelity) and counts outcome k_s = the smallest k whose running weight exceeds t_s.
  * All integer arithmetic: the counts are exact and reproducible.  counts: device, n int64, written;
  * f: device or NULL, n reals of the context precision, written with counts / shots.  QST_E_INPUT for a
- * P that is not finite, above 1, or all zero.  The first call allocates (n + n / 2048) words of scratch. */
+ * P that is not finite, above 1, or all zero.  The first call allocates (n + n / 2048) words of scratch, and n / 4
+ * ints for a table that shortens the draws' searches where there is room for it (the counts do not
+ * depend on it). */
 qst_status qst_sample_counts(qst_ctx* ctx, const double* P, long long shots, unsigned long long seed,
                              long long* counts, void* f);
 
@@ -279,8 +281,8 @@ qst_status qst_eig_counts(const qst_ctx* ctx, long long* refinements, long long*
 
 /* The ordering of the Jacobi eigensolver behind QST_MAP_ABS_P (Sec. 3.2, eq. abs_P) and, but for N = 9, 10
  * and 11, where it takes another partition of the same rounds, qst_state_fidelity (inspection only, no GPU
- * needed): for d = 2^N, round m of a sweep rotates the index pairs
- * {x, x ^ m}, m = 1 .. d - 1, and each pass applies the 2^k - 1 rounds of one k-dimensional subspace of
+ * needed): for d = 2^N, round m of a sweep rotates the index pairs {x, x ^ m}, m = 1 .. d - 1, and each
+ * pass applies the 2^k - 1 rounds of one k-dimensional subspace of
  * GF(2)^N (its nonzero elements; they act within the subspace's cosets of 2^k indices), k = 1 .. 4: a
  * partition of GF(2)^N \ {0} into such subspaces is one sweep.  count = passes per sweep; for the first
  * min(count, cap) passes, dims[p] = k and basis[4 p .. 4 p + k) the subspace's basis in reduced form (top
@@ -349,9 +351,8 @@ qst_status qst_graph_enable(qst_ctx* ctx, int enable);
  * range (nothing changed). */
 /* Testing hook for the device-side wait limits; it involves no GPU fault.  With what =
  * QST_INJECT_TC_LOADS the next `count` launches of the tensor-core products (QST_MIXED, QST_MIXED_BF16, and
- * QST_FP32 with N >= 7),
- * with QST_INJECT_WPASS_LOADS the next `count` launches of the FP32 bulk weight passes, issue none of
- * their operand copies: the waits for those copies run out after their limit (about 2 s), the kernels
+ * QST_FP32 with N >= 7), with QST_INJECT_WPASS_LOADS the next `count` launches of the FP32 bulk weight
+ * passes, issue none of their operand copies: the waits for those copies run out after their limit (about 2 s), the kernels
  * leave their results unwritten and return, and the call that reads the loss (qst_step, qst_loss_grad,
  * qst_reconstruct) returns QST_E_TIMEOUT; the context stays usable (reload its parameters with
  * qst_set_params: the failed step may have updated some of them).  count = 0 clears.  Process-wide;

@@ -9,7 +9,7 @@ step is the headline workload), which the chunk parameter of the weight passes a
     python -m paper_2207_05341_gb300.autotune [--batch 512] [--steps 10] [--out log.json] [--write]
     python -m paper_2207_05341_gb300.autotune --apply log.json    # store a log's best values (no GPU)
 
-Stage 1 picks bulk_chunks_per_cta (least 256-column chunks per CTA of a weight pass) by the mixed
+Stage 1 picks bulk_chunks_per_cta (least 256-column chunks per group of a weight pass) by the mixed
 batch's time, among the values that keep every guard step within 5 % of its time at the smallest
 value (smaller tomographies run mostly in batches, where few CTAs per tomography pay off); stage 2
 picks fused_max_qubits and fused_ctas_per_sm, stage 3 batch_concurrent_runs, each by the sum of the
@@ -134,7 +134,7 @@ def main(argv=None):
     start = qst.qst_get_tuning()
     log = {"workload": f"{args.batch} tomographies, N ~ U{{3..9}}", "start": start, "stage1": [], "stage2": []}
 
-    # stage 1: chunks per CTA of the weight passes
+    # stage 1: chunks per group of the weight passes
     guard_N = [10, 11]
     guard_ref = None
     best1 = None

@@ -1956,19 +1956,26 @@ qst_status qst_batch_reconstruct(qst_batch* bt, const void* const* f, int iters,
   QST_CU(cudaStreamSynchronize(bt->root));
   if (!rho_out && !final_losses) return QST_OK;
   // every tomography's state and loss are enqueued on its own stream before the first loss is waited for
-  for (int b = 0; b < bt->B; ++b) {
+  int begun = 0;
+  qst_status bad = QST_OK;
+  for (; begun < bt->B; ++begun) {
+    const int b = begun;
     qst_ctx* c = bt->ctx[b];
-    if (!f[b]) return QST_E_INVAL;
-    if (!c->params_set) return QST_E_STATE;
-    const qst_status st = QST_DISPATCH(c, rho_begin(c, f[b], rho_out ? rho_out[b] : nullptr, final_losses != nullptr));
-    if (st < 0) return st;
+    bad = !f[b] ? QST_E_INVAL
+                : !c->params_set
+                      ? QST_E_STATE
+                      : QST_DISPATCH(c, rho_begin(c, f[b], rho_out ? rho_out[b] : nullptr, final_losses != nullptr));
+    if (bad < 0) break;
   }
-  for (int b = 0; final_losses && b < bt->B; ++b) {
+  // where one is refused, those before it are still waited for and have their losses; the first failure is returned
+  qst_status first = QST_OK;
+  for (int b = 0; final_losses && b < begun; ++b) {
     qst_ctx* c = bt->ctx[b];
     const qst_status st = QST_DISPATCH(c, loss_end(c, final_losses + b));
-    if (st < 0) return st;
+    if (st < 0 && first >= 0) first = st;
   }
-  return QST_OK;
+  if (first < 0) return first;
+  return bad < 0 ? bad : QST_OK;
 }
 
 long long qst_batch_kernel_launches(const qst_batch* bt) { return bt ? bt->launches : -1; }

@@ -14,8 +14,9 @@
 // would run one after another, with one read and one write of A and V: A' = U^dag A U and V' = V U with U
 // block-diagonal over the cosets.  N <= 5: lines and single rounds, one kernel per pass (each thread a 4 x 4
 // or 2 x 2 block, the CTA's coset unitaries formed by groups of lanes).  N >= 6: subspaces of dimension 3
-// and 4, two kernels per pass (the coset unitaries, a warp per coset; then 64 x 64 tiles of A and V in
-// shared memory).  At N = 11 and 12 a sweep is 273 passes (2047 / 4095 rounds).
+// and 4, two kernels per pass (the coset unitaries, a thread per pair of entries; then 64 x 64 or 32 x 32
+// tiles of A and V in shared memory).  At N = 11 and 12 a sweep is 273 passes (2047 / 4095 rounds); sweeps
+// without eigenvectors take a partition of their own at N = 9 to 11 (build_values_schedule).
 #include <float.h>
 
 #include <algorithm>

@@ -63,7 +63,7 @@ cudaError_t launch_dep(void (*fn)(KArgs...), dim3 grid, dim3 block, size_t smem,
 
 // Process-wide launch parameters (qst_set_tuning; defaults in tuned.h).
 struct Tuning {
-  int bulk_chunks_per_cta;  // least 256-column chunks per CTA of a bulk weight pass (fixes its partition)
+  int bulk_chunks_per_cta;  // least 256-column chunks per group of a bulk weight pass (fixes its partition)
   int fused_ctas_per_sm;    // resident CTAs per SM of the persistent fused batch launch (1 or 2)
   int fused_max_qubits;     // largest N run as one fused iteration when the context asks for the default
   int batch_concurrent_runs;  // 1: a batch's runs of one size start together, 0: one after another
