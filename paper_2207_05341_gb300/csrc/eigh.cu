@@ -489,9 +489,15 @@ __device__ __forceinline__ void load_u_row(const cx_t<R>* src, cx_t<R> (&ux)[RB]
 // column cosets, coset-major), the cosets' unitaries, the tile's row and column indices and the first block
 // column's piece of phi.
 template <class R, int G, int TS> struct TileSmem {
-  // column c of a tile at c + c / G (one word after each coset) and one more per row: the reads of a column
-  // across the row's cosets, and of a row across the column blocks, fall in distinct banks
-  static constexpr int LD = TS + TS / G + 1;
+  // kBySector: consecutive lanes take the same element of consecutive cosets, which are neighbours in memory, so that
+  // a warp takes whole 32-byte sectors of a row (two 16-index cosets are half of each, and the loads bypass L1): an
+  // FP32 A_P step at N = 12 250.9 -> 241.7 ms, a state fidelity at N = 11 90.2 -> 85.7 ms
+  static constexpr bool kBySector = G == 16 && TS == 64;
+  // column c of a tile at c + kPad (c / G) and one more per row: the reads of a column across the row's cosets, of a
+  // row across the column blocks, and the copies of a row fall in distinct banks
+  static constexpr int kPad = kBySector ? 4 : 1;
+  static constexpr int LD = TS + TS / G * kPad + 1;
+  static __device__ __forceinline__ int col(int c) { return c + kPad * (c / G); }
   cx_t<R> a[TS][LD], v[TS][LD];
   cx_t<R> ul[TS / G][G][G], uk[TS / G][G][G];
   int ridx[TS], cidx[TS];
@@ -512,14 +518,16 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
   constexpr int TPC = TS / G, RB = TS / 16;
   constexpr bool kF32 = sizeof(R) == 4;
   extern __shared__ __align__(16) unsigned char sraw[];
-  TileSmem<R, G, TS>& S = *reinterpret_cast<TileSmem<R, G, TS>*>(sraw);
+  using Smem = TileSmem<R, G, TS>;
+  Smem& S = *reinterpret_cast<Smem*>(sraw);
   const int k0 = blockIdx.y * TPC, l0 = blockIdx.x * TPC;
   const int t = threadIdx.x;
   if (t < TS) S.ridx[t] = coset_element(coset_rep(k0 + t / G, p), t % G, p);
   else if (t < 2 * TS) S.cidx[t - TS] = coset_element(coset_rep(l0 + (t - TS) / G, p), (t - TS) % G, p);
   __syncthreads();
   // this thread's column and rows of the tiles (t / TS and every 256 / TS after it)
-  const int tc = t % TS, tr = t / TS, tcs = tc + tc / G;
+  const int tl = t % TS, tr = t / TS;
+  const int tc = Smem::kBySector ? (tl % TPC) * G + tl / TPC : tl, tcs = Smem::col(tc);
   constexpr int kStep = 256 / TS;
   const int gc = S.cidx[tc];
   {
@@ -579,8 +587,8 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
       load_u_row<R, RB>(&S.ul[cc][q][j0], ux, uy);
 #pragma unroll
       for (int i = 0; i < RB; ++i) {
-        const V m = S.a[rr + 16 * i][cc * (G + 1) + q];
-        const V w = HASV ? S.v[rr + 16 * i][cc * (G + 1) + q] : cmake<V>(R(0), R(0));
+        const V m = S.a[rr + 16 * i][Smem::col(cc * G) + q];
+        const V w = HASV ? S.v[rr + 16 * i][Smem::col(cc * G) + q] : cmake<V>(R(0), R(0));
         if constexpr (kF32) {
           const float2 msw = make_float2(-m.y, m.x), wsw = make_float2(-w.y, w.x);  // i m, i w
 #pragma unroll
@@ -602,8 +610,8 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
     for (int i = 0; i < RB; ++i)
 #pragma unroll
       for (int j = 0; j < RB; ++j) {
-        S.a[rr + 16 * i][c0 + j + cc] = acc[i][j];
-        if (HASV) S.v[rr + 16 * i][c0 + j + cc] = accv[i][j];
+        S.a[rr + 16 * i][Smem::col(c0 + j)] = acc[i][j];
+        if (HASV) S.v[rr + 16 * i][Smem::col(c0 + j)] = accv[i][j];
       }
   }
   __syncthreads();
@@ -627,7 +635,7 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
 #pragma unroll
       for (int j = 0; j < RB; ++j) {
         const int c = cs + 16 * j;
-        const V tv = S.a[rc * G + q][c + c / G];
+        const V tv = S.a[rc * G + q][Smem::col(c)];
         if constexpr (kF32) {
           const float2 tsw = make_float2(tv.y, -tv.x);  // -i t
 #pragma unroll
@@ -645,7 +653,7 @@ __global__ void __launch_bounds__(256) k_jacobi_tile(const cx_t<R>* __restrict__
 #pragma unroll
       for (int j = 0; j < RB; ++j) {
         const int c = cs + 16 * j;
-        S.a[r0 + i][c + c / G] = acc[i][j];
+        S.a[r0 + i][Smem::col(c)] = acc[i][j];
       }
   }
   __syncthreads();
@@ -855,7 +863,7 @@ std::vector<JacobiPass> build_schedule(int N) {
 // rounds: 41, 73 and 145 passes a sweep where the lifts by at most 4 dimensions above take 73, 145 and 273 (N = 8 and
 // 12 are 16-index passes throughout either way).  A pass is a chain of latencies (launch, loads, the rounds' rotations
 // one after another) more than work, so half the passes at twice the work each is faster: a state fidelity at FP32
-// N = 9, 10 and 11 7.5, 21.2 and 108.5 ms with A_P's partition, 6.4, 19.0 and 90.2 ms with this one.  A_P keeps its
+// N = 9, 10 and 11 7.5, 21.2 and 108.5 ms with A_P's partition, 6.4, 18.4 and 85.7 ms with this one.  A_P keeps its
 // order: its FP32 states follow the last bit of every rotation.
 std::vector<JacobiPass> build_values_schedule(int N) {
   if (N < 9 || N > 11) return build_schedule(N);
