@@ -90,6 +90,7 @@ __global__ void __launch_bounds__(256) k_weights(const double* __restrict__ P, l
   }
 #pragma unroll
   for (int k = 0; k < kPer / 2; ++k) {
+    if (base + 512LL * k >= n) break;  // the whole slice is past the end
     const unsigned long long w0 = weight_of(pv[k].x, bad), w1 = weight_of(pv[k].y, bad);
     if (!SCAN) {
       total += w0 + w1;
@@ -241,7 +242,9 @@ cudaError_t multinomial_prepare(long long n, const double* P, unsigned long long
 }
 
 // The guide table has a bucket for every four outcomes, or every four shots where those are fewer (building it is then
-// a fraction of the draws); none below 4096 shots.
+// a fraction of the draws).  None below 2^19 shots or 4096 outcomes: its launch costs 4 us, more than it saves on
+// 10^5 draws (N = 6: 39.7 us without, 43.7 with; N = 9 and 10^4 draws 45.7 and 50.8; 10^7 draws at N = 6 277 and 203),
+// and below 4096 outcomes the atomics on the counts are what a draw waits for (N = 5, 10^7 draws: 544 and 545).
 cudaError_t multinomial_draw(long long n, long long shots, unsigned long long seed, unsigned long long W,
                              const unsigned long long* scratch, int* guide, long long* counts, int* kernels,
                              cudaStream_t s) {
@@ -251,7 +254,7 @@ cudaError_t multinomial_draw(long long n, long long shots, unsigned long long se
   while (lm < 30 && (1LL << (lm + 1)) <= shots / 4 && (1LL << (lm + 1)) <= n / 4) ++lm;
   while (bits > 0 && !((W - 1) >> (bits - 1) & 1ull)) --bits;  // (W - 1) >> (bits - lm) < 2^lm
   const int M = 1 << lm, sh = bits > lm ? bits - lm : 0;
-  const bool table = guide && shots >= 4096 && lm >= 4 && sh < 64;
+  const bool table = guide && shots >= (1LL << 19) && n >= 4096 && sh < 64;
   if (table) k_guide<<<grid_of(M + 1), 256, 0, s>>>(scratch, n, M, sh, guide);
   k_draw<<<grid_of(shots), 256, 0, s>>>(scratch, n, shots, seed, table ? guide : nullptr, table ? sh : 0, counts);
   *kernels = table ? 2 : 1;

@@ -48,7 +48,8 @@ def _distribution(kind, n, r):
 
 @pytest.mark.parametrize("kind", ["one", "uniform", "first", "last", "exponents", "half", "above"])
 @pytest.mark.parametrize("N,shots,offset", [(1, 5000, 0), (3, 4095, 0), (3, 4096, 1), (5, 100000, 1), (6, 16384, 0),
-                                            (7, 300001, 0)])
+                                            (7, 300001, 0), (5, 1 << 19, 0), (6, (1 << 19) - 1, 0), (6, 1 << 19, 1),
+                                            (7, 600001, 0), (9, 1 << 20, 1)])
 def test_counts_equal_the_oracle(kind, N, shots, offset):
     n = 4 ** N
     P = _distribution(kind, n, np.random.default_rng(N + shots))
