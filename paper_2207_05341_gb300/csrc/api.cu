@@ -1899,19 +1899,28 @@ qst_status qst_batch_step(qst_batch* bt, const void* const* f, double* losses) {
     // first iteration for these inputs: validate all of them before any tomography steps (a refused call
     // changes nothing), then build each hidden layer (not captured)
     QST_CU(cudaEventRecord(bt->fork, bt->root));  // an earlier iteration may still use the contexts' scratch
-    for (int b = 0; b < bt->B; ++b) {
-      qst_ctx* c = bt->ctx[b];
-      if (c->hidden_valid && c->f_last == f[b]) continue;
-      QST_CU(cudaStreamWaitEvent(c->stream, bt->fork, 0));
-      const qst_status st = c->prec == QST_FP64 ? check_f_begin<double>(c, f[b]) : check_f_begin<float>(c, f[b]);
-      if (st != QST_OK) return st;
+    auto checked = [&](int b) { return bt->ctx[b]->hidden_valid && bt->ctx[b]->f_last == f[b]; };
+    qst_status refused = QST_OK;
+    int begun = 0;
+    for (; begun < bt->B; ++begun) {
+      qst_ctx* c = bt->ctx[begun];
+      if (checked(begun)) continue;
+      refused = cuda_status(cudaStreamWaitEvent(c->stream, bt->fork, 0));
+      if (refused == QST_OK)
+        refused = c->prec == QST_FP64 ? check_f_begin<double>(c, f[begun]) : check_f_begin<float>(c, f[begun]);
+      if (refused != QST_OK) {
+        cudaStreamSynchronize(c->stream);  // whatever of it was enqueued
+        break;
+      }
     }
-    for (int b = 0; b < bt->B; ++b) {  // every check is in flight
-      qst_ctx* c = bt->ctx[b];
-      if (c->hidden_valid && c->f_last == f[b]) continue;
-      const qst_status st = check_f_end(c);
-      if (st != QST_OK) return st;
+    // Every check that was begun is waited for before a refusal is returned: it reads the caller's f and writes the
+    // member's partial sums, which the next iteration (on bt->root, joined to no member's stream) reduces through.
+    for (int b = 0; b < begun; ++b) {
+      if (checked(b)) continue;
+      const qst_status st = check_f_end(bt->ctx[b]);
+      if (refused == QST_OK) refused = st;
     }
+    if (refused != QST_OK) return refused;
     QST_CU(cudaEventRecord(bt->fork, bt->root));
     for (int b = 0; b < bt->B; ++b) {
       qst_ctx* c = bt->ctx[b];
