@@ -170,12 +170,13 @@ __device__ __forceinline__ long long first_above(const unsigned long long* __res
   return lo;
 }
 
-// start[b] = the outcome of the draw t = b 2^sh, b = 0 .. M: a draw t then lies between start[t >> sh] and the entry
-// after it.  Neighbouring buckets search neighbouring places, so this costs far less than as many draws.
+// start[b] = the outcome of the draw t = b 2^sh, b = 0 .. M - 1, and start[M] = n - 1 (M 2^sh is at least the total
+// weight, and 2^64 where that has 64 bits): a draw t then lies between start[t >> sh] and the entry after it.
+// Neighbouring buckets search neighbouring places, so this costs far less than as many draws.
 __global__ void __launch_bounds__(256) k_guide(const unsigned long long* __restrict__ C, long long n, int M, int sh,
                                                 int* __restrict__ start) {
   for (int b = blockIdx.x * blockDim.x + threadIdx.x; b <= M; b += gridDim.x * blockDim.x)
-    start[b] = (int)first_above(C, (unsigned long long)b << sh, 0, n - 1);
+    start[b] = b < M ? (int)first_above(C, (unsigned long long)b << sh, 0, n - 1) : (int)(n - 1);
 }
 
 // One draw: a bucket of the guide table and, within it, a search over the few outcomes that share it (about four at

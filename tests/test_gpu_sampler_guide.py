@@ -65,3 +65,22 @@ def test_counts_equal_the_oracle(kind, N, shots, offset):
         assert np.array_equal(f.cpu().numpy(), (want / shots).astype(np.float32))
     finally:
         qst.qst_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,total", [(6, 0.9995 * 4**6), (6, 0.9999 * 4**6), (6, 2048.0), (6, 2047.0), (7, 4000.0),
+                                     (9, 4095.5)])
+def test_total_weights_up_to_64_bits(N, total):
+    """P need not sum to 1: total weights of 63 and 64 bits (sums from 2^10 to below 2^12)."""
+    n, shots = 4 ** N, 1 << 19
+    P = np.full(n, total / n)
+    if N == 9:
+        P *= np.random.default_rng(N).random(n) * 2.0
+        P *= total / P.sum()
+    assert P.max() <= 1.0
+    ctx = qst.qst_init(N)
+    try:
+        counts = torch.empty(n, dtype=torch.int64, device="cuda")
+        qst.qst_sample_counts(ctx, torch.from_numpy(P).cuda(), shots, 23, counts)
+        assert np.array_equal(counts.cpu().numpy(), O.multinomial_counts_integer(P, shots, 23))
+    finally:
+        qst.qst_destroy(ctx)
