@@ -106,6 +106,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
   const uint32_t acce0 = smem_u32(bars + 2 * kStages + 2);  // accumulator b drained
   const uint32_t done = smem_u32(bars + 2 * kStages + 4);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * kStages + 5);
+  __shared__ int s_fail;  // a drain warp gave up: this CTA's partial tile is not whole
 
   int I, J;  // the tile: rows 128 I .., columns 128 J ..
   const int rank = (int)blockIdx.x % ks;
@@ -132,6 +133,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
       mbar_init(acce0 + 8 * b, kEpiWarps);
     }
     mbar_init(done, 1);
+    s_fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   __syncwarp();
@@ -259,6 +261,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
         *reinterpret_cast<float4*>(out + c) = make_float4(re[c] * u1 * u2, im[c] * u1 * u2, re[c + 1] * u1 * u2,
                                                           im[c + 1] * u1 * u2);
     } else if (lane == 0) {
+      s_fail = 1;
       atomicOr(err, 1u);
     }
   }
@@ -270,6 +273,8 @@ __global__ void __launch_bounds__(kThreads32, 1)
     const float ua = pow2f(-exponent_of(*sA)), ub = pow2f(-exponent_of(*sB));
     const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
     const int rows = kBM / ks;
+    int failed = 0;  // a rank without its partial tile: no rank stores (the flags are read along with the sums)
+    for (int r = 0; r < ks; ++r) failed |= *cl.map_shared_rank(&s_fail, r);
     constexpr int kChunks = kBN / 2, kFly = 4;  // a thread's chunks in flight together
     for (int e0 = threadIdx.x; e0 < rows * kChunks; e0 += kFly * kThreads32) {
       float4 v[kFly];
@@ -292,7 +297,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
 #pragma unroll
       for (int u = 0; u < kFly; ++u) {
         const int e = e0 + u * kThreads32;
-        if (e >= rows * kChunks) continue;
+        if (e >= rows * kChunks || failed) continue;
         const int row = rank * rows + e / kChunks, ch = e % kChunks;
         *reinterpret_cast<float4*>(C + (long long)(I * kBM + row) * d + (long long)J * kBN + 2 * ch) =
             make_float4(v[u].x * u1 * u2, v[u].y * u1 * u2, v[u].z * u1 * u2, v[u].w * u1 * u2);
