@@ -7,7 +7,9 @@
 // exact sum of three BF16 terms x = h + m + l (8 + 8 + 8 significant bits), so the operands carry all 24 bits
 // of FP32, whatever the spread of the entries.  The product keeps the six term pairs down to 2^-18,
 //   l h + h l + m m + m h + h m + h h,
-// and drops m l, l m and l l (at most 2^-26 of |a b|, below half an FP32 ulp of the product).
+// and drops m l, l m and l l: |m| reaches 2^-8 and |l| 2^-17 of |x| (both just above a power of two), so at most
+// 2^-24 of |a b|, half an FP32 ulp, and 2^-27.5 in the mean square over all mantissas.  An infinite entry gives NaN
+// (x - h), where FP32 arithmetic would also give infinities.
 //
 // Accumulation.  The tensor core truncates its FP32 sums: over a K = 2d chain that bias reaches 1.3e-5 at
 // d = 1024 (the mixed path).  Here every block of 32 K elements is a chain of its own, issued from the
