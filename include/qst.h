@@ -393,7 +393,9 @@ qst_status qst_batch_set_params(qst_batch* batch, int b, const void* theta);
 /* One iteration of every tomography.  f: host array of B device pointers (n_b reals
  * each).  losses: host array of B doubles or NULL (synchronises). */
 qst_status qst_batch_step(qst_batch* batch, const void* const* f, double* losses);
-/* iters iterations, then each rho_out[b] (device or host, or rho_out NULL) and final loss. */
+/* iters iterations, then each rho_out[b] (device or host, or rho_out NULL) and final loss.  final_losses: host array of
+ * B doubles or NULL; with it the call synchronises, without it device rho_out are complete once `stream` gets past
+ * them (qst_batch_sync).  A call that is refused has waited for what it began. */
 qst_status qst_batch_reconstruct(qst_batch* batch, const void* const* f, int iters, void* const* rho_out,
                                  double* final_losses);
 long long qst_batch_kernel_launches(const qst_batch* batch);

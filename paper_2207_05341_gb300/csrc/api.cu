@@ -1983,6 +1983,18 @@ qst_status qst_batch_reconstruct(qst_batch* bt, const void* const* f, int iters,
     const qst_status st = QST_DISPATCH(c, loss_end(c, final_losses + b));
     if (st < 0 && first >= 0) first = st;
   }
+  // without losses nothing has been waited for: a refused call waits here, any other leaves the states to bt->root
+  // (qst_batch_sync, and the next iteration, which uses the same buffers)
+  for (int b = 0; !final_losses && b < begun; ++b) {
+    cudaError_t e;
+    if (bad < 0) {
+      e = cudaStreamSynchronize(bt->ctx[b]->stream);
+    } else {
+      e = cudaEventRecord(bt->done[b], bt->ctx[b]->stream);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(bt->root, bt->done[b], 0);
+    }
+    if (e != cudaSuccess && first >= 0) first = cuda_status(e);
+  }
   if (first < 0) return first;
   return bad < 0 ? bad : QST_OK;
 }
