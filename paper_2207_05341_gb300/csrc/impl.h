@@ -226,7 +226,7 @@ struct TomoDesc {
   float* t;             // n reals: t, then dL/dt
   float2 *T, *X, *G, *Y;  // d x d complex scratch
   double* scal;         // [0] Tr X, [1] sum f (read, then rewritten), [2] loss
-  unsigned int* flags;  // [0] clamp count
+  unsigned int* flags;  // [0] clamp count; NULL (with rho): rho alone, no likelihood
   float2* rho;          // not NULL: rho = X / Tr X into it (d x d) and the loss, no update
   int N;
 };

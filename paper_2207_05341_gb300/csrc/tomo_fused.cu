@@ -14,7 +14,7 @@
 //   S9  Rprop on W2^T, b2 (dh from the old weights), b1; Rprop on W1 and the next hidden layer
 //       pre = W1' f + b1', h = LeakyReLU(pre), sum f    (Sec. 4.1)
 // with the same arithmetic for every placement of the tomography, so that a batch and a single context give
-// bit-identical iterations.  With td.rho it stops after S6 and writes rho = X / Tr X instead (qst_get_rho).
+// bit-identical iterations.  With td.rho it writes rho = X / Tr X and stops after S6, or after S4 without td.flags (qst_get_rho).
 // The persistent kernel takes tomographies from a work list (largest first) through an atomic counter: ragged
 // sizes in one launch.  Every sum runs in a fixed order (per-thread partial sums, then a fixed tree).
 //
@@ -268,6 +268,7 @@ __device__ void tomo_iteration(const TomoDesc& td, const PovmB<float>& Bm, const
       td.rho[e] = make_float2(x.x * s, x.y * s);
     }
     __syncthreads();
+    if (!td.flags) return;  // rho alone: no likelihood, and no clamps counted
   }
   // S5: q in place; slot (i, j) then holds the outcome k = interleave(i, j)
   if (SM) apply_modes_tile<float, false>(X, N, P, Bm);
