@@ -714,7 +714,10 @@ template <class R> struct Engine {
     if (st != QST_OK) return st;
     const bool beside = run_hidden && !c->hidden_valid && ((uintptr_t)f & 15u) == 0;
     if (beside && (st = hidden(c, theta, f)) != QST_OK) return st;
-    if ((st = check_f_end(c)) != QST_OK) return st;
+    if ((st = check_f_end(c)) != QST_OK) {
+      if (beside) QST_CU(cudaStreamSynchronize(c->stream));  // the layer still reads the caller's f and parameters
+      return st;
+    }
     return run_hidden && !beside ? hidden(c, theta, f) : QST_OK;
   }
 
