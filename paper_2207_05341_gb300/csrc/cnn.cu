@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
                                                           R* __restrict__ db2, long long n, double* partials,
                                                           unsigned int* counter, RpropCfg<R> rc, R slope) {
   __shared__ R hs[H];
-  __shared__ double red[8][H];
+  __shared__ SumRow<4, R> red[8][H / 4];
   if (threadIdx.x < H) hs[threadIdx.x] = hid[threadIdx.x];
   __syncthreads();
   R acc[H];
@@ -456,13 +456,12 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
 #pragma unroll
   for (int j0 = 0; j0 < H; j0 += 4) {  // H = 4 N: four rows at a time
     const R a4[4] = {acc[j0], acc[j0 + 1], acc[j0 + 2], acc[j0 + 3]};
-    warp_sums<4>(a4, [&](int j, typename SumOf<R>::T x) { red[wp][j0 + j] = x.value(); });
+    warp_sums<4>(a4, red[wp][j0 / 4]);
   }
   __syncthreads();
   for (int j = threadIdx.x; j < H; j += blockDim.x) {
-    double sum = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) sum += red[q][j];
-    partials[(size_t)blockIdx.x * kStride + j] = sum;
+    partials[(size_t)blockIdx.x * kStride + j] =
+        sum_rows((int)(blockDim.x >> 5), j & 3, [&](int q) -> const auto& { return red[q][j >> 2]; });
   }
   if (last_block_arrived(counter)) {
     for (int j = wp; j < H; j += (int)(blockDim.x >> 5)) {

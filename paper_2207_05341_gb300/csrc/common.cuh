@@ -184,11 +184,18 @@ __device__ __forceinline__ WideSum pair_xor(WideSum a, int o) {
   return a;
 }
 
-// Sums of M values each over a warp: out(j, sum) is called once per j, by one lane, with an FP32 pair (or, for FP64
-// values, an FP64 sum).  Step by step a lane hands half of the values it still carries to its partner, which hands
-// over the other half: M = 11 takes 16 additions where M butterflies take 55; and the additions are FP32 two-sums,
-// 10 issue slots each, where an FP64 add with its conversions takes 64 to 192 (two operations per clock and SM).
-template <int M, class R, class F> __device__ __forceinline__ void warp_sums(const R (&v)[M], F out) {
+// Sums of M values each, a warp's in a SumRow and a block's from its warps' rows.  The additions are FP32 two-sums, 10
+// issue slots each, where an FP64 add with its conversions takes 64 to 192 (two operations per clock and SM).  A pair
+// has FP32's exponents, and an overflow or an infinite value leaves NaN in it: a warp with a pair that is not finite
+// forms its sums in FP64 (wide; v then holds their bits), and so is the sum over the warps where it needs to be.
+template <int M, class R> struct SumRow {
+  typename SumOf<R>::T v[M];
+  int wide;
+};
+
+// Step by step a lane hands half of the values it still carries to its partner, which hands over the other half: M = 11
+// takes 16 additions where M butterflies take 55.
+template <int M, class R> __device__ __forceinline__ void warp_sums(const R (&v)[M], SumRow<M, R>& row) {
   static_assert(M >= 1 && M <= 32, "at most one value per lane");
   using S = typename SumOf<R>::T;
   constexpr int L = M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : M <= 16 ? 4 : 5, P = 1 << L;
@@ -223,8 +230,46 @@ template <int M, class R, class F> __device__ __forceinline__ void warp_sums(con
       a[0] = pair_add(a[0], pair_xor(a[0], o));
     }
   }
+  if constexpr (sizeof(R) == 4) {
+    const bool wide = __any_sync(0xffffffffu, !isfinite(a[0].s + a[0].e));
+    if (lane == 0) row.wide = wide;
+    if (wide) {
+#pragma unroll
+      for (int j = 0; j < M; ++j) {
+        const double x = warp_sum((double)v[j]);
+        if (lane == 0) {
+          row.v[j].s = __int_as_float(__double2hiint(x));
+          row.v[j].e = __int_as_float(__double2loint(x));
+        }
+      }
+      return;
+    }
+  }
   const int j = lane >> (5 - L);
-  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) out(j, a[0]);
+  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) row.v[j] = a[0];
+}
+
+// Value j summed over the rows row(0), row(1), .. of n warps, in their order.
+template <class F> __device__ __forceinline__ double sum_rows(int n, int j, F row) {
+  auto s = row(0).v[j];
+  if constexpr (sizeof(s.s) == 4) {
+    int wide = row(0).wide;
+    for (int q = 1; q < n; ++q) {
+      s = pair_add(s, row(q).v[j]);
+      wide |= row(q).wide;
+    }
+    if (wide || !isfinite(s.s + s.e)) {
+      double d = 0.0;
+      for (int q = 0; q < n; ++q) {
+        const auto& r = row(q);
+        d += r.wide ? __hiloint2double(__float_as_int(r.v[j].s), __float_as_int(r.v[j].e)) : r.v[j].value();
+      }
+      return d;
+    }
+  } else {
+    for (int q = 1; q < n; ++q) s = pair_add(s, row(q).v[j]);
+  }
+  return s.value();
 }
 
 // "Last block done": every block has written its partial; the last one to arrive

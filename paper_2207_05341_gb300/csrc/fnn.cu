@@ -32,17 +32,12 @@ constexpr int kRowBatch = 4;
 // Reduce M per-thread values over the block; thread 0 writes them (as double) to out[0..M).
 template <int M, class R>
 __device__ __forceinline__ void block_reduce_to(const R (&v)[M], double* out) {
-  using S = typename SumOf<R>::T;
-  __shared__ S red[8][M];
-  const int w = threadIdx.x >> 5;
-  warp_sums<M>(v, [&](int j, S x) { red[w][j] = x; });
+  __shared__ SumRow<M, R> red[8];
+  warp_sums<M>(v, red[threadIdx.x >> 5]);
   __syncthreads();
   const int nw = blockDim.x >> 5;
-  for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    S s;
-    for (int q = 0; q < nw; ++q) s = pair_add(s, red[q][j]);
-    out[j] = s.value();
-  }
+  for (int j = threadIdx.x; j < M; j += blockDim.x)
+    out[j] = sum_rows(nw, j, [&](int q) -> const auto& { return red[q]; });
 }
 
 // In the last block: warp j sums partials[b * kPartialStride + j] over all blocks b

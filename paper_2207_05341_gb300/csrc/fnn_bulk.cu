@@ -130,15 +130,12 @@ template <class R> __device__ __forceinline__ R leaky_b(R x, R slope) { return x
 // thread of the block calls it (the producer warp contributes nothing).
 template <int M>
 __device__ __forceinline__ void block_sum_to(const float (&v)[M], double* out) {
-  __shared__ PairSum red[kConsumerWarps][M];
+  __shared__ SumRow<M, float> red[kConsumerWarps];
   const int w = threadIdx.x >> 5;
-  if (w < kConsumerWarps) warp_sums<M>(v, [&](int j, PairSum x) { red[w][j] = x; });
+  if (w < kConsumerWarps) warp_sums<M>(v, red[w]);
   __syncthreads();
-  for (int j = threadIdx.x; j < M; j += blockDim.x) {
-    PairSum s;
-    for (int q = 0; q < kConsumerWarps; ++q) s = pair_add(s, red[q][j]);
-    out[j] = s.value();
-  }
+  for (int j = threadIdx.x; j < M; j += blockDim.x)
+    out[j] = sum_rows(kConsumerWarps, j, [&](int q) -> const auto& { return red[q]; });
 }
 
 // The sums over the `groups` partial rows, row j by one warp; fin(j, sum) on its lane 0.
@@ -178,7 +175,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
   __shared__ volatile int s_fail;
   __shared__ int s_stop;
   constexpr int RPT = (H + kGroups - 1) / kGroups;  // rows per consumer thread
-  __shared__ PairSum red[kGroups * kConsumerWarps][RPT + 1];
+  __shared__ SumRow<RPT, float> red[kGroups * kConsumerWarps];
+  __shared__ SumRow<1, float> redf[kConsumerWarps];  // sum f
   // ob2: offset of b2 in theta and step, < 0 when this launch leaves b2 alone (W2 pass);
   // ob1: offset of b1, < 0 when the W2 pass only writes dpre (the caller updates b1)
   const bool with_b2 = W2 && ob2 >= 0;
@@ -330,18 +328,18 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
       }
       // the group's sums: per row the thread partials of its kCols columns, per warp, then over the row group's
       // kConsumerWarps warps in order (the partition of k_l1_forward_cols)
-      warp_sums<RPT>(acc, [&](int l, PairSum x) { red[warp][l] = x; });
+      warp_sums<RPT>(acc, red[warp]);
       if (!W2 && rg == 0) {
         const float one[1] = {accf};
-        warp_sums<1>(one, [&](int, PairSum x) { red[warp][RPT] = x; });
+        warp_sums<1>(one, redf[warp]);
       }
       consumers_sync();
       if (tid == 0) s_stop = s_fail;
       if (tid < (W2 ? H : H + 1)) {
-        const int gr = tid < H ? tid / RPT : 0, l = tid < H ? tid % RPT : RPT;
-        PairSum sum;
-        for (int q = 0; q < kConsumerWarps; ++q) sum = pair_add(sum, red[gr * kConsumerWarps + q][l]);
-        partials[(size_t)g * kPartialStride + tid] = sum.value();
+        partials[(size_t)g * kPartialStride + tid] =
+            tid < H ? sum_rows(kConsumerWarps, tid % RPT,
+                               [&](int q) -> const auto& { return red[tid / RPT * kConsumerWarps + q]; })
+                    : sum_rows(kConsumerWarps, 0, [&](int q) -> const auto& { return redf[q]; });
       }
       consumers_sync();
       if (s_stop) break;

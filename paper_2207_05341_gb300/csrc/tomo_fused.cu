@@ -65,16 +65,13 @@ static_assert(sizeof(Smem) % 16 == 0 && 2 * (kFusedSmem + 1024) <= 227 * 1024, "
 // red[kTot + j] (read them before the next reduction).
 constexpr int kTot = 31 * 16;
 template <int M> __device__ void block_sum(const float (&v)[M], double* red) {
-  static_assert(M <= 16, "at most 16 values per reduction");
-  PairSum* pr = reinterpret_cast<PairSum*>(red);  // (a pair has the size of a double)
+  static_assert(M <= 15, "a warp's row is at most 128 bytes");
+  SumRow<M, float>* rows = reinterpret_cast<SumRow<M, float>*>(red);
   const int warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-  warp_sums<M>(v, [&](int j, PairSum s) { pr[warp * 16 + j] = s; });
+  warp_sums<M>(v, rows[warp]);
   __syncthreads();
-  if (threadIdx.x < M) {
-    PairSum s;
-    for (int w = 0; w < nw; ++w) s = pair_add(s, pr[w * 16 + threadIdx.x]);
-    red[kTot + threadIdx.x] = s.value();  // warps <= 16 leave the last row free
-  }
+  if (threadIdx.x < M)  // warps <= 16 leave the last row free
+    red[kTot + threadIdx.x] = sum_rows(nw, threadIdx.x, [&](int q) -> const auto& { return rows[q]; });
   __syncthreads();
 }
 
