@@ -55,6 +55,7 @@ constexpr int kStage = 3 * kA + 6 * kB;
 constexpr int kStages = 3;
 constexpr int kSmem = kStages * kStage + 1024 + 256;
 constexpr int kTmem = 4 * kBN;                // two accumulators of 256 columns
+constexpr int kMaxSplit = 4;                  // CTAs that share a tile, at most
 static_assert(kBM * kBN * 8 <= kStages * kStage, "a partial tile fits in the ring");
 
 struct Maps32 {
@@ -275,8 +276,9 @@ __global__ void __launch_bounds__(kThreads32, 1)
     const float ua = pow2f(-exponent_of(*sA)), ub = pow2f(-exponent_of(*sB));
     const float u1 = fminf(ua, ub), u2 = fmaxf(ua, ub);
     const int rows = kBM / ks;
-    int failed = 0;  // a rank without its partial tile: no rank stores (the flags are read along with the sums)
-    for (int r = 0; r < ks; ++r) failed |= *cl.map_shared_rank(&s_fail, r);
+    int fail[kMaxSplit];  // a rank without its partial tile: no rank stores (the flags are read along with the sums)
+#pragma unroll
+    for (int r = 0; r < kMaxSplit; ++r) fail[r] = r < ks ? *cl.map_shared_rank(&s_fail, r) : 0;
     constexpr int kChunks = kBN / 2, kFly = 4;  // a thread's chunks in flight together
     for (int e0 = threadIdx.x; e0 < rows * kChunks; e0 += kFly * kThreads32) {
       float4 v[kFly];
@@ -299,7 +301,7 @@ __global__ void __launch_bounds__(kThreads32, 1)
 #pragma unroll
       for (int u = 0; u < kFly; ++u) {
         const int e = e0 + u * kThreads32;
-        if (e >= rows * kChunks || failed) continue;
+        if (e >= rows * kChunks || (fail[0] | fail[1] | fail[2] | fail[3])) continue;
         const int row = rank * rows + e / kChunks, ch = e % kChunks;
         *reinterpret_cast<float4*>(C + (long long)(I * kBM + row) * d + (long long)J * kBN + 2 * ch) =
             make_float4(v[u].x * u1 * u2, v[u].y * u1 * u2, v[u].z * u1 * u2, v[u].w * u1 * u2);
@@ -537,7 +539,7 @@ cudaError_t tc32_split(int d, const float2* A, void* P, int planes, bool keep_sc
 
 // CTAs per tile: one from d = 2048 on (136 and 256 tiles on 152 SMs); below, K shared so that a single product
 // reaches more SMs (the order of the sums depends on d alone, so a batch has the bits of its members).
-static int k_split(int d) { return d >= 2048 ? 1 : d >= 512 ? 2 : 4; }
+static int k_split(int d) { return d >= 2048 ? 1 : d >= 512 ? 2 : kMaxSplit; }
 
 cudaError_t tc32_product(int d, const void* Ap, const void* Bp, const double* sA, const double* sB, float2* C,
                          bool lower, int krange, unsigned int* err, unsigned int* clear, cudaStream_t s) {
