@@ -184,18 +184,12 @@ __device__ __forceinline__ WideSum pair_xor(WideSum a, int o) {
   return a;
 }
 
-// Sums of M values each, a warp's in a SumRow and a block's from its warps' rows.  The additions are FP32 two-sums, 10
-// issue slots each, where an FP64 add with its conversions takes 64 to 192 (two operations per clock and SM).  A pair
-// has FP32's exponents, and an overflow or an infinite value leaves NaN in it: a warp with a pair that is not finite
-// forms its sums in FP64 (wide; v then holds their bits), and so is the sum over the warps where it needs to be.
-template <int M, class R> struct SumRow {
-  typename SumOf<R>::T v[M];
-  int wide;
-};
-
-// Step by step a lane hands half of the values it still carries to its partner, which hands over the other half: M = 11
-// takes 16 additions where M butterflies take 55.
-template <int M, class R> __device__ __forceinline__ void warp_sums(const R (&v)[M], SumRow<M, R>& row) {
+// Sums of M values each over a warp, to sums[0 .. M) as FP32 pairs (or, for FP64 values, FP64 sums).  Step by step a
+// lane hands half of the values it still carries to its partner, which hands over the other half: M = 11 takes 16
+// additions where M butterflies take 55; and the additions are FP32 two-sums, 10 issue slots each, where an FP64 add
+// with its conversions takes 64 to 192 (two operations per clock and SM).
+template <int M, class R>
+__device__ __forceinline__ void warp_sums(const R (&v)[M], typename SumOf<R>::T* sums) {
   static_assert(M >= 1 && M <= 32, "at most one value per lane");
   using S = typename SumOf<R>::T;
   constexpr int L = M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : M <= 16 ? 4 : 5, P = 1 << L;
@@ -230,46 +224,62 @@ template <int M, class R> __device__ __forceinline__ void warp_sums(const R (&v)
       a[0] = pair_add(a[0], pair_xor(a[0], o));
     }
   }
+  const int j = lane >> (5 - L);
+  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) sums[j] = a[0];
+}
+
+// The same in FP64, its bits in the place of the pairs; out of line, a path that is hardly ever taken.
+static __device__ __noinline__ void wide_warp_sums(const float* v, int M, PairSum* sums) {
+#pragma unroll 1
+  for (int j = 0; j < M; ++j) {
+    const double x = warp_sum((double)v[j]);
+    if ((threadIdx.x & 31) == 0) {
+      sums[j].s = __int_as_float(__double2hiint(x));
+      sums[j].e = __int_as_float(__double2loint(x));
+    }
+  }
+}
+template <int M, class R>
+__device__ __forceinline__ void warp_sums(const R (&v)[M], typename SumOf<R>::T* sums, bool wide) {
   if constexpr (sizeof(R) == 4) {
-    const bool wide = __any_sync(0xffffffffu, !isfinite(a[0].s + a[0].e));
-    if (lane == 0) row.wide = wide;
     if (wide) {
+      R c[M];  // (v itself stays in registers)
 #pragma unroll
-      for (int j = 0; j < M; ++j) {
-        const double x = warp_sum((double)v[j]);
-        if (lane == 0) {
-          row.v[j].s = __int_as_float(__double2hiint(x));
-          row.v[j].e = __int_as_float(__double2loint(x));
-        }
-      }
+      for (int j = 0; j < M; ++j) c[j] = v[j];
+      wide_warp_sums(c, M, sums);
       return;
     }
   }
-  const int j = lane >> (5 - L);
-  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) row.v[j] = a[0];
+  warp_sums<M>(v, sums);
 }
 
-// Value j summed over the rows row(0), row(1), .. of n warps, in their order.
-template <class F> __device__ __forceinline__ double sum_rows(int n, int j, F row) {
-  auto s = row(0).v[j];
-  if constexpr (sizeof(s.s) == 4) {
-    int wide = row(0).wide;
-    for (int q = 1; q < n; ++q) {
-      s = pair_add(s, row(q).v[j]);
-      wide |= row(q).wide;
-    }
-    if (wide || !isfinite(s.s + s.e)) {
-      double d = 0.0;
-      for (int q = 0; q < n; ++q) {
-        const auto& r = row(q);
-        d += r.wide ? __hiloint2double(__float_as_int(r.v[j].s), __float_as_int(r.v[j].e)) : r.v[j].value();
-      }
-      return d;
-    }
-  } else {
-    for (int q = 1; q < n; ++q) s = pair_add(s, row(q).v[j]);
+// A sum over n warps, in their order: fill(wide) leaves each warp's part where at(0 .. n - 1) finds it, and the threads
+// with `mine` pass the total to out.  sync: a barrier of all the threads; any: one that also tells whether the
+// argument was true for any of them.  A pair has FP32's exponents, and an overflow or an infinite term leaves NaN in
+// it: where a total is not finite everything is summed again in FP64, which carries them.
+template <class Fill, class At, class Sync, class Any, class Out>
+__device__ __forceinline__ void sums_over_warps(int n, bool mine, Fill fill, At at, Sync sync, Any any, Out out) {
+  constexpr bool kPairs = sizeof(at(0).s) == 4;
+  fill(false);
+  sync();
+  bool redo = false;
+  if (mine) {
+    auto s = at(0);
+    for (int q = 1; q < n; ++q) s = pair_add(s, at(q));
+    out(s.value());
+    if constexpr (kPairs) redo = !isfinite(s.s + s.e);
   }
-  return s.value();
+  if constexpr (kPairs) {
+    if (!any(redo)) return;
+    fill(true);
+    sync();
+    if (mine) {
+      double d = 0.0;
+      for (int q = 0; q < n; ++q) d += __hiloint2double(__float_as_int(at(q).s), __float_as_int(at(q).e));
+      out(d);
+    }
+    sync();
+  }
 }
 
 // "Last block done": every block has written its partial; the last one to arrive

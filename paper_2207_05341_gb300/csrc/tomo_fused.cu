@@ -65,14 +65,13 @@ static_assert(sizeof(Smem) % 16 == 0 && 2 * (kFusedSmem + 1024) <= 227 * 1024, "
 // red[kTot + j] (read them before the next reduction).
 constexpr int kTot = 31 * 16;
 template <int M> __device__ void block_sum(const float (&v)[M], double* red) {
-  static_assert(M <= 15, "a warp's row is at most 128 bytes");
-  SumRow<M, float>* rows = reinterpret_cast<SumRow<M, float>*>(red);
-  const int warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
-  warp_sums<M>(v, rows[warp]);
-  __syncthreads();
-  if (threadIdx.x < M)  // warps <= 16 leave the last row free
-    red[kTot + threadIdx.x] = sum_rows(nw, threadIdx.x, [&](int q) -> const auto& { return rows[q]; });
-  __syncthreads();
+  static_assert(M <= 16, "at most 16 values per reduction");
+  PairSum* pr = reinterpret_cast<PairSum*>(red);  // (a pair has the size of a double)
+  const int j = threadIdx.x;
+  sums_over_warps(
+      (int)(blockDim.x >> 5), j < M, [&](bool wide) { warp_sums<M>(v, pr + (j >> 5) * 16, wide); },
+      [&](int q) { return pr[q * 16 + j]; }, [] { __syncthreads(); }, [](bool x) { return __syncthreads_or(x); },
+      [&](double sum) { red[kTot + j] = sum; });  // warps <= 16 leave the last row free
 }
 
 // The same for one FP64 value; every thread gets the total.
