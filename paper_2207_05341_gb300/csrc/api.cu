@@ -251,11 +251,18 @@ size_t lazy_scratch_bytes(const Dims& D) {
   return 8 * (2 * (size_t)D.n + (size_t)D.n / 512) + 40 * (size_t)D.d * D.d + 512 * (size_t)D.d + 65536;
 }
 
-// An allocation the context can do without: skipped where it fails, or where it would leave less of the
-// budget than `later` bytes (the scratch that calls may still allocate on first use).
+// An allocation the context can do without: skipped where it fails, or where it would leave less of the budget or
+// of the device than `later` bytes (the scratch that calls may still allocate on first use; 16 MiB for the rounding
+// of allocations to pages).
 template <class T> void dalloc_optional(qst_ctx* c, T** p, size_t count, size_t later) {
   const size_t lim = c->opt.device_memory_limit;
   if (lim && c->dev_bytes + count * sizeof(T) + later > lim) return;
+  size_t free_bytes = 0, total = 0;
+  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
+  if (free_bytes < count * sizeof(T) + later + (16u << 20)) return;
   if (dalloc(c, p, count) != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
@@ -369,13 +376,11 @@ template <class R> qst_status alloc_work(qst_ctx* c) {
   }
   // FP32 products on tensor cores where their operand planes fit (else on the CUDA cores)
   if (c->prec == QST_FP32 && c->opt.mapping != QST_MAP_ABS_P && tc32_ok(D.d)) {
-    const size_t later = lazy_scratch_bytes(D);
-    unsigned short *p9 = nullptr, *p6 = nullptr;
-    dalloc_optional(c, &p9, 9 * nn, 12 * nn + later);
-    if (p9) dalloc_optional(c, &p6, 6 * nn, later);
-    if (p6) {
-      w->P9 = p9;
-      w->P6 = p6;
+    unsigned short* planes = nullptr;
+    dalloc_optional(c, &planes, 15 * nn, lazy_scratch_bytes(D));
+    if (planes) {
+      w->P9 = planes;
+      w->P6 = planes + 9 * nn;
     }
   }
   return QST_OK;
