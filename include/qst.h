@@ -289,6 +289,8 @@ qst_status qst_eig_counts(const qst_ctx* ctx, long long* refinements, long long*
  * bits distinct and ascending, each top bit clear in the other vectors; unused entries 0).  Host arrays;
  * may be NULL when cap == 0.  QST_E_INVAL for N outside 1..12 or NULL arrays with cap > 0. */
 qst_status qst_jacobi_schedule(int N, int* count, int* dims, int* basis, int cap);
+/* The same for the sweeps without eigenvectors behind qst_state_fidelity. */
+qst_status qst_jacobi_values_schedule(int N, int* count, int* dims, int* basis, int cap);
 
 /* Number of kernel launches the library has enqueued on this context (graph
  * replays count every kernel node). */

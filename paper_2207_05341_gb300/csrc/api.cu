@@ -1699,15 +1699,23 @@ qst_status qst_eig_counts(const qst_ctx* c, long long* refinements, long long* f
   return QST_OK;
 }
 
-qst_status qst_jacobi_schedule(int N, int* count, int* dims, int* basis, int cap) {
+static qst_status schedule_to(int N, bool values, int* count, int* dims, int* basis, int cap) {
   if (N < 1 || N > 12 || !count || cap < 0 || (cap > 0 && (!dims || !basis))) return QST_E_INVAL;
-  const std::vector<qst::JacobiPass>& s = qst::jacobi_schedule(N);
+  const std::vector<qst::JacobiPass>& s = qst::jacobi_schedule(N, values);
   *count = (int)s.size();
   for (int k = 0; k < cap && k < (int)s.size(); ++k) {
     dims[k] = s[k].k;
     for (int i = 0; i < 4; ++i) basis[4 * k + i] = i < s[k].k ? s[k].basis[i] : 0;
   }
   return QST_OK;
+}
+
+qst_status qst_jacobi_schedule(int N, int* count, int* dims, int* basis, int cap) {
+  return schedule_to(N, false, count, dims, basis, cap);
+}
+
+qst_status qst_jacobi_values_schedule(int N, int* count, int* dims, int* basis, int cap) {
+  return schedule_to(N, true, count, dims, basis, cap);
 }
 
 long long qst_iterations(const qst_ctx* c) { return c ? c->iters : -1; }

@@ -859,12 +859,12 @@ std::vector<JacobiPass> build_schedule(int N) {
 }
 
 // The partition used where no eigenvectors are wanted, 9 <= N <= 11: the graphs u -> (u, c iota(u)) of V(4) in
-// GF(2^k), k = N - 4 (dimension 4, one for each c), and V(k) partitioned as above, so nearly every pass applies 15
-// rounds: 41, 73 and 145 passes a sweep where the lifts by at most 4 dimensions above take 73, 145 and 273 (N = 8 and
-// 12 are 16-index passes throughout either way).  A pass is a chain of latencies (launch, loads, the rounds' rotations
-// one after another) more than work, so half the passes at twice the work each is faster: a state fidelity at FP32
-// N = 9, 10 and 11 7.5, 21.2 and 108.5 ms with A_P's partition, 6.4, 18.4 and 85.7 ms with this one.  A_P keeps its
-// order: its FP32 states follow the last bit of every rotation.
+// GF(2^k), k = N - 4 (dimension 4, one for each c), and V(k) partitioned as above (at N = 9 into one subspace of
+// dimension 3 and eight of dimension 2), so nearly every pass applies 15 rounds: 41, 73 and 145 passes a sweep where
+// the lifts by at most 4 dimensions above take 73, 145 and 273 (N = 8 and 12 are 16-index passes throughout either
+// way).  A pass is a chain of latencies (launch, loads, the rounds' rotations one after another) more than work, so
+// half the passes at twice the work each is faster: a state fidelity at FP32 N = 9, 10 and 11 7.5, 21.2 and 108.5 ms
+// with A_P's partition, 6.4, 18.4 and 85.7 ms with this one.
 std::vector<JacobiPass> build_values_schedule(int N) {
   if (N < 9 || N > 11) return build_schedule(N);
   const int k = N - 4;

@@ -123,6 +123,7 @@ def load(path: str = LIB_PATH) -> ctypes.CDLL:
         "qst_iterations": (ctypes.c_longlong, [vp]),
         "qst_eig_counts": (i, [vp, ctypes.POINTER(ctypes.c_longlong), ctypes.POINTER(ctypes.c_longlong), pd]),
         "qst_jacobi_schedule": (i, [i, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i), i]),
+        "qst_jacobi_values_schedule": (i, [i, ctypes.POINTER(i), ctypes.POINTER(i), ctypes.POINTER(i), i]),
         "qst_kernel_launches": (ctypes.c_longlong, [vp]),
         "qst_sync": (i, [vp]),
         "qst_strerror": (ctypes.c_char_p, [i]),
@@ -362,14 +363,23 @@ def qst_eig_counts(ctx: int, last: bool = False):
     return (a.value, b.value, (v[0], v[1])) if last else (a.value, b.value)
 
 
-def qst_jacobi_schedule(N: int):
-    """Passes of one Jacobi sweep at N qubits (host only): a list of subspace bases (tuples of 1 to 4 ints)."""
-    cnt = ctypes.c_int()
-    _check(load().qst_jacobi_schedule(int(N), ctypes.byref(cnt), None, None, 0), "qst_jacobi_schedule")
+def _schedule(name: str, N: int):
+    fn, cnt = getattr(load(), name), ctypes.c_int()
+    _check(fn(int(N), ctypes.byref(cnt), None, None, 0), name)
     dims = (ctypes.c_int * cnt.value)()
     basis = (ctypes.c_int * (4 * cnt.value))()
-    _check(load().qst_jacobi_schedule(int(N), ctypes.byref(cnt), dims, basis, cnt.value), "qst_jacobi_schedule")
+    _check(fn(int(N), ctypes.byref(cnt), dims, basis, cnt.value), name)
     return [tuple(basis[4 * p:4 * p + dims[p]]) for p in range(cnt.value)]
+
+
+def qst_jacobi_schedule(N: int):
+    """Passes of one Jacobi sweep at N qubits (host only): a list of subspace bases (tuples of 1 to 4 ints)."""
+    return _schedule("qst_jacobi_schedule", N)
+
+
+def qst_jacobi_values_schedule(N: int):
+    """The same for the sweeps without eigenvectors (the state fidelity)."""
+    return _schedule("qst_jacobi_values_schedule", N)
 
 
 def qst_get_tuning() -> dict:
