@@ -397,7 +397,7 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
                                                           R* __restrict__ db2, long long n, double* partials,
                                                           unsigned int* counter, RpropCfg<R> rc, R slope) {
   __shared__ R hs[H];
-  __shared__ typename SumOf<R>::T red[8][H];
+  __shared__ double red[8][H];
   if (threadIdx.x < H) hs[threadIdx.x] = hid[threadIdx.x];
   __syncthreads();
   R acc[H];
@@ -453,18 +453,17 @@ __global__ void __launch_bounds__(256) k_cnn_output_back(R* __restrict__ W2T, R*
     }
   }
   const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  const int j = threadIdx.x;
-  sums_over_warps(
-      (int)(blockDim.x >> 5), j < H,
-      [&](bool wide) {
 #pragma unroll
-        for (int j0 = 0; j0 < H; j0 += 4) {  // H = 4 N: four rows at a time
-          const R a4[4] = {acc[j0], acc[j0 + 1], acc[j0 + 2], acc[j0 + 3]};
-          warp_sums<4>(a4, red[wp] + j0, wide);
-        }
-      },
-      [&](int q) { return red[q][j]; }, [] { __syncthreads(); }, [](bool x) { return __syncthreads_or(x); },
-      [&](double sum) { partials[(size_t)blockIdx.x * kStride + j] = sum; });
+  for (int j0 = 0; j0 < H; j0 += 4) {  // H = 4 N: four rows at a time
+    const R a4[4] = {acc[j0], acc[j0 + 1], acc[j0 + 2], acc[j0 + 3]};
+    warp_sums<4>(a4, [&](int j, typename SumOf<R>::T x) { red[wp][j0 + j] = sum_value(x); });
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < H; j += blockDim.x) {
+    double sum = 0.0;
+    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) sum += red[q][j];
+    partials[(size_t)blockIdx.x * kStride + j] = sum;
+  }
   if (last_block_arrived(counter)) {
     for (int j = wp; j < H; j += (int)(blockDim.x >> 5)) {
       double sum = 0.0;

@@ -138,7 +138,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 }
 
 // A sum kept as an FP32 pair s + e (Knuth's two-sum; a product's rounding error by FMA), so that a thread's terms
-// keep about 48 bits without the FP64 pipe (two operations per clock and SM).
+// keep about 48 bits without the FP64 pipe (two operations per clock and SM).  An infinite term leaves NaN in e, and s
+// as it would leave an FP32 sum.
 struct PairSum {
   float s = 0.f, e = 0.f;
   __device__ __forceinline__ void add(float v) {
@@ -151,7 +152,7 @@ struct PairSum {
     e = __fadd_rn(e, __fmaf_rn(a, b, -p));
     add(p);
   }
-  __device__ __forceinline__ double value() const { return (double)s + (double)e; }
+  __device__ __forceinline__ double value() const { return isfinite(s) ? (double)s + (double)e : (double)s; }
 };
 // The same in FP64 arithmetic for FP64 terms.
 struct WideSum {
@@ -184,12 +185,19 @@ __device__ __forceinline__ WideSum pair_xor(WideSum a, int o) {
   return a;
 }
 
-// Sums of M values each over a warp, to sums[0 .. M) as FP32 pairs (or, for FP64 values, FP64 sums).  Step by step a
-// lane hands half of the values it still carries to its partner, which hands over the other half: M = 11 takes 16
-// additions where M butterflies take 55; and the additions are FP32 two-sums, 10 issue slots each, where an FP64 add
-// with its conversions takes 64 to 192 (two operations per clock and SM).
-template <int M, class R>
-__device__ __forceinline__ void warp_sums(const R (&v)[M], typename SumOf<R>::T* sums) {
+// Pairs have FP32's exponents, and a sum of finite terms must not overflow on its way where an FP64 sum does not: the
+// sums over a warp and a block's warps (at most 2^9 threads) are of 2^-10 of the terms, exact but for terms below
+// 2^-116, which keep their bits down to 2^-140.
+__device__ __forceinline__ float sum_term(float v) { return v * 0x1p-10f; }
+__device__ __forceinline__ double sum_term(double v) { return v; }
+__device__ __forceinline__ double sum_value(const PairSum& s) { return s.value() * 0x1p10; }
+__device__ __forceinline__ double sum_value(const WideSum& s) { return s.value(); }
+
+// Sums of M values each over a warp: out(j, sum) is called once per j, by one lane, with an FP32 pair (or, for FP64
+// values, an FP64 sum) for sum_value.  Step by step a lane hands half of the values it still carries to its partner, which hands
+// over the other half: M = 11 takes 16 additions where M butterflies take 55; and the additions are FP32 two-sums,
+// 10 issue slots each, where an FP64 add with its conversions takes 64 to 192 (two operations per clock and SM).
+template <int M, class R, class F> __device__ __forceinline__ void warp_sums(const R (&v)[M], F out) {
   static_assert(M >= 1 && M <= 32, "at most one value per lane");
   using S = typename SumOf<R>::T;
   constexpr int L = M <= 1 ? 0 : M <= 2 ? 1 : M <= 4 ? 2 : M <= 8 ? 3 : M <= 16 ? 4 : 5, P = 1 << L;
@@ -197,12 +205,13 @@ __device__ __forceinline__ void warp_sums(const R (&v)[M], typename SumOf<R>::T*
   S a[P > 1 ? P / 2 : 1];
   int o = 16;
   if constexpr (P == 1) {
-    a[0].add(v[0]);
+    a[0].add(sum_term(v[0]));
   } else {
     const bool up = (lane & 16) != 0;
 #pragma unroll
     for (int k = 0; k < P / 2; ++k) {
-      const R lo = k < M ? v[k < M ? k : 0] : R(0), hi = k + P / 2 < M ? v[k + P / 2 < M ? k + P / 2 : 0] : R(0);
+      const R lo = k < M ? sum_term(v[k < M ? k : 0]) : R(0);
+      const R hi = k + P / 2 < M ? sum_term(v[k + P / 2 < M ? k + P / 2 : 0]) : R(0);
       const R keep = up ? hi : lo, send = up ? lo : hi;
       a[k].s = keep;
       a[k].add(__shfl_xor_sync(0xffffffffu, send, 16));
@@ -225,61 +234,7 @@ __device__ __forceinline__ void warp_sums(const R (&v)[M], typename SumOf<R>::T*
     }
   }
   const int j = lane >> (5 - L);
-  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) sums[j] = a[0];
-}
-
-// The same in FP64, its bits in the place of the pairs; out of line, a path that is hardly ever taken.
-static __device__ __noinline__ void wide_warp_sums(const float* v, int M, PairSum* sums) {
-#pragma unroll 1
-  for (int j = 0; j < M; ++j) {
-    const double x = warp_sum((double)v[j]);
-    if ((threadIdx.x & 31) == 0) {
-      sums[j].s = __int_as_float(__double2hiint(x));
-      sums[j].e = __int_as_float(__double2loint(x));
-    }
-  }
-}
-template <int M, class R>
-__device__ __forceinline__ void warp_sums(const R (&v)[M], typename SumOf<R>::T* sums, bool wide) {
-  if constexpr (sizeof(R) == 4) {
-    if (wide) {
-      R c[M];  // (v itself stays in registers)
-#pragma unroll
-      for (int j = 0; j < M; ++j) c[j] = v[j];
-      wide_warp_sums(c, M, sums);
-      return;
-    }
-  }
-  warp_sums<M>(v, sums);
-}
-
-// A sum over n warps, in their order: fill(wide) leaves each warp's part where at(0 .. n - 1) finds it, and the threads
-// with `mine` pass the total to out.  sync: a barrier of all the threads; any: one that also tells whether the
-// argument was true for any of them.  A pair has FP32's exponents, and an overflow or an infinite term leaves NaN in
-// it: where a total is not finite everything is summed again in FP64, which carries them.
-template <class Fill, class At, class Sync, class Any, class Out>
-__device__ __forceinline__ void sums_over_warps(int n, bool mine, Fill fill, At at, Sync sync, Any any, Out out) {
-  constexpr bool kPairs = sizeof(at(0).s) == 4;
-  fill(false);
-  sync();
-  bool redo = false;
-  if (mine) {
-    auto s = at(0);
-    for (int q = 1; q < n; ++q) s = pair_add(s, at(q));
-    out(s.value());
-    if constexpr (kPairs) redo = !isfinite(s.s + s.e);
-  }
-  if constexpr (kPairs) {
-    if (!any(redo)) return;
-    fill(true);
-    sync();
-    if (mine) {
-      double d = 0.0;
-      for (int q = 0; q < n; ++q) d += __hiloint2double(__float_as_int(at(q).s), __float_as_int(at(q).e));
-      out(d);
-    }
-    sync();
-  }
+  if ((lane & ((1 << (5 - L)) - 1)) == 0 && j < M) out(j, a[0]);
 }
 
 // "Last block done": every block has written its partial; the last one to arrive

@@ -32,12 +32,17 @@ constexpr int kRowBatch = 4;
 // Reduce M per-thread values over the block; thread 0 writes them (as double) to out[0..M).
 template <int M, class R>
 __device__ __forceinline__ void block_reduce_to(const R (&v)[M], double* out) {
-  __shared__ typename SumOf<R>::T red[8][M];
-  const int j = threadIdx.x;
-  sums_over_warps(
-      (int)(blockDim.x >> 5), j < M, [&](bool wide) { warp_sums<M>(v, red[j >> 5], wide); },
-      [&](int q) { return red[q][j]; }, [] { __syncthreads(); }, [](bool x) { return __syncthreads_or(x); },
-      [&](double sum) { out[j] = sum; });
+  using S = typename SumOf<R>::T;
+  __shared__ S red[8][M];
+  const int w = threadIdx.x >> 5;
+  warp_sums<M>(v, [&](int j, S x) { red[w][j] = x; });
+  __syncthreads();
+  const int nw = blockDim.x >> 5;
+  for (int j = threadIdx.x; j < M; j += blockDim.x) {
+    S s;
+    for (int q = 0; q < nw; ++q) s = pair_add(s, red[q][j]);
+    out[j] = sum_value(s);
+  }
 }
 
 // In the last block: warp j sums partials[b * kPartialStride + j] over all blocks b

@@ -60,19 +60,6 @@ __device__ __forceinline__ bool bar_try(uint32_t bar, uint32_t parity) {
 }
 // barrier of the consumer warps alone (the producer warp goes on issuing copies)
 __device__ __forceinline__ void consumers_sync() { asm volatile("bar.sync 1, %0;" ::"r"(kConsumers) : "memory"); }
-// the same, telling whether x was true for any of them
-__device__ __forceinline__ bool consumers_any(bool x) {
-  uint32_t any;
-  asm volatile(
-      "{\n.reg .pred p, q;\n"
-      "setp.ne.u32 p, %1, 0;\n"
-      "bar.red.or.pred q, 1, %2, p;\n"
-      "selp.u32 %0, 1, 0, q;\n}\n"
-      : "=r"(any)
-      : "r"((uint32_t)x), "r"(kConsumers)
-      : "memory");
-  return any != 0;
-}
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity) {
   if (bar_try(bar, parity)) return true;
   const unsigned long long t0 = clock64();
@@ -144,11 +131,14 @@ template <class R> __device__ __forceinline__ R leaky_b(R x, R slope) { return x
 template <int M>
 __device__ __forceinline__ void block_sum_to(const float (&v)[M], double* out) {
   __shared__ PairSum red[kConsumerWarps][M];
-  const int j = threadIdx.x, w = j >> 5;
-  sums_over_warps(
-      kConsumerWarps, j < M, [&](bool wide) { if (w < kConsumerWarps) warp_sums<M>(v, red[w], wide); },
-      [&](int q) { return red[q][j]; }, [] { __syncthreads(); }, [](bool x) { return __syncthreads_or(x); },
-      [&](double sum) { out[j] = sum; });
+  const int w = threadIdx.x >> 5;
+  if (w < kConsumerWarps) warp_sums<M>(v, [&](int j, PairSum x) { red[w][j] = x; });
+  __syncthreads();
+  for (int j = threadIdx.x; j < M; j += blockDim.x) {
+    PairSum s;
+    for (int q = 0; q < kConsumerWarps; ++q) s = pair_add(s, red[q][j]);
+    out[j] = sum_value(s);
+  }
 }
 
 // The sums over the `groups` partial rows, row j by one warp; fin(j, sum) on its lane 0.
@@ -340,22 +330,20 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
       }
       // the group's sums: per row the thread partials of its kCols columns, per warp, then over the row group's
       // kConsumerWarps warps in order (the partition of k_l1_forward_cols)
-      const int gr = tid < H ? tid / RPT : 0, ls = tid < H ? tid % RPT : RPT;
-      sums_over_warps(
-          kConsumerWarps, tid < (W2 ? H : H + 1),
-          [&](bool wide) {
-            warp_sums<RPT>(acc, red[warp], wide);
-            if (!W2 && rg == 0) {
-              const float one[1] = {accf};
-              warp_sums<1>(one, red[warp] + RPT, wide);
-            }
-          },
-          [&](int q) { return red[gr * kConsumerWarps + q][ls]; }, consumers_sync,
-          [&](bool x) {
-            if (tid == 0) s_stop = s_fail;
-            return consumers_any(x);
-          },
-          [&](double sum) { partials[(size_t)g * kPartialStride + tid] = sum; });
+      warp_sums<RPT>(acc, [&](int l, PairSum x) { red[warp][l] = x; });
+      if (!W2 && rg == 0) {
+        const float one[1] = {accf};
+        warp_sums<1>(one, [&](int, PairSum x) { red[warp][RPT] = x; });
+      }
+      consumers_sync();
+      if (tid == 0) s_stop = s_fail;
+      if (tid < (W2 ? H : H + 1)) {
+        const int gr = tid < H ? tid / RPT : 0, l = tid < H ? tid % RPT : RPT;
+        PairSum sum;
+        for (int q = 0; q < kConsumerWarps; ++q) sum = pair_add(sum, red[gr * kConsumerWarps + q][l]);
+        partials[(size_t)g * kPartialStride + tid] = sum_value(sum);
+      }
+      consumers_sync();
       if (s_stop) break;
 #pragma unroll
       for (int l = 0; l < RPT; ++l) acc[l] = 0.f;

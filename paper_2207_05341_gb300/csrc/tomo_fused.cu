@@ -14,7 +14,8 @@
 //   S9  Rprop on W2^T, b2 (dh from the old weights), b1; Rprop on W1 and the next hidden layer
 //       pre = W1' f + b1', h = LeakyReLU(pre), sum f    (Sec. 4.1)
 // with the same arithmetic for every placement of the tomography, so that a batch and a single context give
-// bit-identical iterations.  With td.rho it writes rho = X / Tr X and stops after S6, or after S4 without td.flags (qst_get_rho).
+// bit-identical iterations.  With td.rho it writes rho = X / Tr X and stops after S6 (without td.flags, after S4):
+// qst_get_rho.
 // The persistent kernel takes tomographies from a work list (largest first) through an atomic counter: ragged
 // sizes in one launch.  Every sum runs in a fixed order (per-thread partial sums, then a fixed tree).
 //
@@ -67,11 +68,15 @@ constexpr int kTot = 31 * 16;
 template <int M> __device__ void block_sum(const float (&v)[M], double* red) {
   static_assert(M <= 16, "at most 16 values per reduction");
   PairSum* pr = reinterpret_cast<PairSum*>(red);  // (a pair has the size of a double)
-  const int j = threadIdx.x;
-  sums_over_warps(
-      (int)(blockDim.x >> 5), j < M, [&](bool wide) { warp_sums<M>(v, pr + (j >> 5) * 16, wide); },
-      [&](int q) { return pr[q * 16 + j]; }, [] { __syncthreads(); }, [](bool x) { return __syncthreads_or(x); },
-      [&](double sum) { red[kTot + j] = sum; });  // warps <= 16 leave the last row free
+  const int warp = threadIdx.x >> 5, nw = (int)(blockDim.x >> 5);
+  warp_sums<M>(v, [&](int j, PairSum s) { pr[warp * 16 + j] = s; });
+  __syncthreads();
+  if (threadIdx.x < M) {
+    PairSum s;
+    for (int w = 0; w < nw; ++w) s = pair_add(s, pr[w * 16 + threadIdx.x]);
+    red[kTot + threadIdx.x] = sum_value(s);  // warps <= 16 leave the last row free
+  }
+  __syncthreads();
 }
 
 // The same for one FP64 value; every thread gets the total.

@@ -100,3 +100,24 @@ def test_step(N, net):
         assert after[p.b1] == np.float32(-1e-3) and after[p.b1 + 1] == np.float32(1e-3)
     finally:
         qst.qst_destroy(ctx)
+
+
+@pytest.mark.parametrize("N,net", CASES)
+def test_infinite_terms(N, net):
+    """Terms that overflow themselves: the sums are infinite, not NaN, and the step moves."""
+    p = Net(N, net)
+    ctx, f = _context(N, net)
+    try:
+        theta, A = _theta(ctx, p, f, False)
+        A = (A / BIG * 3e38).astype(np.float32)
+        theta[p.b2:p.b2 + p.n] *= np.float32(2.0 ** -4)  # |dL/dt| 8 on average
+        theta[p.w2:p.w2 + p.n], theta[p.w2 + p.n:p.w2 + 2 * p.n] = A, -A
+        g = _grad(ctx, theta, f)
+        assert g[p.b1] == np.inf and g[p.b1 + 1] == -np.inf
+        qst.qst_set_params(ctx, theta)
+        qst.qst_step(ctx, f)
+        after = np.empty_like(theta)
+        qst.qst_get_params(ctx, after)
+        assert after[p.b1] == np.float32(-1e-3) and after[p.b1 + 1] == np.float32(1e-3)
+    finally:
+        qst.qst_destroy(ctx)
