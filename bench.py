@@ -172,7 +172,8 @@ def phase_work(phase, N, mixed):
     d = 2 ** N
     H = 2 * N
     if phase == "build_T":
-        return "hbm", (H + 1) * 4 * n + (12 if mixed else 8) * n, "B"
+        # t's 6 or 9 operand planes; t and T below 7 qubits
+        return "hbm", (H + 1) * 4 * n + (12 if mixed else 18 if N >= 7 else 8) * n, "B"
     if phase == "x_fwd":
         return "tensor", 4 * d ** 3, "FLOP"
     if phase == "gt":
@@ -186,7 +187,7 @@ def phase_work(phase, N, mixed):
     if phase == "povm_map":   # qst_probs: lower half of rho read, p written (8 n B, the map's algorithmic bytes)
         return "hbm", 8 * n, "B"
     if phase == "sym":
-        return "hbm", 8 * n + 4 * n, "B"
+        return "hbm", 8 * n + (4 if mixed or N < 7 else 8) * n, "B"  # FP32 on tensor cores reads t too
     if phase == "w2":
         return "hbm", 16 * H * n + 20 * n, "B"
     if phase == "w1":

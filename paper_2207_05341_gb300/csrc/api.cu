@@ -1476,8 +1476,10 @@ qst_status qst_init(qst_ctx** out, int N, const double* povm, int K, const qst_o
   c->net.eta_plus = o.eta_plus;
   c->net.step_min = o.step_min;
   c->net.step_max = o.step_max;
-  // The A_P map carries the last bit of a hidden unit to about 2e-5 of rho at N = 9 (FP32 eigenvectors of close
-  // eigenvalues): the split of its layer-1 sums stays as long as it has been, whatever suits the other maps.
+  // An A_P context keeps the split of its layer-1 sums, and with it its bits.  The FP32 sweeps round differently for
+  // any change of T's bits, and the states of two such runs, each about 2e-5 off the 64-bit one at N = 9, differ by as
+  // much (the map itself moves rho by 1e-10 for an ulp of a hidden unit).  The finer split would be 15 us where this
+  // one takes 36.
   if (o.mapping == QST_MAP_ABS_P) c->net.least_chunks = 32;
   cudaGetDevice(&c->device);
   cudaError_t e = cudaMallocHost((void**)&c->h_scal, 16 * sizeof(double));

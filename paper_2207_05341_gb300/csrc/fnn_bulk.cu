@@ -380,8 +380,9 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) k_wpass_bulk(const __gri
   }
 }
 
-// Layer-1 forward with exactly the partition of the bulk W1 pass (block g the chunks of group g, column t of a chunk to thread t), so that the hidden layer it gives is bit-identical to
-// the one the W1 pass leaves for the next iteration (checkpoint resume depends on this).
+// Layer-1 forward with exactly the partition of the bulk W1 pass (block g the chunks of group g, column t of a chunk
+// to thread t), so that the hidden layer it gives is bit-identical to the one the W1 pass leaves for the next iteration
+// (checkpoint resume depends on this).
 template <int H>
 __global__ void __launch_bounds__(kCols, 2) k_l1_forward_cols(const float* __restrict__ theta,
                                                               const float* __restrict__ f, long long n, float* pre,

@@ -1,4 +1,5 @@
-// Launch parameters chosen by autotune.py from timings on the target GPU (the defaults of qst_tuning).
+// Launch parameters chosen from timings on the target GPU (the defaults of qst_tuning): by autotune.py, and
+// kTunedBulkChunksPerCta by hand since a group of chunks is no longer a CTA of its own in a batch.
 // kFusedThreads fixes the order of the one-CTA iteration's sums, and the chunks per group of the bulk
 // weight passes fix the partition of theirs: a batch and a single context use the same values, so their
 // iterations stay bit-identical.
