@@ -253,16 +253,18 @@ size_t lazy_scratch_bytes(const Dims& D) {
 
 // An allocation the context can do without: skipped where it fails, or where it would leave less of the budget or
 // of the device than `later` bytes (the scratch that calls may still allocate on first use; 16 MiB for the rounding
-// of allocations to pages).
+// of allocations to pages, and for allocations below 8 MiB, which are not worth the 20 us of looking).
 template <class T> void dalloc_optional(qst_ctx* c, T** p, size_t count, size_t later) {
   const size_t lim = c->opt.device_memory_limit;
   if (lim && c->dev_bytes + count * sizeof(T) + later > lim) return;
-  size_t free_bytes = 0, total = 0;
-  if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
-    cudaGetLastError();
-    return;
+  if (count * sizeof(T) >= (8u << 20)) {
+    size_t free_bytes = 0, total = 0;
+    if (cudaMemGetInfo(&free_bytes, &total) != cudaSuccess) {
+      cudaGetLastError();
+      return;
+    }
+    if (free_bytes < count * sizeof(T) + later + (16u << 20)) return;
   }
-  if (free_bytes < count * sizeof(T) + later + (16u << 20)) return;
   if (dalloc(c, p, count) != cudaSuccess) {
     cudaGetLastError();
     *p = nullptr;
